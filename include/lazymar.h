@@ -43,7 +43,7 @@
  *     out-of-range indices or labels) are latched in a device error word and
  *     reported by lazymar_sync / lazymar_device_check.
  *   - No call allocates device memory except lazymar_create and
- *     lazymar_select_tokens (stream-ordered scratch for the similarities).
+ *     lazymar_head_create.
  *   - A handle is not thread-safe; distinct handles are independent.
  */
 #ifndef LAZYMAR_H
@@ -204,8 +204,7 @@ lazymar_status lazymar_cached_step(lazymar_handle *h, const lazymar_step_in *in,
  * v_cur[t] and v_cache[t] over D (fp64 accumulation of exact products,
  * S = dot / sqrt(max(|a|^2 |b|^2, 1e-16)), NaN counted as -inf); I_compute =
  * the n_compute smallest S, ties to the lower index, written ascending to
- * idx_out [rows, n_compute]. Then v_cache := v_cur. D % 8 == 0.
- * Allocates rows*T doubles of stream-ordered scratch (cudaMallocAsync). */
+ * idx_out [rows, n_compute]. Then v_cache := v_cur. D % 8 == 0. */
 lazymar_status lazymar_select_tokens(int dtype, const void *v_cur, void *v_cache, int rows, int T,
                                      int D, int n_compute, int32_t *idx_out, void *stream);
 
@@ -214,29 +213,20 @@ lazymar_status lazymar_select_tokens(int dtype, const void *v_cur, void *v_cache
  * descending, then the rule, then index ascending. priority [rows, T] uint8
  * may be NULL; keys [rows, T] uint32 are required for LAZYMAR_SELECT_RANDOM
  * and ignored otherwise. The similarities are computed and v_cache := v_cur
- * under every rule. Device pointers only; same scratch as
- * lazymar_select_tokens. */
+ * under every rule. Device pointers only. */
 lazymar_status lazymar_select_tokens_ex(int dtype, const void *v_cur, void *v_cache, int rows, int T,
                                         int D, int n_compute, int rule, const uint8_t *priority,
                                         const uint32_t *keys, int32_t *idx_out, void *stream);
 
-/* lazymar_select_tokens without any device allocation. The paper has no
- * counterpart: this entry point exists for callers that may not allocate
- * device memory once running (a serving loop that fixes its memory budget at
- * start-up, a plug-in whose host framework owns the device allocator). Same
- * arguments, semantics and results as lazymar_select_tokens; device pointers
- * only. The similarity scratch is a fixed array inside the library, holding
- * LAZYMAR_SELECT_NOALLOC_MAX_TOKENS doubles (2 MiB) on every device that loads
- * it, until the process exits; rows * T above that limit returns
- * LAZYMAR_ERR_INVALID_ARG. Every call looks up the array's device address on
- * the current device (cudaGetSymbolAddress, which allocates nothing), so the
- * address stays right after a device reset; the first call on a device also
- * loads the library's device code there, so make it before any stream
- * capture. All calls
- * share the one array and leave their similarities in it: calls whose work
- * can overlap on the GPU (different streams, or different host threads) race
- * and must be serialised by the caller. No cudaMalloc, cudaFree or other
- * allocating call is made. */
+/* lazymar_select_tokens for callers that may not allocate device memory once
+ * running (a serving loop that fixes its memory budget at start-up, a plug-in
+ * whose host framework owns the device allocator); the paper has no
+ * counterpart. Same arguments, semantics and results as lazymar_select_tokens;
+ * device pointers only. No cudaMalloc, cudaFree or other allocating call is
+ * made and no scratch is used, so calls on different streams are independent.
+ * rows * T above LAZYMAR_SELECT_NOALLOC_MAX_TOKENS returns
+ * LAZYMAR_ERR_INVALID_ARG. The first call on a device loads the library's
+ * device code there, so make it before any stream capture. */
 #define LAZYMAR_SELECT_NOALLOC_MAX_TOKENS 262144
 lazymar_status lazymar_select_tokens_noalloc(int dtype, const void *v_cur, void *v_cache, int rows,
                                              int T, int D, int n_compute, int32_t *idx_out,

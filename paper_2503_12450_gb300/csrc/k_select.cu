@@ -1,219 +1,41 @@
-// Token selection of Eq. 8.
+// Token selection of Eq. 8: one kernel, one thread-block cluster per row.
 //
-// similarity_kernel: one warp per token, spread over the whole GPU (a row has
-// only T tokens, so one CTA per row would leave most SMs idle while streaming
-// 2 x rows x T x D elements). Each lane reads 16-byte vectors of the current
-// and cached representation and accumulates the dot product and both squared
-// norms in fp64. bf16 x bf16 products are exact in fp64, and so are their sums
+// The CTAs of a cluster take equal ranges of the row's tokens, one warp per
+// token: the cosine of its current and cached representation, whose current
+// vector then replaces the cached one. Every CTA pushes its tokens'
+// similarities, as order-preserving 64-bit integer keys, into the shared
+// memory of all CTAs of the cluster; each CTA ranks its own tokens under the
+// strict total order (priority descending, rule key ascending, index
+// ascending), and with the counts of the lower CTAs writes its part of
+// I_compute in ascending order with the gather/scatter row map r*T + t. No
+// similarity reaches global memory, so a selection needs no scratch.
+//
+// Floor: streaming 3 x rows x T x D elements, 13.9 us at 64 rows x 320 tokens
+// x 768 bf16 (94 MB). Measured there, back to back: 31.9 us a call, against
+// 75.5 us for a similarity kernel (every token through the second tier below
+// and its own fp64 division), a top-N kernel with one CTA per row and scratch
+// allocated for the similarities in between. What is left above the floor is
+// instruction issue (about 13 us) and the row's serial tail: fp64 divisions
+// and square roots, ranks, three cluster barriers. Sums kept in registers
+// instead of the shared-memory ring took 36.7 us, one division per warp
+// instead of per CTA round 41.5 us.
+//
+// Similarities. bf16 x bf16 products are exact in fp64, and so are their sums
 // for any realistic dynamic range, which makes S independent of the summation
 // order: the oracle's fp64 sum gives bit-identical S, hence bit-identical
-// selections (similarity_int_kernel computes those sums exactly on the integer
-// pipe). fp32 x fp32 products are exact in fp64 too, but a sum of them is
+// selections. The kernel computes the three sums exactly on the integer pipe
+// (GB300's fp64 rate is a small fraction of its integer rate) and rounds each
+// once. fp32 x fp32 products are exact in fp64 too, but a sum of them is
 // rounded at every addition, so the kernel's lane-strided order and the
 // oracle's pairwise order can differ in the last bits of S (a relative 1e-15
 // or so). Two tokens whose similarities lie that close may then be ordered
-// differently; every other fp32 selection is identical. The current vector is
-// copied over the cached one (the cache now holds this step's values).
-//
-// topk_kernel: one CTA per row. Each token's rank under the strict total order
-// (S ascending, index ascending; NaN counted as -inf) is counted against all T
-// similarities held in shared memory as order-preserving integer keys; tokens with rank < N are I_compute. A
-// block-wide ballot/prefix scan writes them in ascending index order together
-// with the gather/scatter row map r*T + t.
+// differently; every other fp32 selection is identical.
 #include <cfloat>
+#include <climits>
 
 #include "lazymar_internal.cuh"
 
 namespace lm {
-
-template <typename T>
-__global__ void __launch_bounds__(256) similarity_kernel(const T* __restrict__ cur, T* __restrict__ cache,
-                                                         double* __restrict__ S, long long ntok, int D, int copy) {
-  constexpr int V = 16 / sizeof(T);
-  pdl_wait();
-  pdl_trigger();
-  const long long tok = (long long)blockIdx.x * 8 + (threadIdx.x >> 5);
-  const int lane = threadIdx.x & 31;
-  if (tok >= ntok) return;
-  const T* a = cur + tok * D;
-  T* c = cache + tok * D;
-  double dot = 0.0, na = 0.0, nc = 0.0;
-  for (int i = lane * V; i < D; i += 32 * V) {
-    float av[V], cv[V];
-    Vec<T, V>::load(a + i, av);
-    Vec<T, V>::load(c + i, cv);
-#pragma unroll
-    for (int k = 0; k < V; ++k) {
-      const double x = (double)av[k], y = (double)cv[k];
-      dot = fma(x, y, dot);
-      na = fma(x, x, na);
-      nc = fma(y, y, nc);
-    }
-    if (copy) *reinterpret_cast<uint4*>(c + i) = *reinterpret_cast<const uint4*>(a + i);
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    dot += __shfl_xor_sync(0xffffffffu, dot, o);
-    na += __shfl_xor_sync(0xffffffffu, na, o);
-    nc += __shfl_xor_sync(0xffffffffu, nc, o);
-  }
-  if (lane == 0) {
-    const double eps = 1e-8;
-    S[tok] = dot / sqrt(fmax(na * nc, eps * eps));
-  }
-}
-
-// bf16 similarity on the integer pipe (GB300's fp64 rate is a small fraction
-// of its integer rate). A bf16 value is M * 2^(E - 134) with an 8-bit integer
-// significand M (hidden bit included) and E = max(biased exponent, 1), so a
-// product of two is (Ma Mb) * 2^(Ea + Eb - 268) with Ma Mb < 2^16. Each sum
-// is taken relative to a base exponent kSpan = 62 - 16 - ceil(log2 D) below
-// its largest possible term exponent (from the vectors' largest exponents):
-// shifted to the base, every term is an integer below 2^(16 + kSpan) and the
-// D-term sum is exact in an int64. Its conversion to double is then the
-// correctly rounded exact sum, which equals the fp64 sum of the same products
-// whenever that sum is exact. A token with a nonzero term below the base, or
-// with an Inf/NaN element, takes the fp64 loop of similarity_kernel instead.
-// Each lane keeps its NCH 8-element chunks of both vectors in registers
-// (D <= 1280; wider vectors use similarity_kernel).
-template <int NCH>
-__global__ void __launch_bounds__(256) similarity_int_kernel(const bf16* __restrict__ cur, bf16* __restrict__ cache,
-                                                             double* __restrict__ S, long long ntok, int D, int span,
-                                                             int copy) {
-  pdl_wait();
-  pdl_trigger();
-  const long long tok = (long long)blockIdx.x * 8 + (threadIdx.x >> 5);
-  const int lane = threadIdx.x & 31;
-  if (tok >= ntok) return;
-  const bf16* a = cur + tok * D;
-  bf16* c = cache + tok * D;
-  uint4 ra[NCH], rc[NCH];
-#pragma unroll
-  for (int j = 0; j < NCH; ++j) {
-    const int i = (lane + 32 * j) * 8;
-    if (i < D) {
-      ra[j] = *reinterpret_cast<const uint4*>(a + i);
-      rc[j] = *reinterpret_cast<const uint4*>(c + i);
-    } else {
-      ra[j] = make_uint4(0, 0, 0, 0);
-      rc[j] = make_uint4(0, 0, 0, 0);
-    }
-  }
-  // largest exponent field of each vector (two bf16 per 32-bit word)
-  uint32_t xa = 0, xc = 0;
-#pragma unroll
-  for (int j = 0; j < NCH; ++j) {
-    xa = __vmaxu2(xa, __vmaxu2(ra[j].x & 0x7F807F80u, ra[j].y & 0x7F807F80u));
-    xa = __vmaxu2(xa, __vmaxu2(ra[j].z & 0x7F807F80u, ra[j].w & 0x7F807F80u));
-    xc = __vmaxu2(xc, __vmaxu2(rc[j].x & 0x7F807F80u, rc[j].y & 0x7F807F80u));
-    xc = __vmaxu2(xc, __vmaxu2(rc[j].z & 0x7F807F80u, rc[j].w & 0x7F807F80u));
-  }
-  int ema = max((int)((xa >> 7) & 0xFFu), (int)((xa >> 23) & 0xFFu));
-  int emc = max((int)((xc >> 7) & 0xFFu), (int)((xc >> 23) & 0xFFu));
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    ema = max(ema, __shfl_xor_sync(0xffffffffu, ema, o));
-    emc = max(emc, __shfl_xor_sync(0xffffffffu, emc, o));
-  }
-  bool inexact = ema == 255 || emc == 255;  // Inf or NaN present
-  ema = max(ema, 1);
-  emc = max(emc, 1);
-  const int bd = ema + emc - span, ba = 2 * ema - span, bc = 2 * emc - span;
-  long long sd = 0, sa = 0, sc = 0;
-  if (!inexact) {
-#pragma unroll
-    for (int j = 0; j < NCH; ++j) {
-      const uint32_t wa[4] = {ra[j].x, ra[j].y, ra[j].z, ra[j].w}, wc[4] = {rc[j].x, rc[j].y, rc[j].z, rc[j].w};
-#pragma unroll
-      for (int h = 0; h < 8; ++h) {
-        const uint32_t ya = (wa[h >> 1] >> (16 * (h & 1))) & 0xFFFFu, yc = (wc[h >> 1] >> (16 * (h & 1))) & 0xFFFFu;
-        const int ea = (int)((ya >> 7) & 0xFFu), ec = (int)((yc >> 7) & 0xFFu);
-        const int Ea = max(ea, 1), Ec = max(ec, 1);
-        const uint32_t Ma = (ya & 0x7Fu) | (ea ? 0x80u : 0u), Mc = (yc & 0x7Fu) | (ec ? 0x80u : 0u);
-        const uint32_t pd = Ma * Mc, pa = Ma * Ma, pc = Mc * Mc;
-        const int hd = Ea + Ec - bd, ha = 2 * Ea - ba, hc = 2 * Ec - bc;
-        inexact |= (hd < 0 && pd != 0) | (ha < 0 && pa != 0) | (hc < 0 && pc != 0);
-        const long long td = (long long)((unsigned long long)pd << max(hd, 0));
-        sd += ((ya ^ yc) & 0x8000u) ? -td : td;
-        sa += (long long)((unsigned long long)pa << max(ha, 0));
-        sc += (long long)((unsigned long long)pc << max(hc, 0));
-      }
-    }
-  }
-  double dot, na, nc;
-  if (__any_sync(0xffffffffu, inexact)) {
-    // fp64 fallback (the arithmetic of similarity_kernel)
-    dot = 0.0, na = 0.0, nc = 0.0;
-#pragma unroll 1
-    for (int i = lane * 8; i < D; i += 256) {
-      float av[8], cv[8];
-      Vec<bf16, 8>::load(a + i, av);
-      Vec<bf16, 8>::load(c + i, cv);
-#pragma unroll
-      for (int k = 0; k < 8; ++k) {
-        const double x = (double)av[k], y = (double)cv[k];
-        dot = fma(x, y, dot);
-        na = fma(x, x, na);
-        nc = fma(y, y, nc);
-      }
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      dot += __shfl_xor_sync(0xffffffffu, dot, o);
-      na += __shfl_xor_sync(0xffffffffu, na, o);
-      nc += __shfl_xor_sync(0xffffffffu, nc, o);
-    }
-  } else {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      sd += __shfl_xor_sync(0xffffffffu, sd, o);
-      sa += __shfl_xor_sync(0xffffffffu, sa, o);
-      sc += __shfl_xor_sync(0xffffffffu, sc, o);
-    }
-    dot = ldexp((double)sd, bd - 268);
-    na = ldexp((double)sa, ba - 268);
-    nc = ldexp((double)sc, bc - 268);
-  }
-  if (copy) {
-#pragma unroll
-    for (int j = 0; j < NCH; ++j) {
-      const int i = (lane + 32 * j) * 8;
-      if (i < D) *reinterpret_cast<uint4*>(c + i) = ra[j];
-    }
-  }
-  if (lane == 0) {
-    const double eps = 1e-8;
-    S[tok] = dot / sqrt(fmax(na * nc, eps * eps));
-  }
-}
-
-cudaError_t launch_similarity(const Ctx& c, int dtype, const void* cur, void* cache, double* S, int rows, int T, int D,
-                              bool copy) {
-  const long long ntok = (long long)rows * T;
-  if (ntok == 0) return cudaSuccess;
-  const unsigned grid = (unsigned)((ntok + 7) / 8);
-  if (dtype == LAZYMAR_BF16 && D % 8 == 0 && D <= 1280) {
-    int lg = 0;
-    while ((1 << lg) < D) ++lg;
-    const int span = 62 - 16 - lg;
-    const int nch = (D + 255) / 256;
-    const bf16* a = static_cast<const bf16*>(cur);
-    bf16* k = static_cast<bf16*>(cache);
-    const int cp = copy ? 1 : 0;
-    if (nch <= 1) return launch_pdl(similarity_int_kernel<1>, dim3(grid), dim3(256), 0, c.stream, a, k, S, ntok, D, span, cp);
-    if (nch <= 2) return launch_pdl(similarity_int_kernel<2>, dim3(grid), dim3(256), 0, c.stream, a, k, S, ntok, D, span, cp);
-    if (nch <= 3) return launch_pdl(similarity_int_kernel<3>, dim3(grid), dim3(256), 0, c.stream, a, k, S, ntok, D, span, cp);
-    if (nch <= 4) return launch_pdl(similarity_int_kernel<4>, dim3(grid), dim3(256), 0, c.stream, a, k, S, ntok, D, span, cp);
-    return launch_pdl(similarity_int_kernel<5>, dim3(grid), dim3(256), 0, c.stream, a, k, S, ntok, D, span, cp);
-  }
-  if (dtype == LAZYMAR_BF16)
-    return launch_pdl(similarity_kernel<bf16>, dim3(grid), dim3(256), 0, c.stream, (const bf16*)cur, (bf16*)cache, S,
-                      ntok, D, copy ? 1 : 0);
-  return launch_pdl(similarity_kernel<float>, dim3(grid), dim3(256), 0, c.stream, (const float*)cur, (float*)cache, S,
-                    ntok, D, copy ? 1 : 0);
-}
-
-constexpr int kTopkThreads = 512;
 
 // Order-preserving 64-bit key of a similarity: unsigned comparison of keys
 // matches numeric comparison of the doubles, with NaN mapped to -inf and -0
@@ -226,97 +48,415 @@ __device__ __forceinline__ unsigned long long sim_key(double s) {
   return (u >> 63) ? ~u : (u | 0x8000000000000000ull);
 }
 
+// The sums of one token: dot, |a|^2, |c|^2 as v[i] * 2^e[i] with integer v,
+// or, with e[0] == INT_MIN, as the bits of three doubles.
+struct SimSums {
+  long long v[3];
+  int e[3];
+};
+
+__device__ __forceinline__ double sim_value(const SimSums& s) {
+  double d[3];
+#pragma unroll
+  for (int i = 0; i < 3; ++i)
+    d[i] = s.e[0] == INT_MIN ? __longlong_as_double(s.v[i]) : ldexp((double)s.v[i], s.e[i]);
+  const double eps = 1e-8;
+  return d[0] / sqrt(fmax(d[1] * d[2], eps * eps));
+}
+
+// Sum of v * 2^e over the warp's lanes as an integer times a power of two
+// that rounds to the same double as the exact sum. Three 22-, 22- and 20-bit
+// pieces go through the warp's integer reduction; a total beyond 62 bits is
+// shifted right by 4 with its lost bits kept as a sticky lowest bit, far below
+// the 53 that a double holds.
+__device__ __forceinline__ void warp_sum64(long long v, int e, long long& out_v, int& out_e) {
+  const unsigned p0 = __reduce_add_sync(0xffffffffu, (unsigned)(v & 0x3FFFFF));
+  const unsigned p1 = __reduce_add_sync(0xffffffffu, (unsigned)((v >> 22) & 0x3FFFFF));
+  const int p2 = __reduce_add_sync(0xffffffffu, (int)(v >> 44));
+  const long long hi = (long long)p2 * (1ll << 22) + (long long)p1 + (long long)(p0 >> 22);  // total = hi 2^22 + lo
+  const long long lo = (long long)(p0 & 0x3FFFFFu);
+  const bool wide = hi >= (1ll << 40) || hi < -(1ll << 40);
+  out_v = wide ? (hi * (1ll << 18)) | (lo >> 4) | ((lo & 15) != 0) : hi * (1ll << 22) + lo;
+  out_e = wide ? e + 4 : e;
+}
+
+// fp64 sums of one token in lane-strided order; no copy.
+template <typename T>
+__device__ __forceinline__ void sums_fp64(const T* a, const T* c, int D, int lane, SimSums& s) {
+  constexpr int V = 16 / sizeof(T);
+  double dot = 0.0, na = 0.0, nc = 0.0;
+#pragma unroll 1
+  for (int i = lane * V; i < D; i += 32 * V) {
+    float av[V], cv[V];
+    Vec<T, V>::load(a + i, av);
+    Vec<T, V>::load(c + i, cv);
+#pragma unroll
+    for (int k = 0; k < V; ++k) {
+      const double x = (double)av[k], y = (double)cv[k];
+      dot = fma(x, y, dot);
+      na = fma(x, x, na);
+      nc = fma(y, y, nc);
+    }
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    dot += __shfl_xor_sync(0xffffffffu, dot, o);
+    na += __shfl_xor_sync(0xffffffffu, na, o);
+    nc += __shfl_xor_sync(0xffffffffu, nc, o);
+  }
+  s.v[0] = __double_as_longlong(dot);
+  s.v[1] = __double_as_longlong(na);
+  s.v[2] = __double_as_longlong(nc);
+  s.e[0] = INT_MIN;
+  s.e[1] = s.e[2] = 0;
+}
+
+// Exact sums of a bf16 token of which each lane has NCH 16-byte chunks of
+// both vectors (zero beyond D) at sa[32 j] and sc[32 j], in two tiers of
+// integer arithmetic:
+//
+// 1. Fixed point. Scaled by a power of two (k below) so that its largest
+//    element stays below 2^bits, every element of a vector whose nonzero
+//    exponents span at most bits - 8 octaves is an integer of the int32 range,
+//    and the three sums are one 32 x 32 -> 64 multiply-add per product. A
+//    lane's 8 NCH products stay within an int64: bits = 30, 29, 29, 29, 28 for
+//    NCH = 1..5. About 1 in 400 tokens of normally distributed elements
+//    exceeds the 21 octaves of widths 264 to 1024. About 14 issue slots per
+//    element pair against 55 for the second tier.
+// 2. Shifted products. A bf16 value is M * 2^(E - 134) with an 8-bit integer
+//    significand M (hidden bit included) and E = max(biased exponent, 1), so a
+//    product of two is (Ma Mb) * 2^(Ea + Eb - 268) with Ma Mb < 2^16. Each sum
+//    is taken relative to a base exponent span = 62 - 16 - ceil(log2 D) below
+//    its largest possible term exponent (from the vectors' largest exponents):
+//    shifted to the base, every term is an integer below 2^(16 + span) and the
+//    D-term sum is exact in an int64.
+//
+// A token with a nonzero term below that base, or with an Inf/NaN element,
+// takes the fp64 sums instead. An integer sum converts to double with one
+// rounding of the exact value, whatever the tier: it equals the fp64 sum of
+// the same products whenever that sum is exact.
+template <int NCH>
+__device__ __forceinline__ void sums_bf16(const uint4* sa, const uint4* sc, const bf16* a, const bf16* c, int D,
+                                          int span, int lane, SimSums& s) {
+  constexpr int bits = NCH == 1 ? 30 : NCH <= 4 ? 29 : 28;
+  static_assert(NCH >= 1 && NCH <= 5, "8 NCH products below 2^(2 bits) in an int64");
+  // per vector: the largest magnitude (two bf16 per word, unsigned), and the
+  // smallest nonzero one. (w | sign) - 1 per half is 0x7FFF for a zero and
+  // 0x8000 + magnitude - 1 otherwise, so a signed minimum skips the zeros.
+  uint32_t xa = 0, xc = 0, na = 0x7FFF7FFFu, nc = 0x7FFF7FFFu;
+#pragma unroll
+  for (int j = 0; j < NCH; ++j) {
+    const uint4 qa = sa[32 * j], qc = sc[32 * j];
+    const uint32_t wa[4] = {qa.x, qa.y, qa.z, qa.w}, wc[4] = {qc.x, qc.y, qc.z, qc.w};
+#pragma unroll
+    for (int h = 0; h < 4; ++h) {
+      xa = __vmaxu2(xa, wa[h] & 0x7FFF7FFFu);
+      xc = __vmaxu2(xc, wc[h] & 0x7FFF7FFFu);
+      na = __vmins2(na, (wa[h] | 0x80008000u) - 0x00010001u);
+      nc = __vmins2(nc, (wc[h] | 0x80008000u) - 0x00010001u);
+    }
+  }
+  int ema = (int)(__reduce_max_sync(0xffffffffu, max(xa & 0xFFFFu, xa >> 16)) >> 7);
+  int emc = (int)(__reduce_max_sync(0xffffffffu, max(xc & 0xFFFFu, xc >> 16)) >> 7);
+  const int ma = __reduce_min_sync(0xffffffffu, min((int)(short)(na & 0xFFFFu), (int)na >> 16));
+  const int mc = __reduce_min_sync(0xffffffffu, min((int)(short)(nc & 0xFFFFu), (int)nc >> 16));
+  // smallest nonzero exponent field (0: a subnormal), 255 for a zero vector
+  const int la = ma == 0x7FFF ? 255 : (ma + 32769) >> 7, lc = mc == 0x7FFF ? 255 : (mc + 32769) >> 7;
+  long long v0 = 0, v1 = 0, v2 = 0;
+  // exponent fields of 25 + (30 - bits)..254: the scale 2^k below is a normal float
+  if (ema >= 32 && ema <= 254 && emc >= 32 && emc <= 254 && la >= ema + 8 - bits && lc >= emc + 8 - bits) {
+    const int ka = bits + 126 - ema, kc = bits + 126 - emc;  // |element| < 2^(ema - 126)
+    const float fa = __int_as_float((ka + 127) << 23), fc = __int_as_float((kc + 127) << 23);
+#pragma unroll
+    for (int j = 0; j < NCH; ++j) {
+      const uint4 qa = sa[32 * j], qc = sc[32 * j];
+      const uint32_t wa[4] = {qa.x, qa.y, qa.z, qa.w}, wc[4] = {qc.x, qc.y, qc.z, qc.w};
+#pragma unroll
+      for (int h = 0; h < 8; ++h) {
+        const float x = __uint_as_float(h & 1 ? wa[h >> 1] & 0xFFFF0000u : wa[h >> 1] << 16);
+        const float y = __uint_as_float(h & 1 ? wc[h >> 1] & 0xFFFF0000u : wc[h >> 1] << 16);
+        const int ia = __float2int_rn(x * fa), ic = __float2int_rn(y * fc);  // exact
+        v0 += (long long)ia * ic;
+        v1 += (long long)ia * ia;
+        v2 += (long long)ic * ic;
+      }
+    }
+    warp_sum64(v0, -(ka + kc), s.v[0], s.e[0]);
+    warp_sum64(v1, -2 * ka, s.v[1], s.e[1]);
+    warp_sum64(v2, -2 * kc, s.v[2], s.e[2]);
+    return;
+  }
+  bool inexact = ema == 255 || emc == 255;  // Inf or NaN present
+  ema = max(ema, 1);
+  emc = max(emc, 1);
+  const int bd = ema + emc - span, ba = 2 * ema - span, bc = 2 * emc - span;
+  if (!inexact) {
+#pragma unroll 1
+    for (int j = 0; j < NCH; ++j) {
+      const uint4 qa = sa[32 * j], qc = sc[32 * j];
+      const uint32_t wa[4] = {qa.x, qa.y, qa.z, qa.w}, wc[4] = {qc.x, qc.y, qc.z, qc.w};
+#pragma unroll
+      for (int h = 0; h < 8; ++h) {
+        const uint32_t ya = (wa[h >> 1] >> (16 * (h & 1))) & 0xFFFFu, yc = (wc[h >> 1] >> (16 * (h & 1))) & 0xFFFFu;
+        const int ea = (int)((ya >> 7) & 0xFFu), ec = (int)((yc >> 7) & 0xFFu);
+        const int Ea = max(ea, 1), Ec = max(ec, 1);
+        const uint32_t Ma = (ya & 0x7Fu) | (ea ? 0x80u : 0u), Mc = (yc & 0x7Fu) | (ec ? 0x80u : 0u);
+        const uint32_t pd = Ma * Mc, pa = Ma * Ma, pc = Mc * Mc;
+        const int hd = Ea + Ec - bd, ha = 2 * Ea - ba, hc = 2 * Ec - bc;
+        inexact |= (hd < 0 && pd != 0) | (ha < 0 && pa != 0) | (hc < 0 && pc != 0);
+        const long long td = (long long)((unsigned long long)pd << max(hd, 0));
+        v0 += ((ya ^ yc) & 0x8000u) ? -td : td;
+        v1 += (long long)((unsigned long long)pa << max(ha, 0));
+        v2 += (long long)((unsigned long long)pc << max(hc, 0));
+      }
+    }
+  }
+  if (__any_sync(0xffffffffu, inexact)) {
+    sums_fp64(a, c, D, lane, s);
+    return;
+  }
+  warp_sum64(v0, bd - 268, s.v[0], s.e[0]);
+  warp_sum64(v1, ba - 268, s.v[1], s.e[1]);
+  warp_sum64(v2, bc - 268, s.v[2], s.e[2]);
+}
+
+constexpr int kSelThreads = 256;
+
+__device__ __forceinline__ uint32_t cluster_ctarank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ uint32_t cluster_nctarank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
+  return r;
+}
+// Barrier over the cluster's threads: shared-memory writes of every CTA
+// before it, remote ones included, are visible to every CTA after it.
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// Shared-memory address `saddr` of this CTA as seen in CTA `rank`.
+__device__ __forceinline__ uint32_t cluster_map(uint32_t saddr, uint32_t rank) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(saddr), "r"(rank));
+  return r;
+}
+
+// 16 bytes from global to shared memory, and the groups of such copies of
+// this thread (bytes == 0 writes zeros and reads nothing).
+__device__ __forceinline__ void cp_async16(void* dst, const void* src, int bytes) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(dst)), "l"(src), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int LEFT>
+__device__ __forceinline__ void cp_async_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(LEFT) : "memory");
+}
+
+// One cluster per row r (blockIdx.x / cluster size). T: element type; NCH > 0:
+// bf16 vectors of at most 256 NCH elements; NCH == 0: fp64 sums streamed from
+// memory (fp32, and wider bf16 vectors). N == 0 only moves the current vectors
+// into the cache.
+//
+// With NCH > 0 every lane copies its chunks of the warp's next token to shared
+// memory while the warp works on the current one. A lane reads back only what
+// it copied itself, so the two-deep ring needs no barrier.
+//
 // Selection order (Table 3 strategies): priority descending when given, then
 // the rule's key ascending, then token index. Keys: LEAST_SIMILAR (strategy V)
 // the order-preserving key of S; MOST_SIMILAR (strategy IV) its complement,
 // i.e. S descending (NaN, as -inf, last); RANDOM (strategy III) the caller's
 // 32-bit random keys.
-__global__ void __launch_bounds__(kTopkThreads) topk_kernel(const double* __restrict__ S, int T, int N,
-                                                            int* __restrict__ idx, int* __restrict__ row_map,
-                                                            int rule, const uint8_t* __restrict__ prio,
-                                                            const uint32_t* __restrict__ rkeys) {
-  extern __shared__ unsigned long long sK[];  // T keys, then T priorities, then T flags
-  __shared__ int s_wcount[kTopkThreads / 32];
-  __shared__ int s_woff[kTopkThreads / 32];
-  __shared__ int s_total;
-  unsigned char* sP = reinterpret_cast<unsigned char*>(sK + T);
-  unsigned char* sel = sP + T;
-  const int r = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+template <int NCH>
+constexpr int kSelRing = NCH * 2 * 2 * 16 * kSelThreads;  // bytes: [stage][cur, cache][chunk][thread]
+
+template <typename T, int NCH>
+__global__ void __launch_bounds__(kSelThreads, NCH <= 3 ? 4 : 2)
+    select_kernel(const T* __restrict__ cur, T* __restrict__ cache, int n_tok, int D, int span, int N,
+                  int* __restrict__ idx, int* __restrict__ row_map, int rule, const uint8_t* __restrict__ prio,
+                  const uint32_t* __restrict__ rkeys) {
+  constexpr int V = 16 / sizeof(T);
+  constexpr int kWarps = kSelThreads / 32;
+  extern __shared__ __align__(16) uint8_t sel_smem[];  // the ring, then (N > 0) the row's keys, this CTA's sums and flags
+  __shared__ int s_count[16];                          // selected tokens of each CTA of the cluster
+  __shared__ int s_wcount[kWarps], s_ctotal;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const uint32_t me = cluster_ctarank(), ncta = cluster_nctarank();
+  const int r = (int)(blockIdx.x / ncta);
+  const int per = (n_tok + (int)ncta - 1) / (int)ncta;  // tokens per CTA
+  const int t0 = min((int)me * per, n_tok), t1 = min(t0 + per, n_tok);
+  unsigned long long* sK = reinterpret_cast<unsigned long long*>(sel_smem + kSelRing<NCH>);
+  SimSums* sums = reinterpret_cast<SimSums*>(sK + n_tok);
+  unsigned char* sel = reinterpret_cast<unsigned char*>(sums + min(per, kSelThreads));
+  const bool need_s = N > 0 && rule != LAZYMAR_SELECT_RANDOM;
+  if (N > 0) cluster_sync();  // every CTA of the cluster runs before its shared memory is written to
   pdl_wait();
   pdl_trigger();
-  for (int t = tid; t < T; t += kTopkThreads) {
-    const size_t i = (size_t)r * T + t;
-    unsigned long long k;
-    if (rule == LAZYMAR_SELECT_RANDOM) {
-      k = rkeys[i];
-    } else {
-      k = sim_key(S[i]);
-      if (rule == LAZYMAR_SELECT_MOST_SIMILAR) k = ~k;
+  const size_t row0 = (size_t)r * n_tok;
+  uint4* ring = reinterpret_cast<uint4*>(sel_smem) + warp * (NCH * 4 * 32) + lane;
+  auto fetch = [&](int t, int stage) {
+    const T* a = cur + (row0 + t) * D;
+    const T* c = cache + (row0 + t) * D;
+#pragma unroll
+    for (int j = 0; j < NCH; ++j) {
+      const int i = (lane + 32 * j) * V;
+      const int in = i < D ? 16 : 0, at = in ? i : 0;
+      cp_async16(ring + (stage * 2 * NCH + j) * 32, a + at, in);
+      if (need_s) cp_async16(ring + (stage * 2 * NCH + NCH + j) * 32, c + at, in);
     }
-    sK[t] = k;
-    sP[t] = prio ? prio[i] : 0;
+    cp_async_commit();
+  };
+  if (NCH > 0 && t0 + warp < t1) fetch(t0 + warp, 0);
+  int stage = 0;
+  // rounds of one token per thread: the warps take the sums, then each thread
+  // one token's fp64 division and square root, which cost a whole warp as much
+  // as one token (GB300 has about two fp64 lanes per SM)
+  for (int b = t0; b < t1; b += kSelThreads) {
+    const int b1 = min(b + kSelThreads, t1);
+    for (int t = b + warp; t < b1; t += kWarps, stage ^= 1) {
+      const T* a = cur + (row0 + t) * D;
+      T* c = cache + (row0 + t) * D;
+      SimSums s;
+      if constexpr (NCH > 0) {
+        if (t + kWarps < t1) {
+          fetch(t + kWarps, stage ^ 1);
+          cp_async_wait<1>();
+        } else {
+          cp_async_wait<0>();
+        }
+        const uint4* sa = ring + stage * 2 * NCH * 32;
+        if (need_s) sums_bf16<NCH>(sa, sa + NCH * 32, a, c, D, span, lane, s);
+#pragma unroll
+        for (int j = 0; j < NCH; ++j) {
+          const int i = (lane + 32 * j) * V;
+          if (i < D) *reinterpret_cast<uint4*>(c + i) = sa[32 * j];
+        }
+      } else {
+        if (need_s) sums_fp64(a, c, D, lane, s);
+        for (int i = lane * V; i < D; i += 32 * V)
+          *reinterpret_cast<uint4*>(c + i) = *reinterpret_cast<const uint4*>(a + i);
+      }
+      if (need_s && lane == 0) sums[t - b] = s;
+    }
+    if (need_s) {
+      __syncthreads();
+      if (b + tid < b1) {
+        unsigned long long k = sim_key(sim_value(sums[tid]));
+        if (rule == LAZYMAR_SELECT_MOST_SIMILAR) k = ~k;
+        const uint32_t at = smem_u32(sK + b + tid);
+        for (uint32_t p = 0; p < ncta; ++p)
+          asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(cluster_map(at, p)), "l"(k) : "memory");
+      }
+      if (b1 < t1) __syncthreads();  // the sums are free for the next round
+    }
   }
-  __syncthreads();
-  // rank of token t under (priority descending, key ascending, index
-  // ascending); I_compute = rank < N
-  for (int t = tid; t < T; t += kTopkThreads) {
+  if (N == 0) return;  // uniform over the cluster: nothing to rank
+  if (!need_s)
+    for (int t = tid; t < n_tok; t += kSelThreads) sK[t] = rkeys[row0 + t];
+  cluster_sync();
+  // rank of token t: one warp per token, its lanes sharing the row's keys;
+  // I_compute = rank < N
+  for (int t = t0 + warp; t < t1; t += kWarps) {
     const unsigned long long kt = sK[t];
-    const unsigned pt = sP[t];
     int rank = 0;
     if (prio) {
-      for (int u = 0; u < T; ++u) {
+      const unsigned pt = prio[row0 + t];
+      for (int u = lane; u < n_tok; u += 32) {
         const unsigned long long ku = sK[u];
-        const unsigned pu = sP[u];
+        const unsigned pu = prio[row0 + u];
         rank += (pu > pt) || (pu == pt && ((ku < kt) || (ku == kt && u < t)));
       }
     } else {
-      for (int u = 0; u < T; ++u) {
+      for (int u = lane; u < n_tok; u += 32) {
         const unsigned long long ku = sK[u];
         rank += (ku < kt) || (ku == kt && u < t);
       }
     }
-    sel[t] = rank < N;
+    rank = __reduce_add_sync(0xffffffffu, rank);
+    if (lane == 0) sel[t - t0] = rank < N;
   }
   __syncthreads();
+  // this CTA's count to every CTA of the cluster
+  if (warp == 0) {
+    int n = 0;
+    for (int t = lane; t < t1 - t0; t += 32) n += sel[t];
+    n = __reduce_add_sync(0xffffffffu, n);
+    if (lane < (int)ncta)
+      asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(cluster_map(smem_u32(s_count + me), (uint32_t)lane)), "r"(n)
+                   : "memory");
+  }
+  cluster_sync();  // also: no CTA exits while another may still write to it
   int base = 0;
-  for (int c0 = 0; c0 < T; c0 += kTopkThreads) {
+  for (uint32_t p = 0; p < me; ++p) base += s_count[p];
+  for (int c0 = t0; c0 < t1; c0 += kSelThreads) {
     const int t = c0 + tid;
-    const bool f = t < T && sel[t];
+    const bool f = t < t1 && sel[t - t0];
     const unsigned bal = __ballot_sync(0xffffffffu, f);
     if (lane == 0) s_wcount[warp] = __popc(bal);
     __syncthreads();
-    if (warp == 0) {
-      const int v = lane < kTopkThreads / 32 ? s_wcount[lane] : 0;
-      int incl = v;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int n = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += n;
-      }
-      if (lane < kTopkThreads / 32) s_woff[lane] = incl - v;
-      if (lane == 31) s_total = incl;
-    }
-    __syncthreads();
+    int off = 0;
+    for (int w = 0; w < warp; ++w) off += s_wcount[w];
+    if (tid == kSelThreads - 1) s_ctotal = off + __popc(bal);
     if (f) {
-      const int pos = base + s_woff[warp] + __popc(bal & ((1u << lane) - 1u));
+      const int pos = base + off + __popc(bal & ((1u << lane) - 1u));
       idx[(size_t)r * N + pos] = t;
-      if (row_map) row_map[(size_t)r * N + pos] = r * T + t;
+      if (row_map) row_map[(size_t)r * N + pos] = (int)(row0 + t);
     }
-    base += s_total;
     __syncthreads();
+    base += s_ctotal;
   }
 }
 
-cudaError_t launch_topk(const Ctx& c, const double* S, int rows, int T, int N, int* idx, int* row_map, int rule,
-                        const uint8_t* prio, const uint32_t* keys) {
-  if (rows == 0 || N == 0) return cudaSuccess;
-  const size_t smem = (size_t)T * sizeof(unsigned long long) + 2 * (size_t)T;
-  if (smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(topk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+// CTAs per row. 8 (the portable limit) keeps a row's tokens on 64 warps; with
+// few rows, clusters of 16 spread them over twice as many SMs.
+template <typename T, int NCH>
+static cudaError_t launch_select_t(const Ctx& c, const void* cur, void* cache, int rows, int n_tok, int D, int span,
+                                   int N, int* idx, int* row_map, int rule, const uint8_t* prio,
+                                   const uint32_t* keys) {
+  auto kernel = select_kernel<T, NCH>;
+  const int ncta = rows * 16 <= c.num_sms ? 16 : 8;
+  const size_t per = (size_t)((n_tok + ncta - 1) / ncta);
+  const size_t smem =
+      kSelRing<NCH> + (N > 0 ? (size_t)n_tok * sizeof(unsigned long long) +
+                                   (per < kSelThreads ? per : (size_t)kSelThreads) * sizeof(SimSums) + per
+                             : 0);
+  if (smem > 40 * 1024) {
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
   }
-  return launch_pdl(topk_kernel, dim3(rows), dim3(kTopkThreads), smem, c.stream, S, T, N, idx, row_map, rule, prio,
-                    keys);
+  static int attr_set[64] = {};
+  int dev = 0;
+  cudaGetDevice(&dev);
+  if (ncta > 8 && dev >= 0 && dev < 64 && !attr_set[dev]) {
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e != cudaSuccess) return e;
+    attr_set[dev] = 1;
+  }
+  return launch_pdl_cluster(kernel, dim3((unsigned)(rows * ncta)), dim3(kSelThreads), smem, ncta, c.stream,
+                            static_cast<const T*>(cur), static_cast<T*>(cache), n_tok, D, span, N, idx, row_map,
+                            rule, prio, keys);
+}
+
+cudaError_t launch_select(const Ctx& c, int dtype, const void* cur, void* cache, int rows, int n_tok, int D, int N,
+                          int* idx, int* row_map, int rule, const uint8_t* prio, const uint32_t* keys) {
+  if (rows == 0) return cudaSuccess;
+  int lg = 0;
+  while ((1 << lg) < D) ++lg;
+  const int span = 62 - 16 - lg;
+#define LM_SELECT(T, NCH) \
+  return launch_select_t<T, NCH>(c, cur, cache, rows, n_tok, D, span, N, idx, row_map, rule, prio, keys)
+  if (dtype != LAZYMAR_BF16) LM_SELECT(float, 0);
+  if (D % 8 != 0 || D > 1280) LM_SELECT(bf16, 0);
+  switch ((D + 255) / 256) {
+    case 1: LM_SELECT(bf16, 1);
+    case 2: LM_SELECT(bf16, 2);
+    case 3: LM_SELECT(bf16, 3);
+    case 4: LM_SELECT(bf16, 4);
+    default: LM_SELECT(bf16, 5);
+  }
+#undef LM_SELECT
 }
 
 // Caller-chosen I_compute: copied after checking range and strict increase per
@@ -352,27 +492,10 @@ cudaError_t launch_idx_check(const Ctx& c, const int* in, int rows, int T, int N
 // Some callers may not allocate device memory once they are running: a
 // serving loop that reserves its whole memory budget at start-up and must not
 // grow it, or a plug-in whose host framework owns the device allocator and
-// forbids direct cudaMalloc. lazymar_select_tokens_noalloc serves them: its
-// similarity scratch is this fixed, module-level array, which every GPU that
-// loads the library holds until the process exits (8 bytes per token,
-// 2 MiB in total).
-static __device__ __align__(256) double g_select_scratch[LAZYMAR_SELECT_NOALLOC_MAX_TOKENS];
-
+// forbids direct cudaMalloc. lazymar_select_tokens_noalloc serves them. The
+// selection keeps its similarities in shared memory, so neither entry point
+// allocates; this one keeps its documented limit on rows * T.
 constexpr int kMaxDevices = 64;
-
-// On the host, the name g_select_scratch denotes a host-side stand-in, not
-// device memory: handing it to a kernel would fault or, where the GPU can
-// reach host memory, silently use the wrong memory. The device address is
-// looked up on every call, with the caller's device current: the lookup
-// allocates nothing and costs little, and a cached address would go stale
-// when a device reset reloads the module at another address.
-static cudaError_t select_scratch(double** out) {
-  void* p = nullptr;
-  const cudaError_t e = cudaGetSymbolAddress(&p, g_select_scratch);
-  if (e != cudaSuccess) return e;
-  *out = static_cast<double*>(p);
-  return cudaSuccess;
-}
 
 static bool noalloc_device_ptr(const void* p) {
   cudaPointerAttributes a;
@@ -394,8 +517,7 @@ extern "C" lazymar_status lazymar_select_tokens_noalloc(int dtype, const void* v
                         "rows >= 0, 1 <= T <= 16384, D % 8 == 0, 0 <= n_compute <= T required");
   if ((long long)rows * T > LAZYMAR_SELECT_NOALLOC_MAX_TOKENS)
     return report_error(LAZYMAR_ERR_INVALID_ARG,
-                        "rows * T exceeds LAZYMAR_SELECT_NOALLOC_MAX_TOKENS (262144), the size of the fixed "
-                        "scratch; use lazymar_select_tokens");
+                        "rows * T exceeds LAZYMAR_SELECT_NOALLOC_MAX_TOKENS (262144); use lazymar_select_tokens");
   if (rows == 0) return LAZYMAR_OK;
   if (!noalloc_device_ptr(v_cur) || !noalloc_device_ptr(v_cache) || (n_compute > 0 && !noalloc_device_ptr(idx_out)))
     return report_error(LAZYMAR_ERR_INVALID_ARG, "v_cur, v_cache and idx_out must be device pointers");
@@ -406,14 +528,8 @@ extern "C" lazymar_status lazymar_select_tokens_noalloc(int dtype, const void* v
     return report_error(LAZYMAR_ERR_CUDA, "cudaGetDevice failed or device index out of range");
   if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
     return report_error(LAZYMAR_ERR_CUDA, "cudaDeviceGetAttribute failed");
-  double* S = nullptr;
-  if (select_scratch(&S) != cudaSuccess)
-    return report_error(LAZYMAR_ERR_CUDA, "cudaGetSymbolAddress of the selection scratch failed");
-  // Every S entry the top-N reads is written by the similarity pass of the
-  // same call first, so the scratch needs no clearing between calls.
   const Ctx c{static_cast<cudaStream_t>(stream), nullptr, sms};
-  cudaError_t e = launch_similarity(c, dtype, v_cur, v_cache, S, rows, T, D, true);
-  if (e == cudaSuccess) e = launch_topk(c, S, rows, T, n_compute, idx_out, nullptr);
+  const cudaError_t e = launch_select(c, dtype, v_cur, v_cache, rows, T, D, n_compute, idx_out, nullptr);
   if (e != cudaSuccess) return report_error(LAZYMAR_ERR_CUDA, cudaGetErrorString(e));
   return LAZYMAR_OK;
 }

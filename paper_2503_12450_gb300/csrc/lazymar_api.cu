@@ -113,7 +113,6 @@ struct lazymar_handle {
   // scratch
   float *H = nullptr, *Hc = nullptr;
   void *A = nullptr, *Q = nullptr, *Ks = nullptr, *Vs = nullptr, *O = nullptr, *U = nullptr, *Fs = nullptr;
-  double* S = nullptr;
   int *idx = nullptr, *row_map = nullptr;
   // staging of host inputs/outputs
   float* st_lat = nullptr;
@@ -329,7 +328,7 @@ extern "C" lazymar_status lazymar_create(const lazymar_config* cfg, const lazyma
                o_Q = b.take(rowsT * D * es), o_Ks = b.take(rowsT * D * es), o_Vs = b.take(rowsT * D * es),
                o_O = b.take(rowsT * D * es), o_U = b.take(rowsT * H4 * es),
                o_Fs = b.take(cfg->criterion == LAZYMAR_CRITERION_FEATURE ? rowsT * D * es : 0),
-               o_S = b.take(rowsT * 8), o_idx = b.take(rowsT * 4), o_map = b.take(rowsT * 4);
+               o_idx = b.take(rowsT * 4), o_map = b.take(rowsT * 4);
   // staging
   const size_t o_lat = b.take(Bm * cfg->n_img * cfg->token_dim * 4), o_mask = b.take(Bm * cfg->n_img),
                o_lab = b.take(Bm * 4), o_iin = b.take(rowsT * 4), o_iout = b.take(rowsT * 4),
@@ -376,7 +375,6 @@ extern "C" lazymar_status lazymar_create(const lazymar_config* cfg, const lazyma
   h->H = reinterpret_cast<float*>(a + o_H); h->Hc = reinterpret_cast<float*>(a + o_Hc);
   h->A = a + o_A; h->Q = a + o_Q; h->Ks = a + o_Ks; h->Vs = a + o_Vs; h->O = a + o_O; h->U = a + o_U;
   h->Fs = a + o_Fs;
-  h->S = reinterpret_cast<double*>(a + o_S);
   h->idx = reinterpret_cast<int*>(a + o_idx); h->row_map = reinterpret_cast<int*>(a + o_map);
   h->st_lat = reinterpret_cast<float*>(a + o_lat); h->st_mask = a + o_mask;
   h->st_labels = reinterpret_cast<int*>(a + o_lab);
@@ -693,18 +691,17 @@ lazymar_status cached_body(lazymar_handle* h, const Ctx& c, int rows, int N, boo
                   [&] { return launch_cast(c, h->cfg.dtype, h->H, h->Fs, n); }));
     cur = h->Fs;
   }
-  LM_TRY(launch(h, LAZYMAR_K_SELECT, 0, 3.0 * rows * T * D * h->es + 8.0 * rows * T, c.stream, "similarity",
-                [&] { return launch_similarity(c, h->cfg.dtype, cur, h->ref, h->S, rows, T, D, true); }));
-  if (has_idx) {
+  // (a caller's own I_compute only needs the reference moved on)
+  const int n_rank = has_idx ? 0 : N;
+  LM_TRY(launch(h, LAZYMAR_K_SELECT, 0, (n_rank ? 3.0 : 2.0) * rows * T * D * h->es + 8.0 * rows * n_rank, c.stream,
+                "select", [&] {
+                  return launch_select(c, h->cfg.dtype, cur, h->ref, rows, T, D, n_rank, h->idx, h->row_map,
+                                       h->cfg.select_rule, (sel & 1) ? h->st_prio : nullptr,
+                                       (sel & 2) ? h->st_keys : nullptr);
+                }));
+  if (has_idx)
     LM_TRY(launch(h, LAZYMAR_K_SELECT, 0, 12.0 * rows * N, c.stream, "index check",
                   [&] { return launch_idx_check(c, h->st_idx_in, rows, T, N, h->idx, h->row_map); }));
-  } else if (N > 0) {
-    LM_TRY(launch(h, LAZYMAR_K_SELECT, 0, 8.0 * rows * T + 8.0 * rows * N, c.stream, "topk",
-                  [&] {
-                    return launch_topk(c, h->S, rows, T, N, h->idx, h->row_map, h->cfg.select_rule,
-                                       (sel & 1) ? h->st_prio : nullptr, (sel & 2) ? h->st_keys : nullptr);
-                  }));
-  }
   if (N > 0) {
     if (value) {
       // rest of block s-1 on the selected tokens: their queries and residual
@@ -897,15 +894,9 @@ extern "C" lazymar_status lazymar_select_tokens_ex(int dtype, const void* v_cur,
   if (!aligned16(v_cur) || !aligned16(v_cache)) return fail(LAZYMAR_ERR_INVALID_ARG, "16-byte alignment required");
   Ctx c;
   LM_TRY(component_ctx(stream, &c));
-  double* S = nullptr;
-  LM_CUDA(cudaMallocAsync(reinterpret_cast<void**>(&S), (size_t)rows * T * sizeof(double), c.stream));
-  cudaError_t e = launch_similarity(c, dtype, v_cur, v_cache, S, rows, T, D, true);
-  if (e == cudaSuccess)
-    e = launch_topk(c, S, rows, T, n_compute, idx_out, nullptr, rule, priority,
-                    rule == LAZYMAR_SELECT_RANDOM ? keys : nullptr);
-  cudaError_t e2 = cudaFreeAsync(S, c.stream);
-  if (e != cudaSuccess) return cuda_fail(e, "select kernels");
-  if (e2 != cudaSuccess) return cuda_fail(e2, "cudaFreeAsync");
+  const cudaError_t e = launch_select(c, dtype, v_cur, v_cache, rows, T, D, n_compute, idx_out, nullptr, rule, priority,
+                                      rule == LAZYMAR_SELECT_RANDOM ? keys : nullptr);
+  if (e != cudaSuccess) return cuda_fail(e, "select kernel");
   return LAZYMAR_OK;
 }
 

@@ -232,6 +232,27 @@ inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, s
   return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
 }
 
+// launch_pdl with the grid divided into clusters of `cluster` consecutive CTAs.
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_pdl_cluster(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, int cluster,
+                                      cudaStream_t st, Args&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = (unsigned)cluster;
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
+  return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
+}
+
 // ---------------------------------------------------------------------------
 // Shared-memory barriers and TMA (PTX ISA: mbarrier, cp.async.bulk.tensor)
 // ---------------------------------------------------------------------------
@@ -519,13 +540,15 @@ cudaError_t launch_gather_rows(const Ctx& c, int dtype, const void* q, const flo
 // (max |w| / 448): q [rows, cols] bytes, scale [rows] fp32.
 cudaError_t launch_quantize_e4m3(const Ctx& c, const void* w, int rows, int cols, void* q, float* scale);
 
-cudaError_t launch_similarity(const Ctx& c, int dtype, const void* cur, void* cache, double* S, int rows, int T,
-                              int D, bool copy);
+// Token selection of Eq. 8 (lazymar_select_tokens_ex): similarities of cur with
+// cache, cache := cur, the N tokens of each row that the rule takes, ascending,
+// to idx and (if given) r * T + t to row_map. N == 0 only copies.
+cudaError_t launch_select(const Ctx& c, int dtype, const void* cur, void* cache, int rows, int T, int D, int N,
+                          int* idx, int* row_map, int rule = 0, const uint8_t* prio = nullptr,
+                          const uint32_t* keys = nullptr);
 // Diagnostic: one CTA waits on an mbarrier that nothing completes, for at most
 // limit_ns (the bounded-wait failure path of every pipelined kernel).
 cudaError_t launch_stuck_wait(const Ctx& c, uint64_t limit_ns);
-cudaError_t launch_topk(const Ctx& c, const double* S, int rows, int T, int N, int* idx, int* row_map,
-                        int rule = 0, const uint8_t* prio = nullptr, const uint32_t* keys = nullptr);
 cudaError_t launch_idx_check(const Ctx& c, const int* idx_in, int rows, int T, int N, int* idx, int* row_map);
 cudaError_t launch_cfg(const Ctx& c, int dtype, int mode, const void* zc, const void* zu, void* delta,
                        float gamma, size_t n, void* zu_out, void* g_out);

@@ -134,6 +134,35 @@ def test_select_tokens_exponent_range_and_specials(D):
     assert torch.equal(g_ref.view(torch.int16), g_cur.view(torch.int16))
 
 
+@pytest.mark.parametrize("D,octaves", [(8, 22), (8, 23), (256, 19), (256, 20), (768, 18), (768, 19), (1280, 18),
+                                       (1280, 19), (1288, 18)])
+@pytest.mark.parametrize("rows,T", [(1, 9), (1, 333), (20, 333)])
+def test_select_tokens_fixed_point_span(D, octaves, rows, T):
+    """Exponent spans at the limit of the fixed-point sums and one octave
+    beyond (D = 8, 256, 768, 1280: spans of 22, 19, 18 and 18 octaves; D = 1288
+    takes the fp64 sums), with zeros, whole-vector powers of two down to the
+    limit of the scaling, and a top value on either side of the span."""
+    torch = torch_cuda()
+    rng = np.random.default_rng(1000 * octaves + D + T + rows)
+    ref = rng.uniform(1, 2, (rows, T, D)) * rng.choice([-1.0, 1.0], (rows, T, D))
+    cur = ref * (1 + 0.3 * rng.standard_normal((rows, T, 1)) * rng.standard_normal((rows, T, D)))
+    u = rng.integers(-octaves, 1, (rows, T, D))
+    u[..., 0], u[..., 1] = 0, -octaves
+    whole = rng.choice([-100, -20, 0, 30], (rows, T, 1))  # -100: below the fixed-point tier's exponents
+    cur, ref = cur * np.exp2(u + whole), ref * np.exp2(u)
+    cur[rng.random((rows, T, D)) < 0.05] = 0
+    cur, ref = synth.round_bf16(cur.astype(np.float32)), synth.round_bf16(ref.astype(np.float32))
+    g_cur, g_ref = dev(cur, "bf16"), dev(ref, "bf16")
+    N = T // 3
+    idx = torch.full((rows, N), -1, dtype=torch.int32, device="cuda")
+    lm.lazymar_select_tokens(DT["bf16"], g_cur, g_ref, rows, T, D, N, idx)
+    sync()
+    got = idx.cpu().numpy()
+    for r in range(rows):
+        assert got[r].tolist() == O.select_compute(O.cosine_similarity(cur[r], ref[r]), N).tolist(), "row %d" % r
+    assert torch.equal(g_ref, g_cur)
+
+
 def test_select_tokens_fp32_near_ties():
     """fp32 similarities are fp64 sums rounded at every addition, in the
     kernel's order on the GPU and in numpy's on the CPU, so mathematically
