@@ -1,7 +1,8 @@
 // GEMMs of the MAR block: QKV, attention output, MLP up and down projections
 // (Eq. 9's F(X[I_compute]) for the token subset, and the full-layer forms).
 //
-// bf16: a persistent, warp-specialised tcgen05 kernel. Warp 0 streams A and W
+// bf16: a persistent, warp-specialised tcgen05 kernel, on single CTAs or on
+// CTA pairs that share a 256-row tile (cta_group::2). Warp 0 streams A and W
 // tiles with TMA (128B swizzle) into a ring of shared-memory stages, warp 1
 // issues tcgen05.mma (128 x BN x 16, fp32 accumulators in tensor memory,
 // double-buffered so the epilogue of one tile overlaps the main loop of the
@@ -106,17 +107,22 @@ constexpr bool is_bf16out() { return EK == BF16OUT || EK == BF16OUT_SILU; }
 // F8: E4M3 operands (kind::f8f6f4): a 128-byte atom holds 128 elements and an
 // MMA step is K = 32, still 32 bytes; BK = 128 is one atom, the bytes of a
 // 64-deep bf16 stage.
-template <int BN, int EK, int BK, int F8 = 0>
+// PAIR: two CTAs (a cluster of two on neighbouring SMs) share a 256 x BN tile.
+// Each holds its own 128 rows of A and half of the tile's B rows, so an SM
+// fills and reads 128 + BN / 2 instead of 128 + BN operand rows per K step; the
+// even CTA issues the MMAs (cta_group::2) for both.
+template <int BN, int EK, int BK, int F8 = 0, int PAIR = 0>
 struct Cfg {
   static constexpr int EB = F8 ? 1 : 2;          // bytes per operand element
   static constexpr int ATOM_E = 128 / EB;        // elements per 128-byte swizzle atom
   static constexpr int ATOMS = BK / ATOM_E;
   // (64-wide tiles, with half the B tile per stage, afford one more stage)
-  static constexpr int STAGES = ATOMS == 2 ? (is_wide<EK>() ? 2 : 3) + (BN == 64 ? 1 : 0)
+  static constexpr int SINGLE_STAGES = ATOMS == 2 ? (is_wide<EK>() ? 2 : 3) + (BN == 64 ? 1 : 0)
                                           : is_wide<EK>() ? (BN == 256 ? 3 : BN == 192 ? 4 : 5)
                                                              : (BN == 256 ? 4 : BN == 192 ? 5 : 6);
   static constexpr uint32_t A_BYTES = BM * BK * EB;
-  static constexpr uint32_t B_BYTES = BN * BK * EB;
+  static constexpr int B_ROWS = PAIR ? BN / 2 : BN;  // rows of B in this CTA's shared memory
+  static constexpr uint32_t B_BYTES = B_ROWS * BK * EB;
   static constexpr uint32_t STAGE_BYTES = A_BYTES + B_BYTES;
   // two accumulator buffers (columns [0, BN) and [BN, 2 BN)); the allocation
   // is a power of two
@@ -136,12 +142,15 @@ struct Cfg {
   static constexpr uint32_t ROW_BYTES = is_wide<EK>() ? 128 : 64;
   static constexpr uint32_t STG_PITCH = is_bf16out<EK>() ? 64 : ROW_BYTES + 16;
   static constexpr uint32_t STG_BYTES = 32 * STG_PITCH;
+  // a pair's smaller stages: as many as shared memory holds, at most eight
+  static constexpr int FIT_STAGES = (int)((232448 - 1024 - 256 - EPI_WARPS * STG_BYTES) / STAGE_BYTES);
+  static constexpr int STAGES = !PAIR ? SINGLE_STAGES : FIT_STAGES < 8 ? FIT_STAGES : 8;
   static constexpr size_t SMEM = 1024 + (size_t)STAGES * STAGE_BYTES + EPI_WARPS * STG_BYTES + 256;
   // Instruction descriptor: D fp32 (bit 4); kind::f16 with A and B bf16
   // (bits 7-9 and 10-12 = 1), or kind::f8f6f4 with A and B E4M3 (format 0);
   // both K-major, N >> 3 at bit 17, M >> 4 at bit 24.
   static constexpr uint32_t IDESC = (1u << 4) | (F8 ? 0u : (1u << 7) | (1u << 10)) | ((uint32_t)(BN >> 3) << 17) |
-                                    ((uint32_t)(BM >> 4) << 24);
+                                    ((uint32_t)((PAIR ? 2 * BM : BM) >> 4) << 24);
 };
 
 // Shared-memory matrix descriptor of a K-major tile written by TMA with
@@ -172,14 +181,14 @@ __device__ __forceinline__ bf16* out_row(const GemmEpi& e, int row, int col) {
 }
 }  // namespace tc
 
-template <int BN, int EK, int BK, int F8 = 0>
-__global__ void __launch_bounds__(tc::Cfg<BN, EK, BK, F8>::THREADS, 1)
+template <int BN, int EK, int BK, int F8 = 0, int PAIR = 0>
+__global__ void __launch_bounds__(tc::Cfg<BN, EK, BK, F8, PAIR>::THREADS, 1)
     gemm_bf16_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                         const __grid_constant__ CUtensorMap tmO0, const __grid_constant__ CUtensorMap tmO1,
                         const __grid_constant__ CUtensorMap tmO2, int tma_out, int M, int N, int K, GemmEpi epi,
                         unsigned* err) {
-  using C = tc::Cfg<BN, EK, BK, F8>;
-  constexpr bool RESID = !tc::is_bf16out<EK>();
+  using C = tc::Cfg<BN, EK, BK, F8, PAIR>;
+  static_assert(!(F8 && PAIR), "pairs: bf16 operands only");
   static_assert(!F8 || EK == tc::BF16OUT, "E4M3 operands: bf16-output epilogue only");
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -198,10 +207,15 @@ __global__ void __launch_bounds__(tc::Cfg<BN, EK, BK, F8>::THREADS, 1)
   // cover a few row tiles completely, so each activation row tile is fetched
   // from memory once and shared through L2 by the CTAs that use it (the
   // weights, at most a few MB, stay in L2 throughout).
-  const int num_m = (M + tc::BM - 1) / tc::BM;
+  constexpr int TM = PAIR ? 2 * tc::BM : tc::BM;  // rows of a tile
+  const int num_m = (M + TM - 1) / TM;
   const int num_n = N / BN;
   const int tiles = num_m * num_n;
   const int KB = K / BK;
+  // a pair works on one tile: the even CTA (rank 0) on its first 128 rows and
+  // the first half of its B rows, the odd one on the others
+  const int rank = PAIR ? (int)cluster_ctarank() : 0;
+  const int first = PAIR ? (int)blockIdx.x / 2 : (int)blockIdx.x, step = PAIR ? (int)gridDim.x / 2 : (int)gridDim.x;
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < C::STAGES; ++s) {
@@ -210,7 +224,7 @@ __global__ void __launch_bounds__(tc::Cfg<BN, EK, BK, F8>::THREADS, 1)
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(&acc_full[b], 1);
-      mbar_init(&acc_empty[b], C::EPI_WARPS);
+      mbar_init(&acc_empty[b], PAIR ? 2 * C::EPI_WARPS : C::EPI_WARPS);  // (of a pair: the even CTA's is used)
     }
     *abort_flag = 0;
     fence_mbar_init();
@@ -225,25 +239,54 @@ __global__ void __launch_bounds__(tc::Cfg<BN, EK, BK, F8>::THREADS, 1)
     }
   }
   if (warp == 1) {
-    tmem_alloc(tmem_slot, C::TMEM_COLS);
-    tmem_relinquish();
+    if (PAIR) {
+      tmem_alloc_pair(tmem_slot, C::TMEM_COLS);
+      tmem_relinquish_pair();
+    } else {
+      tmem_alloc(tmem_slot, C::TMEM_COLS);
+      tmem_relinquish();
+    }
   }
   tc_fence_before();
   __syncthreads();
+  if (PAIR) cluster_sync();  // the peer's barriers are initialised
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  // Tile loads complete on the full barrier of the CTA that issues the MMAs.
+  auto expect_stage = [&](int s) {
+    if (rank == 0) mbar_arrive_expect_tx(&full[s], PAIR ? 2 * C::STAGE_BYTES : C::STAGE_BYTES);
+  };
+  auto load_a = [&](int s, int kb, int m0) {
+#pragma unroll
+    for (int a = 0; a < C::ATOMS; ++a) {
+      uint8_t* dst = sA + s * C::A_BYTES + a * (C::A_BYTES / C::ATOMS);
+      if (PAIR)
+        tma_load_2d_pair(&tmA, cluster_map(smem_u32(&full[s]), 0), dst, kb * BK + a * C::ATOM_E, m0);
+      else
+        tma_load_2d(&tmA, &full[s], dst, kb * BK + a * C::ATOM_E, m0);
+    }
+  };
+  auto load_b = [&](int s, int kb, int n0) {
+#pragma unroll
+    for (int a = 0; a < C::ATOMS; ++a) {
+      uint8_t* dst = sB + s * C::B_BYTES + a * (C::B_BYTES / C::ATOMS);
+      if (PAIR)
+        tma_load_2d_pair(&tmB, cluster_map(smem_u32(&full[s]), 0), dst, kb * BK + a * C::ATOM_E,
+                         n0 + rank * C::B_ROWS);
+      else
+        tma_load_2d(&tmB, &full[s], dst, kb * BK + a * C::ATOM_E, n0);
+    }
+  };
   // Weights are never written by any kernel, so the producer fetches the
   // weight tiles of its first stages before waiting for the predecessor grid;
   // every other access follows pdl_wait().
   int pre = 0;
-  if (warp == 0 && lane == 0 && (int)blockIdx.x < tiles) {
-    const int n0 = ((int)blockIdx.x % num_n) * BN;
+  if (warp == 0 && lane == 0 && first < tiles) {
+    const int n0 = (first % num_n) * BN;
     pre = KB < C::STAGES ? KB : C::STAGES;
     for (int s = 0; s < pre; ++s) {
-      mbar_arrive_expect_tx(&full[s], C::STAGE_BYTES);
-#pragma unroll
-      for (int a = 0; a < C::ATOMS; ++a)
-        tma_load_2d(&tmB, &full[s], sB + s * C::B_BYTES + a * (C::B_BYTES / C::ATOMS), s * BK + a * C::ATOM_E, n0);
+      expect_stage(s);
+      load_b(s, s, n0);
     }
   }
   pdl_wait();
@@ -255,25 +298,17 @@ __global__ void __launch_bounds__(tc::Cfg<BN, EK, BK, F8>::THREADS, 1)
       int stage = 0;
       uint32_t phase = 0;
       bool ok = true;
-      for (int tile = blockIdx.x; tile < tiles && ok; tile += gridDim.x) {
-        const int m0 = (tile / num_n) * tc::BM, n0 = (tile % num_n) * BN;
+      for (int tile = first; tile < tiles && ok; tile += step) {
+        const int m0 = (tile / num_n) * TM + rank * tc::BM, n0 = (tile % num_n) * BN;
         for (int kb = 0; kb < KB; ++kb) {
-          if (tile == (int)blockIdx.x && kb < pre) {
+          if (tile == first && kb < pre) {
             // weight tile already in flight on this stage: add the activations
-#pragma unroll
-            for (int a = 0; a < C::ATOMS; ++a)
-              tma_load_2d(&tmA, &full[stage], sA + stage * C::A_BYTES + a * (C::A_BYTES / C::ATOMS),
-                          kb * BK + a * C::ATOM_E, m0);
+            load_a(stage, kb, m0);
           } else {
             if (!mbar_wait(&empty[stage], phase ^ 1u, abort_flag, err)) { ok = false; break; }
-            mbar_arrive_expect_tx(&full[stage], C::STAGE_BYTES);
-#pragma unroll
-            for (int a = 0; a < C::ATOMS; ++a) {
-              tma_load_2d(&tmA, &full[stage], sA + stage * C::A_BYTES + a * (C::A_BYTES / C::ATOMS),
-                          kb * BK + a * C::ATOM_E, m0);
-              tma_load_2d(&tmB, &full[stage], sB + stage * C::B_BYTES + a * (C::B_BYTES / C::ATOMS),
-                          kb * BK + a * C::ATOM_E, n0);
-            }
+            expect_stage(stage);
+            load_a(stage, kb, m0);
+            load_b(stage, kb, n0);
           }
           if (++stage == C::STAGES) { stage = 0; phase ^= 1u; }
         }
@@ -281,13 +316,13 @@ __global__ void __launch_bounds__(tc::Cfg<BN, EK, BK, F8>::THREADS, 1)
     }
     __syncwarp();
   } else if (warp == 1) {
-    // ---------------- MMA issuer ----------------
-    if (lane == 0) {
+    // ---------------- MMA issuer (of a pair: the even CTA's) ----------------
+    if (lane == 0 && rank == 0) {
       int stage = 0;
       uint32_t phase = 0;
       int it = 0;
       bool ok = true;
-      for (int tile = blockIdx.x; tile < tiles && ok; tile += gridDim.x, ++it) {
+      for (int tile = first; tile < tiles && ok; tile += step, ++it) {
         const int buf = it & 1;
         const uint32_t use = (uint32_t)(it >> 1) & 1u;
         if (!mbar_wait(&acc_empty[buf], use ^ 1u, abort_flag, err)) break;
@@ -303,15 +338,25 @@ __global__ void __launch_bounds__(tc::Cfg<BN, EK, BK, F8>::THREADS, 1)
             const int a = k / 4, ks = k % 4;
             const uint64_t ao = (uint64_t)((a * (C::A_BYTES / C::ATOMS)) >> 4) + 2 * ks;
             const uint64_t bo = (uint64_t)((a * (C::B_BYTES / C::ATOMS)) >> 4) + 2 * ks;
-            if (F8)
+            if (PAIR)
+              umma_bf16_pair(d_tmem, a0 + ao, b0 + bo, C::IDESC, (kb | k) != 0 ? 1u : 0u);
+            else if (F8)
               umma_e4m3(d_tmem, a0 + ao, b0 + bo, C::IDESC, (kb | k) != 0 ? 1u : 0u);
             else
               umma_bf16(d_tmem, a0 + ao, b0 + bo, C::IDESC, (kb | k) != 0 ? 1u : 0u);
           }
-          umma_commit(&empty[stage]);
+          if (PAIR)
+            umma_commit_pair(&empty[stage]);
+          else
+            umma_commit(&empty[stage]);
           if (++stage == C::STAGES) { stage = 0; phase ^= 1u; }
         }
-        if (ok) umma_commit(&acc_full[buf]);
+        if (ok) {
+          if (PAIR)
+            umma_commit_pair(&acc_full[buf]);
+          else
+            umma_commit(&acc_full[buf]);
+        }
       }
     }
     __syncwarp();
@@ -335,10 +380,10 @@ __global__ void __launch_bounds__(tc::Cfg<BN, EK, BK, F8>::THREADS, 1)
     const int cq = lane & 3;        // 16-byte block within the 64-byte row segment
     float* const res_base = static_cast<float*>(epi.out);
     int it = 0;
-    for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x, ++it) {
+    for (int tile = first; tile < tiles; tile += step, ++it) {
       const int buf = it & 1;
       const uint32_t use = (uint32_t)(it >> 1) & 1u;
-      const int m0 = (tile / num_n) * tc::BM, n0 = (tile % num_n) * BN;
+      const int m0 = (tile / num_n) * TM + rank * tc::BM, n0 = (tile % num_n) * BN;
       const int rbase = m0 + quarter * 32;  // first of this warp's 32 rows
       const int c0 = half * CHUNKS;
       // residual of a 32-column chunk in the coalesced layout: [16-col half][pass]
@@ -411,7 +456,12 @@ __global__ void __launch_bounds__(tc::Cfg<BN, EK, BK, F8>::THREADS, 1)
       auto release = [&] {
         tc_fence_before();
         __syncwarp();
-        if (lane == 0) mbar_arrive(&acc_empty[buf]);
+        if (lane == 0) {
+          if (PAIR)
+            mbar_arrive_cluster(cluster_map(smem_u32(&acc_empty[buf]), 0));
+          else
+            mbar_arrive(&acc_empty[buf]);
+        }
       };
       if (PIPE) tld(c0);
 #pragma unroll 1
@@ -587,9 +637,13 @@ __global__ void __launch_bounds__(tc::Cfg<BN, EK, BK, F8>::THREADS, 1)
     if (tma_out && lane == 0) bulk_wait_all();  // stores complete before the CTA exits
   }
   __syncthreads();
+  if (PAIR) cluster_sync();  // neither CTA leaves while the other may arrive on its barriers or use its operands
   if (warp == 1) {
     tc_fence_after();
-    tmem_dealloc(tmem_base, C::TMEM_COLS);
+    if (PAIR)
+      tmem_dealloc_pair(tmem_base, C::TMEM_COLS);
+    else
+      tmem_dealloc(tmem_base, C::TMEM_COLS);
   }
 }
 
@@ -705,21 +759,21 @@ bool gemm_supported(int dtype, int M, int N, int K, const GemmEpi& epi, const ch
   return true;
 }
 
-template <int BN, int EK, int BK, int F8 = 0>
+template <int BN, int EK, int BK, int F8 = 0, int PAIR = 0>
 static cudaError_t launch_tc(const Ctx& c, const void* A, const void* W, int M, int N, int K, const GemmEpi& epi) {
-  using C = tc::Cfg<BN, EK, BK, F8>;
+  using C = tc::Cfg<BN, EK, BK, F8, PAIR>;
   const CUtensorMapDataType dt = F8 ? CU_TENSOR_MAP_DATA_TYPE_UINT8 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;
   CUtensorMap ta, tb;
   if (!make_tmap_2d(dt, &ta, A, (uint64_t)K, (uint64_t)M, (uint64_t)K * C::EB, C::ATOM_E, tc::BM,
                     CU_TENSOR_MAP_SWIZZLE_128B) ||
-      !make_tmap_2d(dt, &tb, W, (uint64_t)K, (uint64_t)N, (uint64_t)K * C::EB, C::ATOM_E, BN,
+      !make_tmap_2d(dt, &tb, W, (uint64_t)K, (uint64_t)N, (uint64_t)K * C::EB, C::ATOM_E, C::B_ROWS,
                     CU_TENSOR_MAP_SWIZZLE_128B))
     return cudaErrorInvalidValue;
   static int attr_set[64] = {};
   int dev = 0;
   cudaGetDevice(&dev);
   if (dev >= 0 && dev < 64 && !attr_set[dev]) {
-    cudaError_t e = cudaFuncSetAttribute(gemm_bf16_tc_kernel<BN, EK, BK, F8>,
+    cudaError_t e = cudaFuncSetAttribute(gemm_bf16_tc_kernel<BN, EK, BK, F8, PAIR>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
     if (e != cudaSuccess) return e;
     attr_set[dev] = 1;
@@ -742,12 +796,20 @@ static cudaError_t launch_tc(const Ctx& c, const void* A, const void* W, int M, 
       return cudaErrorInvalidValue;
     }
   }
+  if (PAIR) {
+    const int tiles = ((M + 2 * tc::BM - 1) / (2 * tc::BM)) * (N / BN);
+    const int pairs = tiles < c.num_sms / 2 ? tiles : c.num_sms / 2;
+    return launch_pdl_cluster(gemm_bf16_tc_kernel<BN, EK, BK, F8, PAIR>, dim3(2 * pairs), dim3(C::THREADS), C::SMEM, 2,
+                              c.stream, ta, tb, to[0], to[1], to[2], tma_out, M, N, K, epi, c.err);
+  }
   const int tiles = ((M + tc::BM - 1) / tc::BM) * (N / BN);
   const int grid = tiles < c.num_sms ? tiles : c.num_sms;
-  return launch_pdl(gemm_bf16_tc_kernel<BN, EK, BK, F8>, dim3(grid), dim3(C::THREADS), C::SMEM, c.stream, ta, tb, to[0], to[1],
-                    to[2], tma_out, M, N, K,
-                    epi, c.err);
+  return launch_pdl(gemm_bf16_tc_kernel<BN, EK, BK, F8, PAIR>, dim3(grid), dim3(C::THREADS), C::SMEM, c.stream, ta, tb,
+                    to[0], to[1], to[2], tma_out, M, N, K, epi, c.err);
 }
+
+// Added to a tile width: tiles of 256 rows on CTA pairs.
+constexpr int kPair = 1000;
 
 // Relative time of one round of tiles of width bn (see launch_gemm).
 static int tile_time(int bn, bool resid_half) {
@@ -759,10 +821,24 @@ static int tile_time(int bn, bool resid_half) {
 }
 
 // Tile width with the fewest rounds of tiles over the SMs x the time of one
-// tile, and that cost.
-static int choose_bn(const Ctx& c, int M, int N, const GemmEpi& epi, int K, long* cost) {
+// tile, and that cost; kPair + width for tiles of 256 rows on CTA pairs.
+//
+// A pair's round is shorter than a single CTA's of the same width, because an
+// SM fills and reads 256 instead of 384 operand rows per K step (measured, us
+// per round: Q/K/V at K = 768 4.7 against 5.5, fc2 at K = 3072 17.5 against
+// 20.3, 14.8 against 16.3 at width 192, out-projection at K = 1024 9.4 against
+// 10.0), but a launch of pairs costs about 1.5 us more, which is 54000 / K of
+// the unit (1 / 256 of a single CTA's 256-wide round). The out-projection at
+// K = 768, bound by its residual rows, is slower on pairs (9.2 against 8.2 us
+// a round). Whole GEMMs, one CTA -> pairs (us): M = 20480, width 768: Q/K/V
+// 55.3 -> 46.8, fc1 68.9 -> 67.5, fc2 81.5 -> 70.2; M = 40960, width 1024: Q/K/V
+// 169.8 -> 148.1, out 91.5 -> 87.3, fc1 226.9 -> 201.0, fc2 228.8 -> 211.0. Where
+// the 256-row tiles need more rounds or there is only one short one, single
+// CTAs win (M = 3200, width 768: Q/K/V 11.9 against 13.5, fc2 15.1 against 19.1).
+static int choose_bn(const Ctx& c, int dtype, int M, int N, const GemmEpi& epi, int K, long* cost) {
   const long mt = (M + tc::BM - 1) / tc::BM;
-  const bool resid_half = epi.mode == LAZYMAR_EPI_RESIDUAL && !epi.gate && K >= 2048;
+  const bool resid = epi.mode == LAZYMAR_EPI_RESIDUAL;
+  const bool resid_half = resid && !epi.gate && K >= 2048;
   const int widths[4] = {256, 192, 128, 64};
   int bn = 128;
   long best = -1;
@@ -774,6 +850,19 @@ static int choose_bn(const Ctx& c, int M, int N, const GemmEpi& epi, int K, long
       best = t;
       bn = widths[i];
     }
+  }
+  if (dtype == LAZYMAR_BF16 && epi.mode != LAZYMAR_EPI_SILU && !epi.gate && !(resid && K < 1024)) {
+    const long pt = (mt + 1) / 2, pairs = c.num_sms / 2;
+    auto consider = [&](int width, int time) {
+      if (pairs < 1 || N % width != 0) return;
+      const long t = (pt * (N / width) + pairs - 1) / pairs * time + 54000 / K;
+      if (t < best) {
+        best = t;
+        bn = kPair + width;
+      }
+    };
+    consider(256, resid_half ? 219 : resid ? 228 : 236);
+    if (resid_half) consider(192, 186);
   }
   *cost = best;
   return bn;
@@ -826,6 +915,12 @@ static cudaError_t launch_bn_impl(const Ctx& c, int dtype, const void* A, const 
                  : epi.gate                          ? tc::RESID_WIDE_GATED
                  : K < 2048                          ? tc::RESID_WIDE
                                                      : tc::RESID_HALF;
+  if (bn == kPair + 192) return launch_tc<192, tc::RESID_HALF, 64, 0, 1>(c, A, W, M, N, K, epi);
+  if (bn == kPair + 256) {
+    if (ek == tc::RESID_WIDE) return launch_tc<256, tc::RESID_WIDE, 64, 0, 1>(c, A, W, M, N, K, epi);
+    if (ek == tc::RESID_HALF) return launch_tc<256, tc::RESID_HALF, 64, 0, 1>(c, A, W, M, N, K, epi);
+    return launch_tc<256, tc::BF16OUT, 64, 0, 1>(c, A, W, M, N, K, epi);
+  }
   if (bn == 192) {
     if (ek == tc::RESID_WIDE) return launch_tc<192, tc::RESID_WIDE, 64>(c, A, W, M, N, K, epi);
     if (ek == tc::RESID_WIDE_GATED) return launch_tc<192, tc::RESID_WIDE_GATED, 64>(c, A, W, M, N, K, epi);
@@ -881,21 +976,20 @@ cudaError_t launch_gemm(const Ctx& c, int dtype, const void* A, const void* W, i
     return e;
   }
   // Tile width: the one with the fewest rounds of tiles over the SMs x the
-  // time of one tile. Relative tile times 187 : 243 : 256 for BN = 128 : 192 :
+  // time of one tile, on single CTAs or pairs (choose_bn). Relative tile times 187 : 243 : 256 for BN = 128 : 192 :
   // 256 (measured, one round of 128 x BN x 3072 tiles): a narrower tile does
   // proportionally less work per pipeline stage and runs well below the
   // BN = 256 rate. BN = 64 (153, on the line through the 128 and 256 points)
   // wins only when the 128-wide tiles fit in one round with SMs to spare: the
   // few-row GEMMs of the diffusion head. The fp32-residual epilogue over long K
   // (fc2) costs in proportion to the tile width: its measured round times at
-  // K = 3072 are 153 : 199 : 256 (110 for 64), under which the full-layer fc2
-  // (480 tiles of 256 in 4 rounds, or 640 of 192 in 5) takes the 192-wide tiles.
+  // K = 3072 are 153 : 199 : 256 (110 for 64).
   if (flags == 2 && N % 256 == 0) return launch_bn(c, dtype, A, W, M, N, K, epi, 256);
   if (flags == 3 && N % 192 == 0) return launch_bn(c, dtype, A, W, M, N, K, epi, 192);
   if (flags == 4) return launch_bn(c, dtype, A, W, M, N, K, epi, 64);
   if (flags != 0) return launch_bn(c, dtype, A, W, M, N, K, epi, 128);
   long cost = 0;
-  const int bn = choose_bn(c, M, N, epi, K, &cost);
+  const int bn = choose_bn(c, dtype, M, N, epi, K, &cost);
   // Last-wave split of the fp32-residual GEMM over short K (the
   // out-projection): when its tiles fill several rounds but the last one only
   // partly, the row tiles of the whole waves run as one launch and the
@@ -907,14 +1001,14 @@ cudaError_t launch_gemm(const Ctx& c, int dtype, const void* A, const void* W, i
   // us). The other kinds lose: the residual over long K (fc2) runs its partial
   // last round faster than a full one (32 tiles of 192 in 10.8 us against
   // 17.1 us), and the full-layer Q/K/V went 55.9 -> 57.6 us split.
-  if (dtype == LAZYMAR_BF16 && epi.mode == LAZYMAR_EPI_RESIDUAL && !epi.gate && K < 2048) {
+  if (dtype == LAZYMAR_BF16 && epi.mode == LAZYMAR_EPI_RESIDUAL && !epi.gate && K < 2048 && bn < kPair) {
     const long mt = (M + tc::BM - 1) / tc::BM, nn = N / bn;
     const long rounds = (mt * nn + c.num_sms - 1) / c.num_sms;
     const long body_rt = rounds >= 3 ? (rounds - 1) * c.num_sms / nn : 0;  // whole row tiles of the full waves
     if (body_rt > 0 && body_rt < mt) {
       const int Mb = (int)(body_rt * tc::BM);
       long tail_cost = 0;
-      const int tail_bn = choose_bn(c, M - Mb, N, epi, K, &tail_cost);
+      const int tail_bn = choose_bn(c, dtype, M - Mb, N, epi, K, &tail_cost);
       const long body_rounds = (body_rt * nn + c.num_sms - 1) / c.num_sms;
       const long split_cost = body_rounds * tile_time(bn, false) + tail_cost;
       if (split_cost * 50 <= cost * 49) {

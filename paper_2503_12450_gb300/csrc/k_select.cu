@@ -222,28 +222,6 @@ __device__ __forceinline__ void sums_bf16(const uint4* sa, const uint4* sc, cons
 
 constexpr int kSelThreads = 256;
 
-__device__ __forceinline__ uint32_t cluster_ctarank() {
-  uint32_t r;
-  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-  return r;
-}
-__device__ __forceinline__ uint32_t cluster_nctarank() {
-  uint32_t r;
-  asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
-  return r;
-}
-// Barrier over the cluster's threads: shared-memory writes of every CTA
-// before it, remote ones included, are visible to every CTA after it.
-__device__ __forceinline__ void cluster_sync() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-// Shared-memory address `saddr` of this CTA as seen in CTA `rank`.
-__device__ __forceinline__ uint32_t cluster_map(uint32_t saddr, uint32_t rank) {
-  uint32_t r;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(saddr), "r"(rank));
-  return r;
-}
-
 // 16 bytes from global to shared memory, and the groups of such copies of
 // this thread (bytes == 0 writes zeros and reads nothing).
 __device__ __forceinline__ void cp_async16(void* dst, const void* src, int bytes) {

@@ -306,6 +306,44 @@ def test_linear_last_wave_split(M, N, K, epi):
         _linear_case("bf16", epi, M, N, K, 0, seed=M + N + K, scatter=False)
 
 
+@pytest.mark.parametrize("M,N,K,epi", [
+    (20353, 2304, 768, lm.LAZYMAR_EPI_QKV),        # one row in the even CTA's half of the last tile
+    (20480, 2304, 768, lm.LAZYMAR_EPI_QKV),
+    (6529, 4096, 1024, lm.LAZYMAR_EPI_GELU),       # one row in the odd CTA's half
+    (8577, 1024, 1024, lm.LAZYMAR_EPI_RESIDUAL),
+    (9700, 768, 3072, lm.LAZYMAR_EPI_RESIDUAL),    # 192-wide pairs
+    (2561, 1280, 5120, lm.LAZYMAR_EPI_RESIDUAL),
+    (12345, 768, 3072, lm.LAZYMAR_EPI_RESIDUAL),
+    (20480, 3072, 832, lm.LAZYMAR_EPI_BIAS),       # 13 K steps: the ring wraps within a tile
+])
+def test_linear_pairs_equal_single_ctas(M, N, K, epi):
+    """At these sizes the automatic choice is 256-row tiles on CTA pairs. An
+    accumulator sums the same products in the same order as a single CTA's, so
+    the results equal the 128-wide tiles' bit for bit; rows past M and cache
+    rows outside the row map stay as they were."""
+    torch = torch_cuda()
+    g = torch.Generator(device="cuda")
+    g.manual_seed(M + N + K)
+    r = lambda *s: torch.randn(s, generator=g, device="cuda")
+    a, w, b = r(M, K).bfloat16(), (0.05 * r(N, K)).bfloat16(), r(N).bfloat16()
+    D = N // 3
+    maps = [None, torch.randperm(M + 40, generator=g, device="cuda")[:M].int()] if epi == lm.LAZYMAR_EPI_QKV else [None]
+    for row_map in maps:
+        res = []
+        for flags in (1, 0):
+            if epi == lm.LAZYMAR_EPI_QKV:
+                outs = [torch.full((M + 40, D), 7.0, device="cuda", dtype=torch.bfloat16) for _ in range(3)]
+                lm.lazymar_linear(DT["bf16"], epi, a, w, b, M, N, K, outs[0], D, outs[1], outs[2], row_map, flags)
+            else:
+                dt = torch.float32 if epi == lm.LAZYMAR_EPI_RESIDUAL else torch.bfloat16
+                outs = [torch.full((M + 40, N), 7.0, device="cuda", dtype=dt)]
+                lm.lazymar_linear(DT["bf16"], epi, a, w, b, M, N, K, outs[0], N, flags=flags)
+            sync()
+            res.append(outs)
+        assert all(torch.equal(x, y) for x, y in zip(*res))
+        assert (res[1][0][M:] == 7.0).all()
+
+
 @pytest.mark.parametrize("M,N,K", [(1, 12, 8), (40, 768, 256), (160, 1024, 256), (77, 256, 1024)])
 @pytest.mark.parametrize("epi", [lm.LAZYMAR_EPI_BIAS, lm.LAZYMAR_EPI_GELU, lm.LAZYMAR_EPI_RESIDUAL,
                                  lm.LAZYMAR_EPI_QKV, lm.LAZYMAR_EPI_SILU])
