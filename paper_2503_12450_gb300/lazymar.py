@@ -145,24 +145,42 @@ def _check(status):
 def _ptr(x):
     if x is None:
         return None
+    f = getattr(x, "data_ptr", None)
+    if f is not None:
+        return f()
     if isinstance(x, int):
         return x
-    if hasattr(x, "data_ptr"):
-        return x.data_ptr()
     if hasattr(x, "ctypes"):
         return x.ctypes.data
     raise TypeError("cannot take the address of %r" % type(x))
 
 
+# torch's (current device, raw current stream of a device) functions, once CUDA
+# is known to be available there. torch.cuda.current_stream() builds a stream
+# object and takes 3 us on the GB300's host, torch.cuda.is_available() 0.8 us;
+# these two calls take 0.24 us (a LayerNorm call: 9.6 -> 4.6 us).
+_raw_stream = None
+
+
+def _current_stream():
+    global _raw_stream
+    if _raw_stream is not None:
+        return _raw_stream[1](_raw_stream[0]())
+    try:
+        import torch
+    except ImportError:
+        return None
+    if not torch.cuda.is_available():
+        return None
+    stream = torch.cuda.current_stream().cuda_stream  # initialises CUDA
+    if hasattr(torch._C, "_cuda_getCurrentRawStream") and hasattr(torch._C, "_cuda_getDevice"):
+        _raw_stream = (torch._C._cuda_getDevice, torch._C._cuda_getCurrentRawStream)
+    return stream
+
+
 def _stream(stream):
     if stream is None:
-        try:
-            import torch
-            if torch.cuda.is_available():
-                return torch.cuda.current_stream().cuda_stream
-        except ImportError:
-            pass
-        return None
+        return _current_stream()
     return stream if isinstance(stream, int) else stream.cuda_stream
 
 
