@@ -692,6 +692,115 @@ __global__ void __launch_bounds__(256) gemm_f32_kernel(const float* __restrict__
   }
 }
 
+// fp32, few tiles: the 64 x 64 tiles of the fp32 configuration's GEMMs leave
+// most SMs idle and each runs its whole K in series (fc2 at M = 40: 4 CTAs, 64
+// K steps of two barriers each). Here a CTA owns a TS x TS tile (16 or 32) and
+// its NW warps split K; each warp computes the whole tile over its slice (TS /
+// 8 rows x TS / 4 columns per lane, float4 along K from its own staged chunk, the next chunk's
+// loads in flight meanwhile), and the partial tiles are summed in warp order
+// through shared memory. Measured,
+// against the 64 x 64 tiles (us): 40 x 768 x 256 13.0 -> 2.5, 40 x 256 x 1024
+// 47.6 -> 5.3, 160 x 1024 x 256 13.2 -> 6.6, 640 x 256 x 1024 48.8 -> 23.0
+constexpr int kF32Chunk = 32;               // K per staged chunk
+constexpr int kF32Pitch = kF32Chunk + 4;    // floats: rows 16 bytes apart in banks
+template <int NW, int TS>
+constexpr int kF32Smem = NW * 2 * TS * kF32Pitch * (int)sizeof(float);
+
+template <int NW, int TS>
+__global__ void __launch_bounds__(NW * 32, NW == 8 || TS == 16 ? 2 : 1) gemm_f32_splitk_kernel(const float* __restrict__ A,
+                                                                  const float* __restrict__ W, int M, int N, int K,
+                                                                  GemmEpi epi) {
+  extern __shared__ __align__(16) float f32_smem[];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int m0 = blockIdx.y * TS, n0 = blockIdx.x * TS;
+  constexpr int P = TS / 4, RI = TS / 8, CJ = TS / 4;  // load passes; rows and columns of a lane
+  float* sA = f32_smem + warp * (2 * TS * kF32Pitch);
+  float* sW = sA + TS * kF32Pitch;
+  const int slice = ((K / 4 + NW - 1) / NW) * 4;
+  const int k0 = min(warp * slice, K), k1 = min(k0 + slice, K);
+  // chunk loads: passes of 4 rows x 8 float4
+  const int lr = lane >> 3, lk = (lane & 7) * 4;
+  float4 ra[P], rw[P];
+  auto fetch = [&](const float* src, int r0, int rows, int k, float4 (&r)[P]) {
+#pragma unroll
+    for (int p = 0; p < P; ++p) {
+      const int row = r0 + p * 4 + lr;
+      r[p] = row < rows && k + lk < k1 ? *reinterpret_cast<const float4*>(src + (size_t)row * K + k + lk)
+                                       : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+  };
+  if (k0 < k1) fetch(W, n0, N, k0, rw);  // weights: no kernel writes them
+  pdl_wait();
+  pdl_trigger();
+  if (k0 < k1) fetch(A, m0, M, k0, ra);
+  float acc[RI][CJ] = {};
+  const int ry = lane >> 2, cx = lane & 3;  // this lane's rows ry + 8 i and columns cx + 4 j: no bank conflicts
+  for (int k = k0; k < k1; k += kF32Chunk) {
+    __syncwarp();
+#pragma unroll
+    for (int p = 0; p < P; ++p) {
+      *reinterpret_cast<float4*>(sA + (p * 4 + lr) * kF32Pitch + lk) = ra[p];
+      *reinterpret_cast<float4*>(sW + (p * 4 + lr) * kF32Pitch + lk) = rw[p];
+    }
+    __syncwarp();
+    if (k + kF32Chunk < k1) {
+      fetch(W, n0, N, k + kF32Chunk, rw);
+      fetch(A, m0, M, k + kF32Chunk, ra);
+    }
+#pragma unroll 2
+    for (int kk = 0; kk < kF32Chunk; kk += 4) {
+      float4 a[RI], w;
+#pragma unroll
+      for (int i = 0; i < RI; ++i) a[i] = *reinterpret_cast<const float4*>(sA + (ry + 8 * i) * kF32Pitch + kk);
+#pragma unroll
+      for (int j = 0; j < CJ; ++j) {
+        w = *reinterpret_cast<const float4*>(sW + (cx + 4 * j) * kF32Pitch + kk);
+#pragma unroll
+        for (int i = 0; i < RI; ++i) {
+          acc[i][j] = fmaf(a[i].x, w.x, acc[i][j]);
+          acc[i][j] = fmaf(a[i].y, w.y, acc[i][j]);
+          acc[i][j] = fmaf(a[i].z, w.z, acc[i][j]);
+          acc[i][j] = fmaf(a[i].w, w.w, acc[i][j]);
+        }
+      }
+    }
+  }
+  // partial tiles over the chunk buffers, then NW-term sums
+  __syncthreads();
+  float* part = f32_smem;
+#pragma unroll
+  for (int i = 0; i < RI; ++i)
+#pragma unroll
+    for (int j = 0; j < CJ; ++j) part[(warp * TS + ry + 8 * i) * kF32Pitch + cx + 4 * j] = acc[i][j];
+  __syncthreads();
+  const int row = threadIdx.x / (TS / 4), col = (threadIdx.x % (TS / 4)) * 4;
+  if (threadIdx.x < TS * TS / 4 && m0 + row < M && n0 + col < N) {
+    float v[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int w = 0; w < NW; ++w) {
+      const float4 q = *reinterpret_cast<const float4*>(part + (w * TS + row) * kF32Pitch + col);
+      v[0] += q.x; v[1] += q.y; v[2] += q.z; v[3] += q.w;
+    }
+    epilogue_apply<float, 4>(epi, m0 + row, n0 + col, v);
+  }
+}
+
+template <int NW, int TS>
+static cudaError_t launch_f32_splitk(const Ctx& c, const float* A, const float* W, int M, int N, int K,
+                                     const GemmEpi& epi) {
+  static int attr_set[64] = {};
+  int dev = 0;
+  cudaGetDevice(&dev);
+  if (dev >= 0 && dev < 64 && !attr_set[dev]) {
+    const cudaError_t e = cudaFuncSetAttribute(gemm_f32_splitk_kernel<NW, TS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               kF32Smem<NW, TS>);
+    if (e != cudaSuccess) return e;
+    attr_set[dev] = 1;
+  }
+  return launch_pdl(gemm_f32_splitk_kernel<NW, TS>, dim3((N + TS - 1) / TS, (M + TS - 1) / TS), dim3(NW * 32),
+                    (size_t)kF32Smem<NW, TS>, c.stream, A, W, M, N, K, epi);
+}
+
 // ---------------------------------------------------------------------------
 // Host side
 // ---------------------------------------------------------------------------
@@ -969,9 +1078,20 @@ cudaError_t launch_gemm(const Ctx& c, int dtype, const void* A, const void* W, i
                         const GemmEpi& epi, int flags) {
   if (M == 0) return cudaSuccess;
   if (dtype == LAZYMAR_F32) {
+    const float *a = static_cast<const float*>(A), *w = static_cast<const float*>(W);
     dim3 grid((N + 63) / 64, (M + 63) / 64);
-    const cudaError_t e = launch_pdl(gemm_f32_kernel, grid, dim3(256), 0, c.stream, static_cast<const float*>(A),
-                                     static_cast<const float*>(W), M, N, K, epi);
+    const long tiles32 = (long)((N + 31) / 32) * ((M + 31) / 32);
+    cudaError_t e;
+    // 64 x 64 tiles once they fill the SMs several times (4 per SM: 2560 x 1024 x
+    // 256 takes 48.5 against 49.4 us; 2560 x 768 x 256 still 48.0 against 38.0);
+    // 16 x 16 tiles while 32 x 32 ones would leave half of the SMs idle (40 x 256 x
+    // 1024: 5.3 against 11.7 us)
+    if ((long)grid.x * grid.y > 4L * c.num_sms)
+      e = launch_pdl(gemm_f32_kernel, grid, dim3(256), 0, c.stream, a, w, M, N, K, epi);
+    else if (tiles32 * 2 <= c.num_sms)
+      e = K > 512 ? launch_f32_splitk<16, 16>(c, a, w, M, N, K, epi) : launch_f32_splitk<8, 16>(c, a, w, M, N, K, epi);
+    else
+      e = K > 512 ? launch_f32_splitk<16, 32>(c, a, w, M, N, K, epi) : launch_f32_splitk<8, 32>(c, a, w, M, N, K, epi);
     if (e == cudaSuccess) ++t_gemm_kernels;
     return e;
   }

@@ -353,6 +353,29 @@ def test_linear_fp32(M, N, K, epi):
     _linear_case("fp32", epi, M, N, K, 0, seed=M + N + K + epi)
 
 
+@pytest.mark.parametrize("M,N,K", [(1, 4, 4), (17, 36, 516), (33, 260, 1028), (160, 1024, 256), (300, 772, 260),
+                                   (2561, 1028, 64), (40, 256, 1024), (9, 2048, 2052)])
+@pytest.mark.parametrize("epi", [lm.LAZYMAR_EPI_GELU, lm.LAZYMAR_EPI_RESIDUAL])
+def test_linear_fp32_tiles(M, N, K, epi):
+    """Edges of the 16, 32 and 64 wide fp32 tiles, slices of K that are uneven,
+    empty or not a multiple of the staged chunk."""
+    _linear_case("fp32", epi, M, N, K, 0, seed=M + N + K + epi)
+
+
+@pytest.mark.parametrize("rows,n_q,T,heads,dh", [(2, 5, 32, 2, 64), (1, 9, 33, 3, 30), (1, 4, 127, 1, 128), (2, 3, 128, 2, 64),
+                                                 (1, 6, 129, 2, 64), (1, 2, 300, 2, 66), (3, 1, 1, 2, 1), (1, 5, 8192, 1, 8)])
+def test_attention_fp32_chunks(rows, n_q, T, heads, dh):
+    """fp32 attention at the edges of its key chunks (32 to 128 keys, one chunk
+    or several) and at head widths that are not a multiple of 4."""
+    D = heads * dh
+    q, k, v = (synth.tensor((rows, n, D), 31 + i) for i, n in enumerate((n_q, T, T)))
+    o = empty((rows, n_q, D))
+    lm.lazymar_attention(DT["fp32"], dev(q), dev(k), dev(v), o, rows, n_q, T, heads, dh)
+    sync()
+    ref = np.stack([O.attention(q[r], k[r], v[r], heads) for r in range(rows)])
+    assert max_rel(host(o), ref) < 1e-5
+
+
 # --------------------------------------------------------------------------
 # E4M3 Q/K/V projection (qkv_e4m3): weight quantization, LayerNorm to E4M3,
 # the kind::f8f6f4 GEMM
