@@ -185,8 +185,8 @@ template <int BN, int EK, int BK, int F8 = 0, int PAIR = 0>
 __global__ void __launch_bounds__(tc::Cfg<BN, EK, BK, F8, PAIR>::THREADS, 1)
     gemm_bf16_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                         const __grid_constant__ CUtensorMap tmO0, const __grid_constant__ CUtensorMap tmO1,
-                        const __grid_constant__ CUtensorMap tmO2, int tma_out, int M, int N, int K, GemmEpi epi,
-                        unsigned* err) {
+                        const __grid_constant__ CUtensorMap tmO2, const __grid_constant__ CUtensorMap tmBt, int whole,
+                        int split, int tma_out, int M, int N, int K, GemmEpi epi, unsigned* err) {
   using C = tc::Cfg<BN, EK, BK, F8, PAIR>;
   static_assert(!(F8 && PAIR), "pairs: bf16 operands only");
   static_assert(!F8 || EK == tc::BF16OUT, "E4M3 operands: bf16-output epilogue only");
@@ -210,7 +210,17 @@ __global__ void __launch_bounds__(tc::Cfg<BN, EK, BK, F8, PAIR>::THREADS, 1)
   constexpr int TM = PAIR ? 2 * tc::BM : tc::BM;  // rows of a tile
   const int num_m = (M + TM - 1) / TM;
   const int num_n = N / BN;
-  const int tiles = num_m * num_n;
+  // Pairs: `whole` tiles of the full width, then the others as `split` tiles of
+  // BN / split columns each, which spread a short last round over all SMs.
+  const int tiles = PAIR ? whole + (num_m * num_n - whole) * split : num_m * num_n;
+  struct Tile {
+    int m, n, bn;  // first row and column of the (pair's) tile, and its width
+  };
+  auto tile_at = [&](int t) {
+    if (!PAIR || t < whole) return Tile{(t / num_n) * TM, (t % num_n) * BN, BN};
+    const int u = t - whole, base = whole + u / split, bw = BN / split;
+    return Tile{(base / num_n) * TM, (base % num_n) * BN + (u % split) * bw, bw};
+  };
   const int KB = K / BK;
   // a pair works on one tile: the even CTA (rank 0) on its first 128 rows and
   // the first half of its B rows, the odd one on the others
@@ -253,8 +263,9 @@ __global__ void __launch_bounds__(tc::Cfg<BN, EK, BK, F8, PAIR>::THREADS, 1)
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
   // Tile loads complete on the full barrier of the CTA that issues the MMAs.
-  auto expect_stage = [&](int s) {
-    if (rank == 0) mbar_arrive_expect_tx(&full[s], PAIR ? 2 * C::STAGE_BYTES : C::STAGE_BYTES);
+  auto expect_stage = [&](int s, int bw) {
+    if (rank == 0)
+      mbar_arrive_expect_tx(&full[s], PAIR ? 2 * (C::A_BYTES + (uint32_t)bw * BK) : C::STAGE_BYTES);
   };
   auto load_a = [&](int s, int kb, int m0) {
 #pragma unroll
@@ -266,13 +277,13 @@ __global__ void __launch_bounds__(tc::Cfg<BN, EK, BK, F8, PAIR>::THREADS, 1)
         tma_load_2d(&tmA, &full[s], dst, kb * BK + a * C::ATOM_E, m0);
     }
   };
-  auto load_b = [&](int s, int kb, int n0) {
+  auto load_b = [&](int s, int kb, int n0, int bw) {
 #pragma unroll
     for (int a = 0; a < C::ATOMS; ++a) {
       uint8_t* dst = sB + s * C::B_BYTES + a * (C::B_BYTES / C::ATOMS);
       if (PAIR)
-        tma_load_2d_pair(&tmB, cluster_map(smem_u32(&full[s]), 0), dst, kb * BK + a * C::ATOM_E,
-                         n0 + rank * C::B_ROWS);
+        tma_load_2d_pair(bw == BN ? &tmB : &tmBt, cluster_map(smem_u32(&full[s]), 0), dst, kb * BK + a * C::ATOM_E,
+                         n0 + rank * (bw / 2));
       else
         tma_load_2d(&tmB, &full[s], dst, kb * BK + a * C::ATOM_E, n0);
     }
@@ -282,11 +293,11 @@ __global__ void __launch_bounds__(tc::Cfg<BN, EK, BK, F8, PAIR>::THREADS, 1)
   // every other access follows pdl_wait().
   int pre = 0;
   if (warp == 0 && lane == 0 && first < tiles) {
-    const int n0 = (first % num_n) * BN;
+    const Tile t = tile_at(first);
     pre = KB < C::STAGES ? KB : C::STAGES;
     for (int s = 0; s < pre; ++s) {
-      expect_stage(s);
-      load_b(s, s, n0);
+      expect_stage(s, t.bn);
+      load_b(s, s, t.n, t.bn);
     }
   }
   pdl_wait();
@@ -299,16 +310,17 @@ __global__ void __launch_bounds__(tc::Cfg<BN, EK, BK, F8, PAIR>::THREADS, 1)
       uint32_t phase = 0;
       bool ok = true;
       for (int tile = first; tile < tiles && ok; tile += step) {
-        const int m0 = (tile / num_n) * TM + rank * tc::BM, n0 = (tile % num_n) * BN;
+        const Tile t = tile_at(tile);
+        const int m0 = t.m + rank * tc::BM, n0 = t.n;
         for (int kb = 0; kb < KB; ++kb) {
           if (tile == first && kb < pre) {
             // weight tile already in flight on this stage: add the activations
             load_a(stage, kb, m0);
           } else {
             if (!mbar_wait(&empty[stage], phase ^ 1u, abort_flag, err)) { ok = false; break; }
-            expect_stage(stage);
+            expect_stage(stage, t.bn);
             load_a(stage, kb, m0);
-            load_b(stage, kb, n0);
+            load_b(stage, kb, n0, t.bn);
           }
           if (++stage == C::STAGES) { stage = 0; phase ^= 1u; }
         }
@@ -328,6 +340,8 @@ __global__ void __launch_bounds__(tc::Cfg<BN, EK, BK, F8, PAIR>::THREADS, 1)
         if (!mbar_wait(&acc_empty[buf], use ^ 1u, abort_flag, err)) break;
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + (uint32_t)(buf * BN);
+        // N of the MMAs (bits 17 up of the instruction descriptor)
+        const uint32_t idesc = PAIR ? C::IDESC - ((uint32_t)((BN - tile_at(tile).bn) >> 3) << 17) : C::IDESC;
         for (int kb = 0; kb < KB; ++kb) {
           if (!mbar_wait(&full[stage], phase, abort_flag, err)) { ok = false; break; }
           tc_fence_after();
@@ -339,7 +353,7 @@ __global__ void __launch_bounds__(tc::Cfg<BN, EK, BK, F8, PAIR>::THREADS, 1)
             const uint64_t ao = (uint64_t)((a * (C::A_BYTES / C::ATOMS)) >> 4) + 2 * ks;
             const uint64_t bo = (uint64_t)((a * (C::B_BYTES / C::ATOMS)) >> 4) + 2 * ks;
             if (PAIR)
-              umma_bf16_pair(d_tmem, a0 + ao, b0 + bo, C::IDESC, (kb | k) != 0 ? 1u : 0u);
+              umma_bf16_pair(d_tmem, a0 + ao, b0 + bo, idesc, (kb | k) != 0 ? 1u : 0u);
             else if (F8)
               umma_e4m3(d_tmem, a0 + ao, b0 + bo, C::IDESC, (kb | k) != 0 ? 1u : 0u);
             else
@@ -383,9 +397,13 @@ __global__ void __launch_bounds__(tc::Cfg<BN, EK, BK, F8, PAIR>::THREADS, 1)
     for (int tile = first; tile < tiles; tile += step, ++it) {
       const int buf = it & 1;
       const uint32_t use = (uint32_t)(it >> 1) & 1u;
-      const int m0 = (tile / num_n) * TM + rank * tc::BM, n0 = (tile % num_n) * BN;
+      const Tile t = tile_at(tile);
+      const int m0 = t.m + rank * tc::BM, n0 = t.n;
       const int rbase = m0 + quarter * 32;  // first of this warp's 32 rows
-      const int c0 = half * CHUNKS;
+      // this warp's chunks: a narrower tile gives each warp fewer, some none
+      const int per = t.bn == BN ? CHUNKS : (t.bn / 32 + C::EPI_WARPS / 4 - 1) / (C::EPI_WARPS / 4);
+      const int c0 = half * per;
+      const int c1 = t.bn == BN ? c0 + CHUNKS : min(c0 + per, t.bn / 32);
       // residual of a 32-column chunk in the coalesced layout: [16-col half][pass]
       float4 res[2][4];
       uint2 rbias[2];  // the 4 bias values of this lane's columns in each 16-column half (bf16)
@@ -433,9 +451,10 @@ __global__ void __launch_bounds__(tc::Cfg<BN, EK, BK, F8, PAIR>::THREADS, 1)
           for (int j = 0; j < 4; ++j) bpre[j] = bp[j];
         }
       };
-      if (EK == tc::RESID_HALF) load_res(n0 + c0 * 32);
-      if (tc::is_wide<EK>()) load_resw(n0 + c0 * 32);
-      if (tc::is_bf16out<EK>() && !F8) load_bias(n0 + c0 * 32);
+      const bool some = !PAIR || c0 < c1;
+      if (EK == tc::RESID_HALF && some) load_res(n0 + c0 * 32);
+      if (tc::is_wide<EK>() && some) load_resw(n0 + c0 * 32);
+      if (tc::is_bf16out<EK>() && !F8 && some) load_bias(n0 + c0 * 32);
       const bool ok = mbar_wait(&acc_full[buf], use, abort_flag, err);
       if (__any_sync(0xffffffffu, !ok)) break;
       tc_fence_after();
@@ -463,11 +482,15 @@ __global__ void __launch_bounds__(tc::Cfg<BN, EK, BK, F8, PAIR>::THREADS, 1)
             mbar_arrive(&acc_empty[buf]);
         }
       };
+      if (!some) {
+        release();
+        continue;
+      }
       if (PIPE) tld(c0);
 #pragma unroll 1
-      for (int c = c0; c < c0 + CHUNKS; ++c) {
+      for (int c = c0; c < c1; ++c) {
         const int col = n0 + c * 32;
-        const bool more = c + 1 < c0 + CHUNKS;
+        const bool more = c + 1 < c1;
         if (!PIPE) tld(c);
         tmem_wait_ld_regs(r);
         if (tc::is_wide<EK>()) {
@@ -489,7 +512,7 @@ __global__ void __launch_bounds__(tc::Cfg<BN, EK, BK, F8, PAIR>::THREADS, 1)
             cur[p] = resw[p];
             if (EK == tc::RESID_WIDE_GATED) curg[p] = gatew[p];
           }
-          if (c + 1 < c0 + CHUNKS) load_resw(col + 32);  // prefetch the next chunk
+          if (c + 1 < c1) load_resw(col + 32);  // prefetch the next chunk
 #pragma unroll
           for (int p = 0; p < 8; ++p) {
             const int lr = p * 4 + wr;
@@ -520,7 +543,7 @@ __global__ void __launch_bounds__(tc::Cfg<BN, EK, BK, F8, PAIR>::THREADS, 1)
 #pragma unroll
             for (int p = 0; p < 4; ++p) cur[h][p] = res[h][p];
           const uint2 cbias[2] = {rbias[0], rbias[1]};  // prefetched with the residual
-          if (c + 1 < c0 + CHUNKS) load_res(col + 32);  // prefetch the next chunk
+          if (c + 1 < c1) load_res(col + 32);  // prefetch the next chunk
 #pragma unroll
           for (int h = 0; h < 2; ++h) {
             // stage 16 raw fp32 accumulator columns of this thread's row
@@ -583,7 +606,7 @@ __global__ void __launch_bounds__(tc::Cfg<BN, EK, BK, F8, PAIR>::THREADS, 1)
               for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
             }
             // the next chunk's bias loads while this chunk is converted and stored
-            if (c + 1 < c0 + CHUNKS) load_bias(col + 32);
+            if (c + 1 < c1) load_bias(col + 32);
           }
           if (EK == tc::BF16OUT_SILU) {
 #pragma unroll
@@ -868,6 +891,31 @@ bool gemm_supported(int dtype, int M, int N, int K, const GemmEpi& epi, const ch
   return true;
 }
 
+// How `base` tiles of width bn run on `pairs` CTA pairs: `whole` of them at full
+// width, the others, a last round that would leave pairs idle, as `split` tiles
+// each. Returns the cost of all rounds, `time` being a full-width round's.
+static long pair_rounds(long base, long pairs, int bn, long time, int* whole, int* split) {
+  const long rounds = base / pairs, rem = base - rounds * pairs;
+  *whole = (int)base;
+  *split = 1;
+  if (rem == 0) return rounds * time;
+  long best = time;
+  // a round of half-width tiles takes about 68 %, of quarter-width ones 50 % of a
+  // full one. Measured, one launch of equal tiles -> with a split last round (us):
+  // M = 20480, width 768: fc2 69.1 -> 65.3; width 1024: out 51.2 -> 47.9, fc2
+  // 111.3 -> 104.7; M = 5440, width 1024: out 17.4 -> 15.0, fc2 44.4 -> 38.4
+  if (rounds > 0)
+    for (int s = 2; s <= 4; s *= 2) {
+      const long t = (rem * s + pairs - 1) / pairs * (time * (s == 2 ? 68 : 50) / 100);
+      if (bn % (64 * s) == 0 && t < best) {
+        best = t;
+        *whole = (int)(rounds * pairs);
+        *split = s;
+      }
+    }
+  return rounds * time + best;
+}
+
 template <int BN, int EK, int BK, int F8 = 0, int PAIR = 0>
 static cudaError_t launch_tc(const Ctx& c, const void* A, const void* W, int M, int N, int K, const GemmEpi& epi) {
   using C = tc::Cfg<BN, EK, BK, F8, PAIR>;
@@ -905,16 +953,24 @@ static cudaError_t launch_tc(const Ctx& c, const void* A, const void* W, int M, 
       return cudaErrorInvalidValue;
     }
   }
+  CUtensorMap tbt = tb;
   if (PAIR) {
-    const int tiles = ((M + 2 * tc::BM - 1) / (2 * tc::BM)) * (N / BN);
+    const int base = ((M + 2 * tc::BM - 1) / (2 * tc::BM)) * (N / BN);
+    int whole = 0, split = 1;
+    pair_rounds(base, c.num_sms / 2, BN, 100, &whole, &split);
+    const int tiles = whole + (base - whole) * split;
+    if (split > 1 && !make_tmap_2d(dt, &tbt, W, (uint64_t)K, (uint64_t)N, (uint64_t)K * C::EB, C::ATOM_E,
+                                   BN / split / 2, CU_TENSOR_MAP_SWIZZLE_128B))
+      return cudaErrorInvalidValue;
     const int pairs = tiles < c.num_sms / 2 ? tiles : c.num_sms / 2;
     return launch_pdl_cluster(gemm_bf16_tc_kernel<BN, EK, BK, F8, PAIR>, dim3(2 * pairs), dim3(C::THREADS), C::SMEM, 2,
-                              c.stream, ta, tb, to[0], to[1], to[2], tma_out, M, N, K, epi, c.err);
+                              c.stream, ta, tb, to[0], to[1], to[2], tbt, whole, split, tma_out, M, N, K,
+                              epi, c.err);
   }
   const int tiles = ((M + tc::BM - 1) / tc::BM) * (N / BN);
   const int grid = tiles < c.num_sms ? tiles : c.num_sms;
   return launch_pdl(gemm_bf16_tc_kernel<BN, EK, BK, F8, PAIR>, dim3(grid), dim3(C::THREADS), C::SMEM, c.stream, ta, tb,
-                    to[0], to[1], to[2], tma_out, M, N, K, epi, c.err);
+                    to[0], to[1], to[2], tbt, 0, 1, tma_out, M, N, K, epi, c.err);
 }
 
 // Added to a tile width: tiles of 256 rows on CTA pairs.
@@ -964,7 +1020,8 @@ static int choose_bn(const Ctx& c, int dtype, int M, int N, const GemmEpi& epi, 
     const long pt = (mt + 1) / 2, pairs = c.num_sms / 2;
     auto consider = [&](int width, int time) {
       if (pairs < 1 || N % width != 0) return;
-      const long t = (pt * (N / width) + pairs - 1) / pairs * time + 54000 / K;
+      int whole, split;
+      const long t = pair_rounds(pt * (N / width), pairs, width, time, &whole, &split) + 54000 / K;
       if (t < best) {
         best = t;
         bn = kPair + width;

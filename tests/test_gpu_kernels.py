@@ -315,6 +315,10 @@ def test_linear_last_wave_split(M, N, K, epi):
     (2561, 1280, 5120, lm.LAZYMAR_EPI_RESIDUAL),
     (12345, 768, 3072, lm.LAZYMAR_EPI_RESIDUAL),
     (20480, 3072, 832, lm.LAZYMAR_EPI_BIAS),       # 13 K steps: the ring wraps within a tile
+    # a last round of 64-wide tiles (the first three also have one of 128-wide ones)
+    (20480, 768, 3072, lm.LAZYMAR_EPI_RESIDUAL),
+    (10001, 1024, 1024, lm.LAZYMAR_EPI_RESIDUAL),
+    (5000, 1024, 1024, lm.LAZYMAR_EPI_BIAS),
 ])
 def test_linear_pairs_equal_single_ctas(M, N, K, epi):
     """At these sizes the automatic choice is 256-row tiles on CTA pairs. An
