@@ -333,6 +333,7 @@ __global__ void __launch_bounds__(kSelThreads, NCH <= 3 ? 4 : 2)
   if (N == 0) return;  // uniform over the cluster: nothing to rank
   if (!need_s)
     for (int t = tid; t < n_tok; t += kSelThreads) sK[t] = rkeys[row0 + t];
+  __syncwarp();
   cluster_sync();
   // rank of token t: one warp per token, its lanes sharing the row's keys;
   // I_compute = rank < N
@@ -365,6 +366,7 @@ __global__ void __launch_bounds__(kSelThreads, NCH <= 3 ? 4 : 2)
       asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(cluster_map(smem_u32(s_count + me), (uint32_t)lane)), "r"(n)
                    : "memory");
   }
+  __syncwarp();
   cluster_sync();  // also: no CTA exits while another may still write to it
   int base = 0;
   for (uint32_t p = 0; p < me; ++p) base += s_count[p];

@@ -348,6 +348,38 @@ def test_linear_pairs_equal_single_ctas(M, N, K, epi):
         assert (res[1][0][M:] == 7.0).all()
 
 
+@pytest.mark.parametrize("M,N,K", [(1, 384, 128), (63, 768, 256), (65, 768, 3072), (200, 2304, 768), (449, 1024, 1024),
+                                   (320, 1536, 640)])
+@pytest.mark.parametrize("epi", [lm.LAZYMAR_EPI_BIAS, lm.LAZYMAR_EPI_GELU, lm.LAZYMAR_EPI_RESIDUAL,
+                                 lm.LAZYMAR_EPI_QKV, lm.LAZYMAR_EPI_SILU])
+def test_linear_few_rows_equal_128_row_tiles(M, N, K, epi):
+    """Few rows take 64-row tiles (K % 128 == 0, one round of 64 x 64 tiles):
+    bit for bit the 128-row tiles' results, rows past M untouched."""
+    torch = torch_cuda()
+    g = torch.Generator(device="cuda")
+    g.manual_seed(M + N + K + epi)
+    r = lambda *s: torch.randn(s, generator=g, device="cuda")
+    a, w, b = r(M, K).bfloat16(), (0.05 * r(N, K)).bfloat16(), r(N).bfloat16()
+    D = N // 3
+    if epi == lm.LAZYMAR_EPI_QKV and (N % 3 or D % 32):
+        pytest.skip("not a QKV shape")
+    maps = [None, torch.randperm(M + 40, generator=g, device="cuda")[:M].int()] if epi == lm.LAZYMAR_EPI_QKV else [None]
+    for row_map in maps:
+        res = []
+        for flags in (1, 0):
+            if epi == lm.LAZYMAR_EPI_QKV:
+                outs = [torch.full((M + 40, D), 7.0, device="cuda", dtype=torch.bfloat16) for _ in range(3)]
+                lm.lazymar_linear(DT["bf16"], epi, a, w, b, M, N, K, outs[0], D, outs[1], outs[2], row_map, flags)
+            else:
+                dt = torch.float32 if epi == lm.LAZYMAR_EPI_RESIDUAL else torch.bfloat16
+                outs = [torch.full((M + 40, N), 7.0, device="cuda", dtype=dt)]
+                lm.lazymar_linear(DT["bf16"], epi, a, w, b, M, N, K, outs[0], N, flags=flags)
+            sync()
+            res.append(outs)
+        assert all(torch.equal(x, y) for x, y in zip(*res))
+        assert (res[1][0][M:] == 7.0).all()
+
+
 @pytest.mark.parametrize("M,N,K", [(1, 12, 8), (40, 768, 256), (160, 1024, 256), (77, 256, 1024)])
 @pytest.mark.parametrize("epi", [lm.LAZYMAR_EPI_BIAS, lm.LAZYMAR_EPI_GELU, lm.LAZYMAR_EPI_RESIDUAL,
                                  lm.LAZYMAR_EPI_QKV, lm.LAZYMAR_EPI_SILU])
