@@ -3,9 +3,10 @@
 // sequence, fresh ones for I_compute and cached ones for I_cache (Eq. 9). The
 // full-layer form is the same kernel with every token as a query.
 //
-// bf16: attention_tc_kernel, tcgen05 tensor cores with the accumulators in
-// tensor memory and Q/K/V tiles staged by TMA, for heads of width 64 (MAR-B,
-// MAR-L) and 80 (MAR-H).
+// bf16: attention_tc_kernel and attention_tm_kernel, tcgen05 tensor cores with
+// the accumulators in tensor memory and Q/K/V tiles staged by TMA, for heads of
+// width 64 (MAR-B, MAR-L) and 80 (MAR-H); the latter keeps the probabilities in
+// tensor memory too and serves the larger grids.
 //
 // f32: one warp per query on CUDA cores (fp32 configuration).
 #include <cuda.h>
@@ -297,21 +298,21 @@ __global__ void __launch_bounds__(at2::THREADS, at2::Cfg<DH>::MIN_BLOCKS)
           umma_bf16(tmem, sw32_desc(smem_u32(sQ2)), sw32_desc(smem_u32(sK2 + (c & 1) * KV2_BYTES)), IDESC_S, 1u);
         umma_commit(&bars[B_S_FULL]);
       };
-      bool ok = mbar_wait(&bars[B_Q], 0, abort_flag, err) && mbar_wait(&bars[B_K], 0, abort_flag, err);
+      bool ok = mbar_wait<false>(&bars[B_Q], 0, abort_flag, err) && mbar_wait<false>(&bars[B_K], 0, abort_flag, err);
       if (ok) {
         tc_fence_after();
         issue_s(0);
       }
       for (int c = 0; c < nck && ok; ++c) {
         if (c + 1 < nck) {
-          ok = mbar_wait(&bars[B_K + ((c + 1) & 1)], (uint32_t)((c + 1) >> 1) & 1u, abort_flag, err) &&
-               mbar_wait(&bars[B_S_FREE], (uint32_t)c & 1u, abort_flag, err);
+          ok = mbar_wait<false>(&bars[B_K + ((c + 1) & 1)], (uint32_t)((c + 1) >> 1) & 1u, abort_flag, err) &&
+               mbar_wait<false>(&bars[B_S_FREE], (uint32_t)c & 1u, abort_flag, err);
           if (!ok) break;
           tc_fence_after();
           issue_s(c + 1);
         }
-        ok = mbar_wait(&bars[B_P_FULL], (uint32_t)c & 1u, abort_flag, err) &&
-             mbar_wait(&bars[B_V + (c & 1)], (uint32_t)(c >> 1) & 1u, abort_flag, err);
+        ok = mbar_wait<false>(&bars[B_P_FULL], (uint32_t)c & 1u, abort_flag, err) &&
+             mbar_wait<false>(&bars[B_V + (c & 1)], (uint32_t)(c >> 1) & 1u, abort_flag, err);
         if (!ok) break;
         tc_fence_after();
         // 16 keys per MMA: 16 rows of the MN-major V tile = 2048 bytes (512
@@ -342,7 +343,7 @@ __global__ void __launch_bounds__(at2::THREADS, at2::Cfg<DH>::MIN_BLOCKS)
     float m_run = -FLT_MAX, l_run = 0.f;
     bool ok = true;
     for (int c = 0; c < nck; ++c) {
-      ok = __all_sync(0xffffffffu, mbar_wait(&bars[B_S_FULL], (uint32_t)c & 1u, abort_flag, err));
+      ok = __all_sync(0xffffffffu, mbar_wait<false>(&bars[B_S_FULL], (uint32_t)c & 1u, abort_flag, err));
       if (!ok) break;
       tc_fence_after();
       if (tid == 0 && c + 2 < nck) load_k(c + 2);  // S(c) has read K stage c & 1
@@ -410,7 +411,7 @@ __global__ void __launch_bounds__(at2::THREADS, at2::Cfg<DH>::MIN_BLOCKS)
       const float psum = ps0 + ps1;
       // PV(c-1) must be complete before O is rescaled or P is overwritten.
       if (c > 0) {
-        ok = __all_sync(0xffffffffu, mbar_wait(&bars[B_O_DONE], (uint32_t)(c - 1) & 1u, abort_flag, err));
+        ok = __all_sync(0xffffffffu, mbar_wait<false>(&bars[B_O_DONE], (uint32_t)(c - 1) & 1u, abort_flag, err));
         if (!ok) break;
         tc_fence_after();
         if (tid == 0 && c + 1 < nck) load_v(c + 1);  // V stage (c + 1) & 1 held V(c - 1)
@@ -447,7 +448,7 @@ __global__ void __launch_bounds__(at2::THREADS, at2::Cfg<DH>::MIN_BLOCKS)
     // epilogue: O / l for this row, staged through the P tile for whole-row
     // stores of the first 64 columns; the 16-column remainder of an 80-wide
     // head is stored by each thread (32 contiguous bytes)
-    if (ok) ok = __all_sync(0xffffffffu, mbar_wait(&bars[B_O_DONE], (uint32_t)(nck - 1) & 1u, abort_flag, err));
+    if (ok) ok = __all_sync(0xffffffffu, mbar_wait<false>(&bars[B_O_DONE], (uint32_t)(nck - 1) & 1u, abort_flag, err));
     if (ok) {
       tc_fence_after();
       const float inv = 1.f / l_run;
@@ -497,6 +498,374 @@ __global__ void __launch_bounds__(at2::THREADS, at2::Cfg<DH>::MIN_BLOCKS)
         const int qi = qt * QT + row;
         if (qi < n_q) {
           const uint4 val = *reinterpret_cast<const uint4*>(sP + sw(row, ch));
+          *reinterpret_cast<uint4*>(o + (size_t)(r * n_q + qi) * D + col + 8 * ch) = val;
+        }
+      }
+    }
+    tc_fence_before();
+  }
+  __syncthreads();
+  if (warp == 4) {
+    tc_fence_after();
+    tmem_dealloc(tmem, C::TMEM_COLS);
+  }
+}
+
+// One CTA per (128-query tile, head, row), four CTAs per SM. Warps 0-3 run the
+// softmax (thread t owns query row t = tensor-memory lane t); lane 0 of warp 4
+// issues the loads and the MMAs. Keys stream in chunks c of KC:
+//   S(c)  = Q K(c)^T      (tcgen05.mma 128 x KC x DH, K-major operands) into
+//                         tensor-memory columns [0, KC);
+//   P(c)  = exp2(S(c) * log2(e)/sqrt(d) - m), written back as packed bf16 over
+//                         the columns [0, KC / 2) of the scores it came from;
+//   O    += P(c) V(c)     (A = P from tensor memory, B = the V tile as loaded,
+//                         MN-major) into columns [KC, KC + DH), accumulated
+//                         across chunks; then S(c + 1) may overwrite P(c).
+// The chunks of one CTA form a serial chain; the other three CTAs' chains fill
+// its gaps. An MMA lasts as long as its shared-memory operands take to read, 64
+// cycles for 128 rows of A whatever N is, so P V with P in shared memory cost
+// the tensor pipe as much as S (and P's way there a proxy fence per chunk).
+// Measured, against attention_tc_kernel (us): 64 rows x 12 heads x 320 x 320 of
+// width 64 45.2 -> 39.6, 128 x 16 109 -> 93.4, 16 x 16 x 1088 x 1088 118 -> 101; of
+// width 80, 64 x 16 x 320 x 320 85.9 -> 67.4, 50 queries 32.2 -> 26.7.
+//
+// The running max m is raised only when a row's chunk max exceeds it by more
+// than 8 (log2 units): the final O / l is the same for any m that is at least
+// every key's score - 8 and P stays below 2^8, while O in tensor memory is
+// rescaled only on those (rare) raises. K and V have two-stage rings: K(c + 2)
+// refills once S(c) has been read, V(c + 2) once P(c) V(c) is complete.
+//
+// A head of width 80: Q and K are a 64-column part (128-byte swizzle, as for
+// width 64) and a 16-column remainder (32-byte swizzle: rows of 32 bytes, 8-row
+// groups 256 bytes apart), and S takes four 16-deep MMAs on the first part and
+// one on the remainder. V is five panels of 16 columns with the 32-byte
+// swizzle, so that P V is one MMA of N = 80 per 16 keys. 48 keys per chunk keep
+// S and O within 128 columns.
+namespace at4 {
+constexpr int QT = 128;   // queries per CTA (MMA M)
+constexpr int THREADS = 160;
+constexpr int Q_BYTES = QT * 128;    // 128 rows x 64 bf16, 128B swizzle (also the output staging tile)
+constexpr int Q2_BYTES = QT * 32;    // 128 rows x 16 bf16, 32B swizzle (80-wide heads)
+constexpr float RESCALE_THRESHOLD = 8.0f;
+template <int DH>
+struct Cfg {
+  static_assert(DH == 64 || DH == 80, "head width 64 or 80");
+  static constexpr bool TAIL = DH == 80;
+  static constexpr int KC = TAIL ? 48 : 64;  // keys per chunk
+  static constexpr int K_BYTES = KC * 128;   // KC rows x 64 bf16
+  static constexpr int K2_BYTES = TAIL ? KC * 32 : 0;  // KC rows x 16 bf16
+  static constexpr int V_BYTES = KC * DH * 2;
+  static constexpr int SMEM = 1024 + Q_BYTES + (TAIL ? Q2_BYTES : 0) + 2 * (K_BYTES + K2_BYTES + V_BYTES) + 256;
+  static constexpr uint32_t TMEM_COLS = 128;  // S [0, KC), P [0, KC / 2), O [KC, KC + DH)
+  static constexpr uint32_t Q_TX = Q_BYTES + (TAIL ? Q2_BYTES : 0);
+  static constexpr uint32_t K_TX = K_BYTES + K2_BYTES;
+  static constexpr uint32_t V_TX = V_BYTES;
+  static constexpr int MIN_BLOCKS = 4;
+  static_assert(KC + DH <= 128 && MIN_BLOCKS * (SMEM + 1024) <= 233472, "four CTAs per SM");
+};
+// kind::f16, D fp32, A/B bf16, M = 128, N = n; bit 16 marks B as MN-major.
+constexpr uint32_t idesc(int n) {
+  return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
+}
+// Shared-memory descriptors, 128B swizzle. K-major operand (Q, K): the stride
+// between 8-row groups (SBO) is 1024 B, the leading offset unused (1). MN-major
+// V tile (rows = keys = the K dimension, 64 head dims = one 128-byte swizzle
+// atom along N): 8-key groups are 1024 B apart; N is a single atom, so the
+// N-direction offset never applies and is given the same 1024 B.
+__device__ __forceinline__ uint64_t sw128_desc(uint32_t saddr) {
+  return (uint64_t)((saddr >> 4) & 0x3FFFu) | ((uint64_t)1 << 16) | ((uint64_t)(1024 >> 4) << 32) |
+         ((uint64_t)1 << 46) | ((uint64_t)2 << 61);
+}
+__device__ __forceinline__ uint64_t sw128_mn_desc(uint32_t saddr) {
+  return (uint64_t)((saddr >> 4) & 0x3FFFu) | ((uint64_t)(1024 >> 4) << 16) | ((uint64_t)(1024 >> 4) << 32) |
+         ((uint64_t)1 << 46) | ((uint64_t)2 << 61);
+}
+// 32B swizzle (layout 6), 32-byte rows in 8-row groups 256 B apart (SBO); as an
+// MN-major operand the 16-column atoms along N are `panel` bytes apart (LBO).
+__device__ __forceinline__ uint64_t sw32_desc(uint32_t saddr, uint32_t panel) {
+  return (uint64_t)((saddr >> 4) & 0x3FFFu) | ((uint64_t)(panel >> 4) << 16) | ((uint64_t)(256 >> 4) << 32) |
+         ((uint64_t)1 << 46) | ((uint64_t)6 << 61);
+}
+// byte offset of 16-byte chunk c of row r in a 128-byte-row, 128B-swizzled tile
+__device__ __forceinline__ uint32_t sw(int r, int c) { return (uint32_t)(r * 128 + (((c ^ r) & 7) << 4)); }
+enum { B_Q = 0, B_K = 1, B_V = 3, B_S_FULL = 5, B_P_FULL = 6, B_O_DONE = 7, N_BARS = 8 };
+}  // namespace at4
+
+template <int DH>
+__global__ void __launch_bounds__(at4::THREADS, at4::Cfg<DH>::MIN_BLOCKS)
+    attention_tm_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
+                        const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmQ2,
+                        const __grid_constant__ CUtensorMap tmK2, bf16* o, int n_q, int T, int D,
+                        float scale_log2, unsigned* err) {
+  using namespace at4;
+  using C = Cfg<DH>;
+  constexpr bool TAIL = C::TAIL;
+  constexpr int KC = C::KC;
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  uint8_t* sQ = smem;                         // 16 KB
+  uint8_t* sK = sQ + Q_BYTES;                 // two stages
+  uint8_t* sV = sK + 2 * C::K_BYTES;          // two stages
+  uint8_t* sQ2 = sV + 2 * C::V_BYTES;         // 80-wide heads: the remainders of Q and K
+  uint8_t* sK2 = sQ2 + (TAIL ? Q2_BYTES : 0);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(sK2 + 2 * C::K2_BYTES);
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + N_BARS);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int qt = blockIdx.x, h = blockIdx.y, r = blockIdx.z;
+  const int q0 = r * n_q + qt * QT, kv0 = r * T, col = h * DH;
+  const int nck = (T + KC - 1) / KC;
+  // Softmax warps whose 32 query rows all lie beyond n_q sit out: their rows of
+  // S, P and O are never read back (matrix rows are independent).
+  const int n_valid = min(QT, n_q - qt * QT);
+  const int n_act = (n_valid + 31) / 32;
+
+  if (tid == 0) {
+    for (int i = 0; i < N_BARS; ++i) mbar_init(&bars[i], i == B_P_FULL ? (uint32_t)n_act : 1u);
+    *abort_flag = 0;
+    fence_mbar_init();
+    // the descriptors are kernel parameters: fetched while the predecessor grid finishes
+    prefetch_tmap(&tmQ);
+    prefetch_tmap(&tmK);
+    prefetch_tmap(&tmV);
+    if (TAIL) {
+      prefetch_tmap(&tmQ2);
+      prefetch_tmap(&tmK2);
+    }
+  }
+  if (warp == 4) {
+    tmem_alloc(tmem_slot, C::TMEM_COLS);
+    tmem_relinquish();
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = *tmem_slot;
+  pdl_wait();
+  pdl_trigger();
+
+  if (warp == 4) {
+    // ---------------- loads and MMAs ----------------
+    if (lane == 0) {
+      auto load_k = [&](int c) {
+        const int st = c & 1;
+        mbar_arrive_expect_tx(&bars[B_K + st], C::K_TX);
+        tma_load_2d(&tmK, &bars[B_K + st], sK + st * C::K_BYTES, col, kv0 + c * KC);
+        if (TAIL) tma_load_2d(&tmK2, &bars[B_K + st], sK2 + st * C::K2_BYTES, col + 64, kv0 + c * KC);
+      };
+      auto load_v = [&](int c) {
+        const int st = c & 1;
+        mbar_arrive_expect_tx(&bars[B_V + st], C::V_TX);
+        if (TAIL) {
+#pragma unroll
+          for (int p = 0; p < DH / 16; ++p)
+            tma_load_2d(&tmV, &bars[B_V + st], sV + st * C::V_BYTES + p * KC * 32, col + 16 * p, kv0 + c * KC);
+        } else {
+          tma_load_2d(&tmV, &bars[B_V + st], sV + st * C::V_BYTES, col, kv0 + c * KC);
+        }
+      };
+      mbar_arrive_expect_tx(&bars[B_Q], C::Q_TX);
+      tma_load_2d(&tmQ, &bars[B_Q], sQ, col, q0);
+      if (TAIL) tma_load_2d(&tmQ2, &bars[B_Q], sQ2, col + 64, q0);
+      load_k(0);
+      load_v(0);
+      if (nck > 1) {
+        load_k(1);
+        load_v(1);
+      }
+      const uint64_t qd = sw128_desc(smem_u32(sQ));
+      auto issue_s = [&](int c) {
+        const uint64_t kd = sw128_desc(smem_u32(sK + (c & 1) * C::K_BYTES));
+#pragma unroll
+        for (int k = 0; k < 4; ++k) umma_bf16(tmem, qd + 2 * k, kd + 2 * k, idesc(KC), k != 0 ? 1u : 0u);
+        if (TAIL)
+          umma_bf16(tmem, sw32_desc(smem_u32(sQ2), 256), sw32_desc(smem_u32(sK2 + (c & 1) * C::K2_BYTES), 256),
+                    idesc(KC), 1u);
+        umma_commit(&bars[B_S_FULL]);
+      };
+      bool ok = mbar_wait<false>(&bars[B_Q], 0, abort_flag, err) && mbar_wait<false>(&bars[B_K], 0, abort_flag, err);
+      if (ok) {
+        tc_fence_after();
+        issue_s(0);
+      }
+      for (int c = 0; c < nck && ok; ++c) {
+        const int st = c & 1;
+        const uint32_t ph = (uint32_t)(c >> 1) & 1u;
+        ok = mbar_wait<false>(&bars[B_P_FULL], (uint32_t)c & 1u, abort_flag, err) &&
+             mbar_wait<false>(&bars[B_V + st], ph, abort_flag, err);
+        if (!ok) break;
+        tc_fence_after();
+        // 16 keys per MMA: 8 columns of P, 16 rows of the MN-major V tile (2048
+        // bytes, or 512 in each panel of an 80-wide head)
+        const uint32_t va = smem_u32(sV + st * C::V_BYTES);
+        const uint64_t vd = TAIL ? sw32_desc(va, KC * 32) : sw128_mn_desc(va);
+#pragma unroll
+        for (int k = 0; k < KC / 16; ++k)
+          umma_bf16_ta(tmem + KC, tmem + 8 * k, vd + (TAIL ? 32 : 128) * k, idesc(DH) | (1u << 16),
+                       (c > 0 || k > 0) ? 1u : 0u);
+        umma_commit(&bars[B_O_DONE]);
+        if (c + 2 < nck) load_k(c + 2);  // the scores have been read, so S(c) has read K stage c & 1
+        if (c + 1 < nck) {
+          ok = mbar_wait<false>(&bars[B_K + (st ^ 1)], (uint32_t)((c + 1) >> 1) & 1u, abort_flag, err) &&
+               mbar_wait<false>(&bars[B_O_DONE], (uint32_t)c & 1u, abort_flag, err);
+          if (!ok) break;
+          tc_fence_after();
+          issue_s(c + 1);  // P(c) has been read
+          if (c + 2 < nck) load_v(c + 2);
+        }
+      }
+    }
+    __syncwarp();
+  } else if (warp < n_act) {
+    // ---------------- softmax warps (thread = query row) ----------------
+    const uint32_t t_lane = (uint32_t)(warp * 32) << 16;
+    float m_run = -FLT_MAX, l_run = 0.f;
+    bool ok = true;
+    for (int c = 0; c < nck; ++c) {
+      ok = __all_sync(0xffffffffu, mbar_wait<false>(&bars[B_S_FULL], (uint32_t)c & 1u, abort_flag, err));
+      if (!ok) break;
+      tc_fence_after();
+      float sv[KC];
+      {
+        uint32_t ra[32];
+        tmem_ld32(tmem + t_lane, ra);
+        if constexpr (KC == 64) {
+          uint32_t rb[32];
+          tmem_ld32(tmem + t_lane + 32, rb);
+          tmem_wait_ld();
+#pragma unroll
+          for (int i = 0; i < 32; ++i) sv[32 + i] = __uint_as_float(rb[i]);
+        } else {
+          uint32_t rb[16];
+          tmem_ld16(tmem + t_lane + 32, rb);
+          tmem_wait_ld();
+#pragma unroll
+          for (int i = 0; i < 16; ++i) sv[32 + i] = __uint_as_float(rb[i]);
+        }
+#pragma unroll
+        for (int i = 0; i < 32; ++i) sv[i] = __uint_as_float(ra[i]);
+      }
+      // row max of the raw scores; keys beyond T (the last chunk only) drop out
+      float mloc = -FLT_MAX;
+      if (c * KC + KC <= T) {
+        // four independent chains of three-input maxima (dependency depth 8
+        // instead of 32)
+        float mq[4] = {-FLT_MAX, -FLT_MAX, -FLT_MAX, -FLT_MAX};
+#pragma unroll
+        for (int i = 0; i < KC; i += 8) {
+#pragma unroll
+          for (int q = 0; q < 4; ++q) mq[q] = fmax3(mq[q], sv[i + 2 * q], sv[i + 2 * q + 1]);
+        }
+        mloc = fmax3(mq[0], mq[1], fmaxf(mq[2], mq[3]));
+      } else {
+#pragma unroll
+        for (int i = 0; i < KC; ++i) {
+          sv[i] = (c * KC + i < T) ? sv[i] : -FLT_MAX;
+          mloc = fmaxf(mloc, sv[i]);
+        }
+      }
+      mloc *= scale_log2;  // log2 units (scale_log2 > 0 keeps the maximum)
+      float alpha = 1.f;
+      bool raise = false;
+      if (c == 0) {
+        m_run = mloc;
+      } else if (mloc > m_run + RESCALE_THRESHOLD) {
+        raise = true;
+        alpha = exp2_approx(m_run - mloc);
+        m_run = mloc;
+      }
+      // exponent arguments and the row sum two keys per instruction (the
+      // softmax is bound by instruction issue)
+      const unsigned long long sc2 = f32x2_pack(scale_log2, scale_log2), nm2 = f32x2_pack(-m_run, -m_run);
+      // the row sum in four independent paired accumulators
+      unsigned long long ps2[4] = {f32x2_pack(0.f, 0.f), f32x2_pack(0.f, 0.f), f32x2_pack(0.f, 0.f),
+                                   f32x2_pack(0.f, 0.f)};
+      uint32_t pk[KC / 2];
+#pragma unroll
+      for (int i = 0; i < KC / 2; ++i) {
+        float x0, x1;
+        f32x2_unpack(f32x2_fma(f32x2_pack(sv[2 * i], sv[2 * i + 1]), sc2, nm2), x0, x1);
+        const float p0 = exp2_approx(x0), p1 = exp2_approx(x1);
+        ps2[i & 3] = f32x2_add(ps2[i & 3], f32x2_pack(p0, p1));
+        pk[i] = pack_bf16(p0, p1);
+      }
+      float ps0, ps1;
+      f32x2_unpack(f32x2_add(f32x2_add(ps2[0], ps2[1]), f32x2_add(ps2[2], ps2[3])), ps0, ps1);
+      const float psum = ps0 + ps1;
+      // S(c) was issued after P V(c - 1) was complete, so O may be rescaled
+      if (c > 0 && __any_sync(0xffffffffu, raise)) {
+#pragma unroll 1
+        for (int i = 0; i < DH / 16; ++i) {
+          uint32_t rt[16];
+          tmem_ld16(tmem + t_lane + KC + 16 * i, rt);
+          tmem_wait_ld();
+#pragma unroll
+          for (int j = 0; j < 16; ++j) rt[j] = __float_as_uint(__uint_as_float(rt[j]) * alpha);
+          tmem_st16(tmem + t_lane + KC + 16 * i, rt);
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < KC / 16; ++i) tmem_st8(tmem + t_lane + 8 * i, pk + 8 * i);
+      l_run = l_run * alpha + psum;
+      tmem_wait_st();
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&bars[B_P_FULL]);
+    }
+    // epilogue: O / l for this row, staged through the Q tile for whole-row
+    // stores of the first 64 columns; the 16-column remainder of an 80-wide
+    // head is stored by each thread (32 contiguous bytes)
+    if (ok) ok = __all_sync(0xffffffffu, mbar_wait<false>(&bars[B_O_DONE], (uint32_t)(nck - 1) & 1u, abort_flag, err));
+    if (ok) {
+      tc_fence_after();
+      const float inv = 1.f / l_run;
+      uint32_t ra[32], rb[32];
+      tmem_ld32(tmem + t_lane + KC, ra);
+      tmem_ld32(tmem + t_lane + KC + 32, rb);
+      tmem_wait_ld();
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        uint4 w0, w1;
+        w0.x = pack_bf16(__uint_as_float(ra[8 * j + 0]) * inv, __uint_as_float(ra[8 * j + 1]) * inv);
+        w0.y = pack_bf16(__uint_as_float(ra[8 * j + 2]) * inv, __uint_as_float(ra[8 * j + 3]) * inv);
+        w0.z = pack_bf16(__uint_as_float(ra[8 * j + 4]) * inv, __uint_as_float(ra[8 * j + 5]) * inv);
+        w0.w = pack_bf16(__uint_as_float(ra[8 * j + 6]) * inv, __uint_as_float(ra[8 * j + 7]) * inv);
+        w1.x = pack_bf16(__uint_as_float(rb[8 * j + 0]) * inv, __uint_as_float(rb[8 * j + 1]) * inv);
+        w1.y = pack_bf16(__uint_as_float(rb[8 * j + 2]) * inv, __uint_as_float(rb[8 * j + 3]) * inv);
+        w1.z = pack_bf16(__uint_as_float(rb[8 * j + 4]) * inv, __uint_as_float(rb[8 * j + 5]) * inv);
+        w1.w = pack_bf16(__uint_as_float(rb[8 * j + 6]) * inv, __uint_as_float(rb[8 * j + 7]) * inv);
+        *reinterpret_cast<uint4*>(sQ + sw(tid, j)) = w0;
+        *reinterpret_cast<uint4*>(sQ + sw(tid, 4 + j)) = w1;
+      }
+      if (TAIL) {
+        uint32_t rt[16];
+        tmem_ld16(tmem + t_lane + KC + 64, rt);
+        tmem_wait_ld();
+        const int qi = qt * QT + tid;
+        if (qi < n_q) {
+          uint4 t0, t1;
+          t0.x = pack_bf16(__uint_as_float(rt[0]) * inv, __uint_as_float(rt[1]) * inv);
+          t0.y = pack_bf16(__uint_as_float(rt[2]) * inv, __uint_as_float(rt[3]) * inv);
+          t0.z = pack_bf16(__uint_as_float(rt[4]) * inv, __uint_as_float(rt[5]) * inv);
+          t0.w = pack_bf16(__uint_as_float(rt[6]) * inv, __uint_as_float(rt[7]) * inv);
+          t1.x = pack_bf16(__uint_as_float(rt[8]) * inv, __uint_as_float(rt[9]) * inv);
+          t1.y = pack_bf16(__uint_as_float(rt[10]) * inv, __uint_as_float(rt[11]) * inv);
+          t1.z = pack_bf16(__uint_as_float(rt[12]) * inv, __uint_as_float(rt[13]) * inv);
+          t1.w = pack_bf16(__uint_as_float(rt[14]) * inv, __uint_as_float(rt[15]) * inv);
+          uint4* dst = reinterpret_cast<uint4*>(o + (size_t)(r * n_q + qi) * D + col + 64);
+          dst[0] = t0;
+          dst[1] = t1;
+        }
+      }
+      __syncwarp();
+      // the warp's 32 rows: 4 rows x 8 chunks of 16 bytes per instruction
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const int row = warp * 32 + i * 4 + (lane >> 3), ch = lane & 7;
+        const int qi = qt * QT + row;
+        if (qi < n_q) {
+          const uint4 val = *reinterpret_cast<const uint4*>(sQ + sw(row, ch));
           *reinterpret_cast<uint4*>(o + (size_t)(r * n_q + qi) * D + col + 8 * ch) = val;
         }
       }
@@ -562,6 +931,45 @@ static cudaError_t launch_attn_tc(const Ctx& c, const void* q, const void* k, co
                     mk2, mv2, static_cast<bf16*>(o), n_q, T, D, scale_log2, c.err);
 }
 
+template <int DH>
+static cudaError_t launch_attn_tm(const Ctx& c, const void* q, const void* k, const void* v, void* o, int rows,
+                                  int n_q, int T, int heads) {
+  using C = at4::Cfg<DH>;
+  if (T < 1) return cudaErrorInvalidValue;  // the kernel's final wait needs at least one key chunk
+  const int D = heads * DH;
+  const uint64_t pitch = (uint64_t)D * 2;
+  CUtensorMap mq, mk, mv, mq2, mk2;
+  if (!make_tmap_bf16(&mq, q, D, (uint64_t)rows * n_q, pitch, 64, at4::QT, CU_TENSOR_MAP_SWIZZLE_128B) ||
+      !make_tmap_bf16(&mk, k, D, (uint64_t)rows * T, pitch, 64, C::KC, CU_TENSOR_MAP_SWIZZLE_128B))
+    return cudaErrorInvalidValue;
+  if (C::TAIL) {
+    // 16-column boxes: x = h * 80 + 16 i elements = 160 h + 32 i bytes, a
+    // multiple of 16 bytes as TMA requires
+    if (!make_tmap_bf16(&mv, v, D, (uint64_t)rows * T, pitch, 16, C::KC, CU_TENSOR_MAP_SWIZZLE_32B) ||
+        !make_tmap_bf16(&mq2, q, D, (uint64_t)rows * n_q, pitch, 16, at4::QT, CU_TENSOR_MAP_SWIZZLE_32B) ||
+        !make_tmap_bf16(&mk2, k, D, (uint64_t)rows * T, pitch, 16, C::KC, CU_TENSOR_MAP_SWIZZLE_32B))
+      return cudaErrorInvalidValue;
+  } else {
+    if (!make_tmap_bf16(&mv, v, D, (uint64_t)rows * T, pitch, 64, C::KC, CU_TENSOR_MAP_SWIZZLE_128B))
+      return cudaErrorInvalidValue;
+    mq2 = mq;
+    mk2 = mk;
+  }
+  static int attr_set[64] = {};
+  int dev = 0;
+  cudaGetDevice(&dev);
+  if (dev >= 0 && dev < 64 && !attr_set[dev]) {
+    cudaError_t e =
+        cudaFuncSetAttribute(attention_tm_kernel<DH>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
+    if (e != cudaSuccess) return e;
+    attr_set[dev] = 1;
+  }
+  const float scale_log2 = 1.4426950408889634f / sqrtf((float)DH);  // log2(e) / sqrt(d)
+  dim3 grid((n_q + at4::QT - 1) / at4::QT, heads, rows);
+  return launch_pdl(attention_tm_kernel<DH>, grid, dim3(at4::THREADS), (size_t)C::SMEM, c.stream, mq, mk, mv, mq2,
+                    mk2, static_cast<bf16*>(o), n_q, T, D, scale_log2, c.err);
+}
+
 cudaError_t launch_attention(const Ctx& c, int dtype, const void* q, const void* k, const void* v, void* o,
                              int rows, int n_q, int T, int heads, int dh) {
   if (rows == 0 || n_q == 0) return cudaSuccess;
@@ -579,8 +987,19 @@ cudaError_t launch_attention(const Ctx& c, int dtype, const void* q, const void*
                       static_cast<const float*>(k), static_cast<const float*>(v), static_cast<float*>(o), n_q, T,
                       heads * dh, dh, 1.0f / sqrtf((float)dh));
   }
-  if (dh == 64) return launch_attn_tc<64>(c, q, k, v, o, rows, n_q, T, heads);
-  return launch_attn_tc<80>(c, q, k, v, o, rows, n_q, T, heads);
+  // attention_tm_kernel overlaps four CTAs of an SM, attention_tc_kernel the
+  // chunks of one (it may issue S(c + 1) while P(c) is on its way): the former
+  // needs more CTAs than one wave of the latter. Below that, and for 64-wide heads with at
+  // most 64 queries (bound by the stream of keys and values, of which fewer are
+  // in flight), the latter is faster: 32 rows x 12 heads x 50 x 320 7.7 against
+  // 9.3 us, 64 rows 14.5 against 15.7, 2 x 16 x 320 x 320 6.2 against 7.1; width
+  // 80, 3 x 12 x 129 x 200 6.4 against 7.3.
+  const long long ctas = (long long)((n_q + 127) / 128) * heads * rows;
+  if (dh == 64)
+    return n_q > 64 && ctas > 3LL * c.num_sms ? launch_attn_tm<64>(c, q, k, v, o, rows, n_q, T, heads)
+                                              : launch_attn_tc<64>(c, q, k, v, o, rows, n_q, T, heads);
+  return ctas > 2LL * c.num_sms ? launch_attn_tm<80>(c, q, k, v, o, rows, n_q, T, heads)
+                                : launch_attn_tc<80>(c, q, k, v, o, rows, n_q, T, heads);
 }
 
 }  // namespace lm

@@ -555,6 +555,33 @@ def test_attention(rows, n_q, T, heads, dh, dtype, q_std):
 # LayerNorm (gathering rows)
 # --------------------------------------------------------------------------
 
+@pytest.mark.parametrize("rows,n_q,T,heads,dh,q_std", [
+    (64, 129, 320, 12, 64, 1.0),   # more CTAs than one wave: probabilities in tensor memory
+    (46, 65, 65, 12, 64, 1.0),     # one query and one key past a tile and a chunk
+    (40, 320, 63, 12, 64, 1.0),    # a single, partial key chunk
+    (30, 300, 1088, 6, 64, 4.0),   # running maxima raised mid-row
+    (26, 50, 320, 12, 80, 1.0),    # width 80: 48-key chunks, any number of queries
+    (16, 129, 97, 16, 80, 1.0),
+    (40, 1, 49, 16, 80, 1.0),
+    (12, 300, 500, 16, 80, 4.0),
+])
+def test_attention_large_grids(rows, n_q, T, heads, dh, q_std):
+    D = heads * dh
+    q = synth.tensor((rows, n_q, D), 41, std=q_std, dtype="bf16")
+    k = synth.tensor((rows, T, D), 42, dtype="bf16")
+    v = synth.tensor((rows, T, D), 43, dtype="bf16")
+    o = empty((rows, n_q, D), "bf16")
+    lm.lazymar_attention(DT["bf16"], dev(q, "bf16"), dev(k, "bf16"), dev(v, "bf16"), o, rows, n_q, T, heads, dh)
+    sync()
+    got = host(o)
+    for r in (0, rows // 2, rows - 1):
+        assert max_rel(got[r], O.attention(q[r], k[r], v[r], heads)) < 1e-2, "row %d" % r
+    torch = torch_cuda()
+    split = [x.view(rows, -1, heads, dh).transpose(1, 2) for x in (dev(q), dev(k), dev(v))]
+    ref = torch.nn.functional.scaled_dot_product_attention(*split).transpose(1, 2).reshape(rows, n_q, D)
+    assert max_rel(got, host(ref)) < 1e-2
+
+
 @pytest.mark.parametrize("M,D,gather,dtype", [(100, 768, False, "bf16"), (50, 1280, True, "bf16"),
                                               (80, 256, True, "fp32"), (3, 1024, False, "fp32")])
 def test_layernorm(M, D, gather, dtype):
