@@ -336,12 +336,12 @@ __global__ void __launch_bounds__(tc::Cfg<BN, EK, BK, F8, PAIR, ROWS>::THREADS, 
     __syncwarp();
   } else if (warp == 1) {
     // ---------------- MMA issuer (of a pair: the even CTA's) ----------------
-    // For the narrow tiles and the bf16-output pairs the warp runs converged and
+    // For the small tiles and the bf16-output pairs the warp runs converged and
     // one elected lane issues (few-row fc2, a stage of eight 128 x 64 x 16 MMAs:
     // 0.322 us against 0.347 with a single lane in the loop, 0.252 of it the
     // MMAs; full-layer Q/K/V 47.7 -> 45.0 us, fc1 65.2 -> 65.6); the other kinds
     // are up to 2 % faster with the single lane.
-    constexpr bool CONVERGED = BN == 64 || (PAIR && tc::is_bf16out<EK>());
+    constexpr bool CONVERGED = BN == 64 || ROWS == 64 || (PAIR && tc::is_bf16out<EK>());
     if (rank == 0 && (CONVERGED || lane == 0)) {
       const bool lead = CONVERGED ? elect_one() : true;
       auto wait = [&](uint64_t* bar, uint32_t parity) {
@@ -1057,7 +1057,13 @@ static int choose_bn(const Ctx& c, int dtype, int M, int N, const GemmEpi& epi, 
   // 64 x 64 (us): M = 50, width 768: out 4.5 -> 3.9, fc2 10.6 -> 8.8; M = 320 fc2
   // 11.3 -> 9.0; M = 200, width 1024: out 5.2 -> 4.5, fc2 13.9 -> 11.2; the diffusion
   // head's sampling of 128 tokens 9.74 -> 8.64 ms
-  if (dtype == LAZYMAR_BF16 && K % 128 == 0 && (long)((M + 63) / 64) * (N / 64) <= c.num_sms) bn = kRows64 + 64;
+  if (dtype == LAZYMAR_BF16 && K % 128 == 0 && (long)((M + 63) / 64) * (N / 64) <= c.num_sms)
+    bn = kRows64 + 64;
+  // Residual kinds whose 128 x 128 tiles occupy at most half of the SMs: 64 x
+  // 128 tiles (M = 1600, width 768: out 6.6 -> 5.6 us, fc2 13.3 -> 12.4)
+  else if (bn == 128 && dtype == LAZYMAR_BF16 && resid && !epi.gate && K % 128 == 0 &&
+           (long)((M + 63) / 64) * (N / 128) <= c.num_sms)
+    bn = kRows64 + 128;
   *cost = best;
   return bn;
 }
@@ -1109,6 +1115,10 @@ static cudaError_t launch_bn_impl(const Ctx& c, int dtype, const void* A, const 
                  : epi.gate                          ? tc::RESID_WIDE_GATED
                  : K < 2048                          ? tc::RESID_WIDE
                                                      : tc::RESID_HALF;
+  if (bn == kRows64 + 128) {
+    if (ek == tc::RESID_WIDE) return launch_tc<128, tc::RESID_WIDE, 128, 0, 0, 64>(c, A, W, M, N, K, epi);
+    return launch_tc<128, tc::RESID_HALF, 128, 0, 0, 64>(c, A, W, M, N, K, epi);
+  }
   if (bn == kRows64 + 64) {
     if (ek == tc::RESID_WIDE) return launch_tc<64, tc::RESID_WIDE, 128, 0, 0, 64>(c, A, W, M, N, K, epi);
     if (ek == tc::RESID_WIDE_GATED) return launch_tc<64, tc::RESID_WIDE_GATED, 128, 0, 0, 64>(c, A, W, M, N, K, epi);

@@ -349,12 +349,12 @@ def test_linear_pairs_equal_single_ctas(M, N, K, epi):
 
 
 @pytest.mark.parametrize("M,N,K", [(1, 384, 128), (63, 768, 256), (65, 768, 3072), (200, 2304, 768), (449, 1024, 1024),
-                                   (320, 1536, 640)])
+                                   (320, 1536, 640), (1537, 768, 768), (1600, 768, 3072)])
 @pytest.mark.parametrize("epi", [lm.LAZYMAR_EPI_BIAS, lm.LAZYMAR_EPI_GELU, lm.LAZYMAR_EPI_RESIDUAL,
                                  lm.LAZYMAR_EPI_QKV, lm.LAZYMAR_EPI_SILU])
 def test_linear_few_rows_equal_128_row_tiles(M, N, K, epi):
-    """Few rows take 64-row tiles (K % 128 == 0, one round of 64 x 64 tiles):
-    bit for bit the 128-row tiles' results, rows past M untouched."""
+    """Few rows take 64-row tiles (K % 128 == 0, one round of 64 x 64 tiles, or of
+    64 x 128 ones in the residual kinds): bit for bit the 128-row tiles' results, rows past M untouched."""
     torch = torch_cuda()
     g = torch.Generator(device="cuda")
     g.manual_seed(M + N + K + epi)
