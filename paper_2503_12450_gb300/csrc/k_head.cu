@@ -20,6 +20,8 @@
 // The guidance scale and temperature are read from device memory, so they may
 // change between calls. The time embeddings of the kept steps depend on the
 // weights only and are computed once at create.
+#include <cuda.h>
+
 #include <cmath>
 #include <cstring>
 #include <map>
@@ -30,6 +32,10 @@
 #include "lazymar_internal.cuh"
 
 namespace lm {
+
+bool make_tmap_bf16(CUtensorMap* m, const void* base, uint64_t inner, uint64_t outer, uint64_t pitch_bytes,
+                    uint32_t box_inner, uint32_t box_outer, CUtensorMapSwizzle swz);
+
 namespace hd {
 
 // Four packed bf16 values as floats.
@@ -190,6 +196,262 @@ __global__ void __launch_bounds__(256) ln_mod_kernel(float* __restrict__ xh, con
   constexpr int w = 128 * VPL;
   ln_mod_row<VPL, INPROJ>(xh + (size_t)r * w, x + (size_t)(r < M ? r : r - M) * td, win_t, bin,
                           mod + (size_t)r * ldm, shift_off, scale_off, hb + (size_t)r * w, td, eps, lane);
+}
+
+// ---------------------------------------------------------------------------
+// fc2, gated residual and the next block's modulated LayerNorm in one kernel
+// ---------------------------------------------------------------------------
+// xh += gate * (u W2^T + b2); hb = LN(xh) (1 + scale) + shift, for the 64 rows
+// of one cluster, whose w / 64 CTAs hold 64 columns each. A CTA's main loop is
+// that of a 64-row GEMM tile (k_gemm.cu); its epilogue keeps the new residual
+// rows in shared memory, sends each row's mean and sum of squared deviations
+// over its 64 columns to every CTA of the cluster, and after one cluster
+// barrier combines them (Chan's pairwise update over equal counts) and writes
+// its columns of the normalised rows. The kernel chain of a denoising step is
+// bound by latency, launch by launch; this removes the separate LayerNorm
+// launch of every block but the first. Width 1024, 6 blocks, 100 steps, against
+// separate launches: 32 tokens 8.04 -> 7.54 ms, 128 8.72 -> 8.31, 224 9.70 -> 9.28.
+// Wider rows would need more CTAs than a cluster has, or 128 columns per CTA,
+// which brought nothing (width 1280 12.04 -> 12.05 ms, 1536 20.9 -> 21.7): they
+// keep the separate launches.
+struct FusedCfg {
+  static constexpr int ROWS = 64, BN = 64, BK = 128, ATOMS = 2;
+  static constexpr uint32_t A_BYTES = ROWS * BK * 2, B_BYTES = BN * BK * 2, STAGE_BYTES = A_BYTES + B_BYTES;
+  static constexpr int STAGES = 6;
+  static constexpr int HP = BN + 4;  // floats per residual row in shared memory
+  static constexpr int MAXC = 16;    // CTAs of a cluster
+  static constexpr int EPI_WARPS = 8, THREADS = 64 + EPI_WARPS * 32;
+  static constexpr int CHUNKS = BN / 64;  // 32-column chunks per epilogue warp
+  static constexpr size_t SMEM = 1024 + (size_t)STAGES * STAGE_BYTES + ROWS * HP * 4 + MAXC * ROWS * 8 + ROWS * 8 + 256;
+  static_assert(SMEM <= 232448, "shared memory of one CTA");
+  static constexpr uint32_t IDESC = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) |
+                                    ((uint32_t)(ROWS >> 4) << 24);
+};
+
+__global__ void __launch_bounds__(FusedCfg::THREADS, 1)
+    fc2_ln_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
+                  const bf16* __restrict__ bias, const bf16* __restrict__ mod, int ldm, int gate_off, int shift_off,
+                  int scale_off, float* xh, bf16* __restrict__ hb, int R, int w, float eps, unsigned* err) {
+  using C = FusedCfg;
+  constexpr int BN = C::BN;
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  uint8_t* sA = smem;
+  uint8_t* sB = smem + C::STAGES * C::A_BYTES;
+  float* sH = reinterpret_cast<float*>(smem + C::STAGES * C::STAGE_BYTES);  // [64][HP]
+  float2* sStat = reinterpret_cast<float2*>(sH + C::ROWS * C::HP);          // [CTA][row]: mean, squared deviations
+  float2* sNorm = sStat + C::MAXC * C::ROWS;                                // [row]: mean, 1 / deviation
+  uint64_t* full = reinterpret_cast<uint64_t*>(sNorm + C::ROWS);
+  uint64_t* empty = full + C::STAGES;
+  uint64_t* acc_full = empty + C::STAGES;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_full + 1);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint32_t rank = cluster_ctarank(), ncta = cluster_nctarank();
+  const int m0 = (int)(blockIdx.x / ncta) * C::ROWS, n0 = (int)rank * BN;
+  const int KB = w / C::BK;
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < C::STAGES; ++s) {
+      mbar_init(&full[s], 1);
+      mbar_init(&empty[s], 1);
+    }
+    mbar_init(acc_full, 1);
+    *abort_flag = 0;
+    fence_mbar_init();
+    prefetch_tmap(&tmA);
+    prefetch_tmap(&tmB);
+  }
+  if (warp == 1) {
+    tmem_alloc(tmem_slot, BN);
+    tmem_relinquish();
+  }
+  tc_fence_before();
+  __syncthreads();
+  cluster_sync();  // every CTA of the cluster runs before its shared memory is written to
+  tc_fence_after();
+  const uint32_t tmem = *tmem_slot;
+  auto load = [&](const CUtensorMap* tm, uint8_t* dst, uint32_t bytes, int s, int kb, int r0) {
+#pragma unroll
+    for (int a = 0; a < C::ATOMS; ++a)
+      tma_load_2d(tm, &full[s], dst + s * bytes + a * (bytes / C::ATOMS), kb * C::BK + a * 64, r0);
+  };
+  const int pre = KB < C::STAGES ? KB : C::STAGES;
+  if (warp == 0 && lane == 0)
+    for (int s = 0; s < pre; ++s) {  // weights: no kernel writes them
+      mbar_arrive_expect_tx(&full[s], C::STAGE_BYTES);
+      load(&tmB, sB, C::B_BYTES, s, s, n0);
+    }
+  pdl_wait();
+  pdl_trigger();
+  bool ok = true;
+  if (warp == 0) {
+    if (lane == 0) {
+      int stage = 0;
+      uint32_t phase = 0;
+      for (int kb = 0; kb < KB; ++kb) {
+        if (kb < pre) {
+          load(&tmA, sA, C::A_BYTES, stage, kb, m0);
+        } else {
+          if (!mbar_wait(&empty[stage], phase ^ 1u, abort_flag, err)) break;
+          mbar_arrive_expect_tx(&full[stage], C::STAGE_BYTES);
+          load(&tmA, sA, C::A_BYTES, stage, kb, m0);
+          load(&tmB, sB, C::B_BYTES, stage, kb, n0);
+        }
+        if (++stage == C::STAGES) { stage = 0; phase ^= 1u; }
+      }
+    }
+    __syncwarp();
+  } else if (warp == 1) {
+    const bool lead = elect_one();
+    int stage = 0;
+    uint32_t phase = 0;
+    for (int kb = 0; kb < KB; ++kb) {
+      ok = __all_sync(0xffffffffu, mbar_wait(&full[stage], phase, abort_flag, err));
+      if (!ok) break;
+      tc_fence_after();
+      if (lead) {
+        // K-major 128-byte-swizzled tiles: 8-row groups 1024 bytes apart
+        constexpr uint64_t kDesc = ((uint64_t)1 << 16) | ((uint64_t)(1024 >> 4) << 32) | ((uint64_t)1 << 46) | ((uint64_t)2 << 61);
+        const uint64_t a0 = kDesc | ((smem_u32(sA + stage * C::A_BYTES) >> 4) & 0x3FFFu);
+        const uint64_t b0 = kDesc | ((smem_u32(sB + stage * C::B_BYTES) >> 4) & 0x3FFFu);
+#pragma unroll
+        for (int k = 0; k < C::ATOMS * 4; ++k)
+          umma_bf16(tmem, a0 + ((uint64_t)(k / 4 * (C::A_BYTES / C::ATOMS)) >> 4) + 2 * (k % 4),
+                    b0 + ((uint64_t)(k / 4 * (C::B_BYTES / C::ATOMS)) >> 4) + 2 * (k % 4), C::IDESC,
+                    (kb | k) != 0 ? 1u : 0u);
+        umma_commit(&empty[stage]);
+      }
+      __syncwarp();
+      if (++stage == C::STAGES) { stage = 0; phase ^= 1u; }
+    }
+    if (ok && lead) umma_commit(acc_full);
+    __syncwarp();
+  } else {
+    const int quarter = warp & 3, half = (warp - 2) >> 2;
+    const int wr = lane >> 3, wq = lane & 7;  // row within a pass of 4, 16-byte block of a 32-column chunk
+    // what the epilogue reads, ahead of the accumulator: row lr = 16 quarter +
+    // 4 p + wr, columns c0 + 4 wq ..
+    float4 x[C::CHUNKS][4];
+    uint2 gt[C::CHUNKS][4], sh[C::CHUNKS][4], sc[C::CHUNKS][4], bi[C::CHUNKS];
+#pragma unroll
+    for (int j = 0; j < C::CHUNKS; ++j) {
+      const int col = n0 + (half * C::CHUNKS + j) * 32 + 4 * wq;
+      bi[j] = *reinterpret_cast<const uint2*>(bias + col);
+#pragma unroll
+      for (int p = 0; p < 4; ++p) {
+        const int row = m0 + quarter * 16 + p * 4 + wr;
+        x[j][p] = make_float4(0.f, 0.f, 0.f, 0.f);
+        gt[j][p] = sh[j][p] = sc[j][p] = make_uint2(0u, 0u);
+        if (row < R) {
+          const bf16* mr = mod + (size_t)row * ldm + col;
+          x[j][p] = *reinterpret_cast<const float4*>(xh + (size_t)row * w + col);
+          gt[j][p] = *reinterpret_cast<const uint2*>(mr + gate_off);
+          sh[j][p] = *reinterpret_cast<const uint2*>(mr + shift_off);
+          sc[j][p] = *reinterpret_cast<const uint2*>(mr + scale_off);
+        }
+      }
+    }
+    ok = __all_sync(0xffffffffu, mbar_wait(acc_full, 0, abort_flag, err));
+    tc_fence_after();
+#pragma unroll
+    for (int j = 0; j < C::CHUNKS; ++j) {
+      const int ch = half * C::CHUNKS + j;
+      uint32_t r[32];
+      tmem_ld32(tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(ch * 32), r);
+      tmem_wait_ld();
+      if (lane < 16) {  // at M = 64 a lane quarter holds 16 rows
+        float4* srow = reinterpret_cast<float4*>(sH + (quarter * 16 + lane) * C::HP + ch * 32);
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+          srow[i] = make_float4(__uint_as_float(r[4 * i]), __uint_as_float(r[4 * i + 1]), __uint_as_float(r[4 * i + 2]),
+                                __uint_as_float(r[4 * i + 3]));
+      }
+      __syncwarp();
+      float b[4];
+      unpack4_bf16(bi[j], b);
+#pragma unroll
+      for (int p = 0; p < 4; ++p) {
+        const int lr = quarter * 16 + p * 4 + wr, row = m0 + lr;
+        float4* hp = reinterpret_cast<float4*>(sH + lr * C::HP + ch * 32 + 4 * wq);
+        const float4 a = *hp;
+        float g[4];
+        unpack4_bf16(gt[j][p], g);
+        float4 h;
+        h.x = fmaf(g[0], a.x + b[0], x[j][p].x);
+        h.y = fmaf(g[1], a.y + b[1], x[j][p].y);
+        h.z = fmaf(g[2], a.z + b[2], x[j][p].z);
+        h.w = fmaf(g[3], a.w + b[3], x[j][p].w);
+        x[j][p] = h;
+        *hp = h;
+        if (row < R && ok) *reinterpret_cast<float4*>(xh + (size_t)row * w + n0 + ch * 32 + 4 * wq) = h;
+      }
+    }
+    tc_fence_before();
+    asm volatile("bar.sync 1, %0;" ::"n"(C::EPI_WARPS * 32) : "memory");  // the epilogue warps
+    // statistics of this CTA's columns, four lanes per row
+    const int t = (int)threadIdx.x - 64, lr = t >> 2, q = t & 3;
+    const float* hr = sH + lr * C::HP + q * (BN / 4);
+    float sum = 0.f;
+#pragma unroll
+    for (int i = 0; i < BN / 4; i += 4) {
+      const float4 h = *reinterpret_cast<const float4*>(hr + i);
+      sum += (h.x + h.y) + (h.z + h.w);
+    }
+    sum += __shfl_xor_sync(0xffffffffu, sum, 1);
+    sum += __shfl_xor_sync(0xffffffffu, sum, 2);
+    const float mean = sum * (1.f / BN);
+    float dev = 0.f;
+#pragma unroll
+    for (int i = 0; i < BN / 4; i += 4) {
+      const float4 h = *reinterpret_cast<const float4*>(hr + i);
+      const float a = h.x - mean, b = h.y - mean, c = h.z - mean, d = h.w - mean;
+      dev += (a * a + b * b) + (c * c + d * d);
+    }
+    dev += __shfl_xor_sync(0xffffffffu, dev, 1);
+    dev += __shfl_xor_sync(0xffffffffu, dev, 2);
+    const uint32_t at = smem_u32(sStat + rank * C::ROWS + lr);
+    for (uint32_t p = (uint32_t)q; p < ncta; p += 4)
+      asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(cluster_map(at, p)), "f"(mean), "f"(dev) : "memory");
+    __syncwarp();
+    cluster_sync();  // the whole rows' statistics are here
+    if (t < C::ROWS) {
+      float mu = 0.f;
+      for (uint32_t p = 0; p < ncta; ++p) mu += sStat[p * C::ROWS + t].x;
+      mu /= (float)ncta;
+      float m2 = 0.f;
+      for (uint32_t p = 0; p < ncta; ++p) {
+        const float2 v = sStat[p * C::ROWS + t];
+        const float d = v.x - mu;
+        m2 += fmaf((float)BN * d, d, v.y);
+      }
+      sNorm[t] = make_float2(mu, rsqrtf(m2 / (float)w + eps));
+    }
+    asm volatile("bar.sync 1, %0;" ::"n"(C::EPI_WARPS * 32) : "memory");
+#pragma unroll
+    for (int p = 0; p < 4; ++p) {
+      const int lr2 = quarter * 16 + p * 4 + wr, row = m0 + lr2;
+      const float2 nm = sNorm[lr2];
+      if (row < R && ok) {
+#pragma unroll
+        for (int j = 0; j < C::CHUNKS; ++j) {
+          float a[4], c[4];
+          unpack4_bf16(sh[j][p], a);
+          unpack4_bf16(sc[j][p], c);
+          const float4 h = x[j][p];
+          uint2 o;
+          o.x = pack_bf16(fmaf((h.x - nm.x) * nm.y, 1.f + c[0], a[0]), fmaf((h.y - nm.x) * nm.y, 1.f + c[1], a[1]));
+          o.y = pack_bf16(fmaf((h.z - nm.x) * nm.y, 1.f + c[2], a[2]), fmaf((h.w - nm.x) * nm.y, 1.f + c[3], a[3]));
+          *reinterpret_cast<uint2*>(hb + (size_t)row * w + n0 + (half * C::CHUNKS + j) * 32 + 4 * wq) = o;
+        }
+      }
+    }
+  }
+  if (warp < 2) cluster_sync();  // the epilogue warps' barrier is the cluster's
+  __syncthreads();
+  if (warp == 1) {
+    tc_fence_after();
+    tmem_dealloc(tmem, BN);
+  }
 }
 
 // Schedule constants of one kept step: mean = a_x x - a_eps eps; the log
@@ -390,6 +652,7 @@ bool width_ok(int w) {
 struct lazymar_head {
   lazymar_head_config cfg{};
   int dev = 0, num_sms = 0, w = 0, td = 0, nmod = 0;
+  bool fused = false;  // fc2_ln_kernel serves this width
   int chunk = 1;  // kept steps whose modulations are computed by one GEMM
   uint8_t* arena = nullptr;
   // weights (bf16 unless noted)
@@ -497,6 +760,53 @@ cudaError_t launch_final(const Ctx& c, lazymar_head* h, size_t smem, const bf16*
   }
 }
 
+// Rows up to which fc2_ln_kernel is used: one wave of 16-CTA clusters.
+constexpr int kFuseRows = 512;
+
+// fc2_ln_kernel for block b's W2 and the modulations of block b + 1.
+cudaError_t launch_fc2_ln(const Ctx& c, lazymar_head* h, int b, const bf16* mod, int R) {
+  using C = hd::FusedCfg;
+  constexpr int BN = C::BN;
+  const int w = h->w;
+  CUtensorMap ta, tb;
+  if (!make_tmap_bf16(&ta, h->u, (uint64_t)w, (uint64_t)R, (uint64_t)w * 2, 64, C::ROWS, CU_TENSOR_MAP_SWIZZLE_128B) ||
+      !make_tmap_bf16(&tb, h->w2[b], (uint64_t)w, (uint64_t)w, (uint64_t)w * 2, 64, BN, CU_TENSOR_MAP_SWIZZLE_128B))
+    return cudaErrorInvalidValue;
+  return launch_pdl_cluster(hd::fc2_ln_kernel, dim3((unsigned)((R + 63) / 64 * (w / BN))), dim3(C::THREADS), C::SMEM,
+                            w / BN, c.stream, ta, tb, (const bf16*)h->b2[b], mod, h->nmod, 3 * w * b + 2 * w,
+                            3 * w * (b + 1), 3 * w * (b + 1) + w, h->xh, h->hb, R, w, h->cfg.ln_eps, h->err);
+}
+
+// Whether fc2_ln_kernel serves width w on the current device (a cluster of w /
+// 64 CTAs fits); sets its launch attributes.
+bool fc2_ln_fits(int w) {
+  using C = hd::FusedCfg;
+  constexpr int BN = C::BN;
+  auto kernel = hd::fc2_ln_kernel;
+  if (w % BN != 0 || w / BN > C::MAXC) return false;
+  if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM) != cudaSuccess ||
+      cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(w / BN));
+  cfg.blockDim = dim3(C::THREADS);
+  cfg.dynamicSmemBytes = C::SMEM;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = (unsigned)(w / BN);
+  attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  int n = 0;
+  if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return n >= 1;
+}
+
 // Gathers the z rows and embeds them (W_c z + b_c), once per call.
 lazymar_status prologue(lazymar_head* h, const Ctx& c, const void* z, int B, int n_img, int n_new, int M) {
   const int R = 2 * M, cd = h->cfg.cond_dim;
@@ -538,13 +848,21 @@ lazymar_status modulations(lazymar_head* h, const Ctx& c, int M, int j0, int cnt
 lazymar_status network(lazymar_head* h, const Ctx& c, int M, int j, const bf16* mod, bool done, float* eval_out,
                        bool first_done = false, const bf16* next_mod = nullptr) {
   const int R = 2 * M, w = h->w, depth = h->cfg.depth, td = h->td;
+  const bool fuse = h->fused && R <= kFuseRows;
   for (int b = 0; b < depth; ++b) {
-    if (b > 0 || !first_done)
+    const bool normed = b > 0 ? fuse : first_done;  // hb already holds this block's input
+    if (!normed)
       HD_TRY(hlaunch(h, b == 0 ? 2.0 * R * td * w : 0.0, "head layernorm", [&] {
         return launch_ln_mod(c, h, mod, b == 0, R, M, 3 * w * b, 3 * w * b + w);
       }));
     HD_TRY(hgemm(h, c, h->hb, h->w1[b], R, w, w,
                  GemmEpi{LAZYMAR_EPI_SILU, h->b1[b], h->u, w, nullptr, nullptr, nullptr, 0}));
+    if (fuse && b + 1 < depth) {
+      HD_TRY(hlaunch(h, 2.0 * R * w * w, "head fc2 + layernorm", [&] {
+        return launch_fc2_ln(c, h, b, mod, R);
+      }));
+      continue;
+    }
     GemmEpi e2{LAZYMAR_EPI_RESIDUAL, h->b2[b], h->xh, w, nullptr, nullptr, nullptr, 0};
     e2.gate = mod + 3 * w * b + 2 * w;
     e2.ldg = h->nmod;
@@ -704,6 +1022,7 @@ extern "C" lazymar_status lazymar_head_create(const lazymar_head_config* cfg, co
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&h->num_sms, cudaDevAttrMultiProcessorCount, h->dev);
   if (e != cudaSuccess) return destroy(head_cuda(e, "device query"));
 
+  h->fused = fc2_ln_fits(c.width);
   const size_t W = c.width, F = c.freq_dim, CD = c.cond_dim, TD = c.token_dim, NM = h->nmod, NS = c.n_steps;
   const size_t R = 2 * (size_t)c.max_tokens, MT = c.max_tokens;
   // modulations of up to `chunk` kept steps at once, within 1 GB and with
