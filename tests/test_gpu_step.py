@@ -115,6 +115,29 @@ def test_tiny_full_then_cached_step(tiny):
         assert np.array_equal(z1g[row, keep], z0g[row, keep])
 
 
+@pytest.mark.parametrize("batch,dtype,over", [
+    (35, "fp32", {}),                        # runs of 4 (pair, token) items per CTA, the last one shorter
+    (12, "fp32", {"n_img": 61}),             # odd runs: an item without a partner
+    (3, "bf16", {"width": 256, "heads": 4}),
+    (2, "fp32", {"token_dim": 12}),          # other latent widths: the general kernel
+])
+def test_embedding_of_many_pairs(batch, dtype, over):
+    """Embedding of both pathways (full step) and of the conditional one
+    (condition-reuse step) through a one-block model: every pair's features
+    against the oracle, class and masked and decoded tokens alike."""
+    r = Run("tiny", batch=batch, depth=1, dtype=dtype, **over)
+    cfg = r.cfg
+    N = cfg["T"]
+    c = O.Cache(cfg, batch)
+    st0, st1 = r.state(20), r.state(40)
+    z0, _ = O.full_step(cfg, r.W, c, st0[0], st0[1], r.labels, GAMMA)
+    z0g, _ = r.full(st0)
+    assert max_rel(z0g, z0) < TOL[dtype]
+    z1, _, _, _ = O.cached_step(cfg, r.W, c, st1[0], st1[1], r.labels, N, True, GAMMA)
+    z1g, _, _ = r.cached(st1, N, True)
+    assert max_rel(z1g, z1) < TOL[dtype]
+
+
 def _valid_rule_selection(I, S, n, rule, prio, keys, margin=1e-6):
     """I is a valid choice of the n first tokens under the rule's order, with
     similarities allowed to differ from the oracle's S by `margin` (fp32)."""
