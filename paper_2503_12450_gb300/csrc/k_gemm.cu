@@ -187,7 +187,7 @@ __device__ __forceinline__ bf16* out_row(const GemmEpi& e, int row, int col) {
 }
 }  // namespace tc
 
-template <int BN, int EK, int BK, int F8 = 0, int PAIR = 0, int ROWS = 128>
+template <int BN, int EK, int BK, int F8 = 0, int PAIR = 0, int ROWS = 128, bool SPLIT = false>
 __global__ void __launch_bounds__(tc::Cfg<BN, EK, BK, F8, PAIR, ROWS>::THREADS, 1)
     gemm_bf16_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                         const __grid_constant__ CUtensorMap tmO0, const __grid_constant__ CUtensorMap tmO1,
@@ -217,14 +217,14 @@ __global__ void __launch_bounds__(tc::Cfg<BN, EK, BK, F8, PAIR, ROWS>::THREADS, 
   constexpr int TM = PAIR ? 2 * tc::BM : ROWS;  // rows of a tile
   const int num_m = (M + TM - 1) / TM;
   const int num_n = N / BN;
-  // Pairs: `whole` tiles of the full width, then the others as `split` tiles of
+  // `whole` tiles of the full width, then the others as `split` tiles of
   // BN / split columns each, which spread a short last round over all SMs.
-  const int tiles = PAIR ? whole + (num_m * num_n - whole) * split : num_m * num_n;
+  const int tiles = SPLIT ? whole + (num_m * num_n - whole) * split : num_m * num_n;
   struct Tile {
-    int m, n, bn;  // first row and column of the (pair's) tile, and its width
+    int m, n, bn;  // first row and column of the CTA's or pair's tile, and its width
   };
   auto tile_at = [&](int t) {
-    if (!PAIR || t < whole) return Tile{(t / num_n) * TM, (t % num_n) * BN, BN};
+    if (!SPLIT || t < whole) return Tile{(t / num_n) * TM, (t % num_n) * BN, BN};
     const int u = t - whole, base = whole + u / split, bw = BN / split;
     return Tile{(base / num_n) * TM, (base % num_n) * BN + (u % split) * bw, bw};
   };
@@ -271,8 +271,8 @@ __global__ void __launch_bounds__(tc::Cfg<BN, EK, BK, F8, PAIR, ROWS>::THREADS, 
   const uint32_t tmem_base = *tmem_slot;
   // Tile loads complete on the full barrier of the CTA that issues the MMAs.
   auto expect_stage = [&](int s, int bw) {
-    if (rank == 0)
-      mbar_arrive_expect_tx(&full[s], PAIR ? 2 * (C::A_BYTES + (uint32_t)bw * BK) : C::STAGE_BYTES);
+    const uint32_t b_bytes = (uint32_t)bw * BK * C::EB;
+    if (rank == 0) mbar_arrive_expect_tx(&full[s], PAIR ? 2 * C::A_BYTES + b_bytes : C::A_BYTES + b_bytes);
   };
   auto load_a = [&](int s, int kb, int m0) {
 #pragma unroll
@@ -292,7 +292,7 @@ __global__ void __launch_bounds__(tc::Cfg<BN, EK, BK, F8, PAIR, ROWS>::THREADS, 
         tma_load_2d_pair(bw == BN ? &tmB : &tmBt, cluster_map(smem_u32(&full[s]), 0), dst, kb * BK + a * C::ATOM_E,
                          n0 + rank * (bw / 2));
       else
-        tma_load_2d(&tmB, &full[s], dst, kb * BK + a * C::ATOM_E, n0);
+        tma_load_2d(bw == BN ? &tmB : &tmBt, &full[s], dst, kb * BK + a * C::ATOM_E, n0);
     }
   };
   // Weights are never written by any kernel, so the producer fetches the
@@ -359,7 +359,7 @@ __global__ void __launch_bounds__(tc::Cfg<BN, EK, BK, F8, PAIR, ROWS>::THREADS, 
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + (uint32_t)(buf * BN);
         // N of the MMAs (bits 17 up of the instruction descriptor)
-        const uint32_t idesc = PAIR ? C::IDESC - ((uint32_t)((BN - tile_at(tile).bn) >> 3) << 17) : C::IDESC;
+        const uint32_t idesc = C::IDESC - ((uint32_t)((BN - tile_at(tile).bn) >> 3) << 17);
         for (int kb = 0; kb < KB; ++kb) {
           ok = wait(&full[stage], phase);
           if (!ok) break;
@@ -375,9 +375,9 @@ __global__ void __launch_bounds__(tc::Cfg<BN, EK, BK, F8, PAIR, ROWS>::THREADS, 
               if (PAIR)
                 umma_bf16_pair(d_tmem, a0 + ao, b0 + bo, idesc, (kb | k) != 0 ? 1u : 0u);
               else if (F8)
-                umma_e4m3(d_tmem, a0 + ao, b0 + bo, C::IDESC, (kb | k) != 0 ? 1u : 0u);
+                umma_e4m3(d_tmem, a0 + ao, b0 + bo, idesc, (kb | k) != 0 ? 1u : 0u);
               else
-                umma_bf16(d_tmem, a0 + ao, b0 + bo, C::IDESC, (kb | k) != 0 ? 1u : 0u);
+                umma_bf16(d_tmem, a0 + ao, b0 + bo, idesc, (kb | k) != 0 ? 1u : 0u);
             }
             if (PAIR)
               umma_commit_pair(&empty[stage]);
@@ -474,7 +474,7 @@ __global__ void __launch_bounds__(tc::Cfg<BN, EK, BK, F8, PAIR, ROWS>::THREADS, 
           for (int j = 0; j < 4; ++j) bpre[j] = bp[j];
         }
       };
-      const bool some = !PAIR || c0 < c1;
+      const bool some = !SPLIT || c0 < c1;
       if (EK == tc::RESID_HALF && some) load_res(n0 + c0 * 32);
       if (tc::is_wide<EK>() && some) load_resw(n0 + c0 * 32);
       if (tc::is_bf16out<EK>() && !F8 && some) load_bias(n0 + c0 * 32);
@@ -914,25 +914,35 @@ bool gemm_supported(int dtype, int M, int N, int K, const GemmEpi& epi, const ch
   return true;
 }
 
-// How `base` tiles of width bn run on `pairs` CTA pairs: `whole` of them at full
-// width, the others, a last round that would leave pairs idle, as `split` tiles
-// each. Returns the cost of all rounds, `time` being a full-width round's.
-static long pair_rounds(long base, long pairs, int bn, long time, int* whole, int* split) {
-  const long rounds = base / pairs, rem = base - rounds * pairs;
+// How `base` tiles of width bn run on `slots` CTAs or pairs: `whole` of them at
+// full width, the others, a last round that would leave slots idle, as `split`
+// tiles each (equal parts of a multiple of 32 columns, at least 64). Returns
+// the cost of all rounds, `time` being a full-width round's.
+//
+// A round of split tiles takes these parts of a full one, measured in per cent
+// (half, third and quarter width): residual kinds 68, 56, 60 below K = 2048 and
+// 50 above; bf16 outputs 80, -, 70 on pairs and 83, -, 75 on single CTAs.
+// Measured, one launch of equal tiles -> with a split last round (us). Pairs: M
+// = 20480, width 768: fc2 69.1 -> 65.3; width 1024: fc2 111.3 -> 104.7; M = 5440,
+// width 1024: fc2 44.4 -> 38.4. Single CTAs: out at M = 20480,
+// width 768 32.6 -> 29.6, M = 5440, width 1024 18.0 -> 14.6, M = 6400 19.1 -> 16.2;
+// fc1 at M = 1600, width 768 12.5 -> 10.7, width 1024 15.2 -> 14.0.
+static long rounds_cost(long base, long slots, int bn, long time, bool pair, bool resid, int K, int* whole,
+                        int* split) {
+  const long rounds = base / slots, rem = base - rounds * slots;
   *whole = (int)base;
   *split = 1;
   if (rem == 0) return rounds * time;
   long best = time;
-  // a round of half-width tiles takes about 68 %, of quarter-width ones 50 % of a
-  // full one. Measured, one launch of equal tiles -> with a split last round (us):
-  // M = 20480, width 768: fc2 69.1 -> 65.3; width 1024: out 51.2 -> 47.9, fc2
-  // 111.3 -> 104.7; M = 5440, width 1024: out 17.4 -> 15.0, fc2 44.4 -> 38.4
   if (rounds > 0)
-    for (int s = 2; s <= 4; s *= 2) {
-      const long t = (rem * s + pairs - 1) / pairs * (time * (s == 2 ? 68 : 50) / 100);
-      if (bn % (64 * s) == 0 && t < best) {
+    for (int s = 2; s <= 4; ++s) {
+      if (bn % (32 * s) != 0 || bn / s < 64) continue;
+      const long pct = resid ? (s == 2 ? 68 : s == 3 ? 56 : K < 2048 ? 60 : 50)
+                             : (s == 2 ? (pair ? 80 : 83) : (pair ? 70 : 75));
+      const long t = (rem * s + slots - 1) / slots * (time * pct / 100);
+      if (t < best) {
         best = t;
-        *whole = (int)(rounds * pairs);
+        *whole = (int)(rounds * slots);
         *split = s;
       }
     }
@@ -949,12 +959,19 @@ static cudaError_t launch_tc(const Ctx& c, const void* A, const void* W, int M, 
       !make_tmap_2d(dt, &tb, W, (uint64_t)K, (uint64_t)N, (uint64_t)K * C::EB, C::ATOM_E, C::B_ROWS,
                     CU_TENSOR_MAP_SWIZZLE_128B))
     return cudaErrorInvalidValue;
+  // Single CTAs have a kernel of their own for launches with a split round: a
+  // tile width known only at run time costs short launches 2 to 5 % (out at M =
+  // 1600, width 768: 5.6 against 5.8 us).
+  constexpr bool CAN_SPLIT = PAIR || (BN == 256 && !F8 && (EK == tc::BF16OUT || EK == tc::RESID_WIDE));
+  const auto kernel = gemm_bf16_tc_kernel<BN, EK, BK, F8, PAIR, ROWS, PAIR != 0>;
+  const auto split_kernel = gemm_bf16_tc_kernel<BN, EK, BK, F8, PAIR, ROWS, CAN_SPLIT>;
   static int attr_set[64] = {};
   int dev = 0;
   cudaGetDevice(&dev);
   if (dev >= 0 && dev < 64 && !attr_set[dev]) {
-    cudaError_t e = cudaFuncSetAttribute(gemm_bf16_tc_kernel<BN, EK, BK, F8, PAIR, ROWS>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
+    if (e == cudaSuccess && CAN_SPLIT)
+      e = cudaFuncSetAttribute(split_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
     if (e != cudaSuccess) return e;
     attr_set[dev] = 1;
   }
@@ -976,81 +993,89 @@ static cudaError_t launch_tc(const Ctx& c, const void* A, const void* W, int M, 
       return cudaErrorInvalidValue;
     }
   }
+  constexpr int TM = PAIR ? 2 * tc::BM : ROWS;
+  const int base = ((M + TM - 1) / TM) * (N / BN), slots = PAIR ? c.num_sms / 2 : c.num_sms;
+  int whole = base, split = 1;
+  if (CAN_SPLIT) rounds_cost(base, slots, BN, 100, PAIR, !tc::is_bf16out<EK>(), K, &whole, &split);
   CUtensorMap tbt = tb;
-  if (PAIR) {
-    const int base = ((M + 2 * tc::BM - 1) / (2 * tc::BM)) * (N / BN);
-    int whole = 0, split = 1;
-    pair_rounds(base, c.num_sms / 2, BN, 100, &whole, &split);
-    const int tiles = whole + (base - whole) * split;
-    if (split > 1 && !make_tmap_2d(dt, &tbt, W, (uint64_t)K, (uint64_t)N, (uint64_t)K * C::EB, C::ATOM_E,
-                                   BN / split / 2, CU_TENSOR_MAP_SWIZZLE_128B))
-      return cudaErrorInvalidValue;
-    const int pairs = tiles < c.num_sms / 2 ? tiles : c.num_sms / 2;
-    return launch_pdl_cluster(gemm_bf16_tc_kernel<BN, EK, BK, F8, PAIR, ROWS>, dim3(2 * pairs), dim3(C::THREADS), C::SMEM, 2,
-                              c.stream, ta, tb, to[0], to[1], to[2], tbt, whole, split, tma_out, M, N, K,
-                              epi, c.err);
-  }
-  const int tiles = ((M + ROWS - 1) / ROWS) * (N / BN);
-  const int grid = tiles < c.num_sms ? tiles : c.num_sms;
-  return launch_pdl(gemm_bf16_tc_kernel<BN, EK, BK, F8, PAIR, ROWS>, dim3(grid), dim3(C::THREADS), C::SMEM, c.stream, ta, tb,
-                    to[0], to[1], to[2], tbt, 0, 1, tma_out, M, N, K, epi, c.err);
+  if (split > 1 && !make_tmap_2d(dt, &tbt, W, (uint64_t)K, (uint64_t)N, (uint64_t)K * C::EB, C::ATOM_E,
+                                 C::B_ROWS / split, CU_TENSOR_MAP_SWIZZLE_128B))
+    return cudaErrorInvalidValue;
+  const int tiles = whole + (base - whole) * split;
+  const int grid = tiles < slots ? tiles : slots;
+  if (PAIR)
+    return launch_pdl_cluster(kernel, dim3(2 * grid), dim3(C::THREADS), C::SMEM, 2, c.stream, ta, tb, to[0], to[1], to[2],
+                              tbt, whole, split, tma_out, M, N, K, epi, c.err);
+  return launch_pdl(split > 1 ? split_kernel : kernel, dim3(grid), dim3(C::THREADS), C::SMEM, c.stream, ta, tb,
+                    to[0], to[1], to[2], tbt, whole, split, tma_out, M, N, K, epi, c.err);
 }
 
 // Added to a tile width: tiles of 256 rows on CTA pairs; of 64 rows.
 constexpr int kPair = 1000, kRows64 = 2000;
 
-// Relative time of one round of tiles of width bn (see launch_gemm).
-static int tile_time(int bn, bool resid_half) {
-  static const int widths[4] = {256, 192, 128, 64};
-  static const int t_bf[4] = {256, 243, 187, 153}, t_rh[4] = {256, 199, 153, 110};
-  for (int i = 0; i < 4; ++i)
-    if (widths[i] == bn) return resid_half ? t_rh[i] : t_bf[i];
-  return 256;
+// Relative time of one round of tiles of width bn on single CTAs, measured: a
+// narrower tile does proportionally less work per pipeline stage and runs well
+// below the 256-wide rate, least so with the fp32-residual epilogue over long K
+// (fc2), whose cost follows the width. 64-wide tiles win only where 128-wide
+// ones fit in one round with SMs to spare. (M = 3200, width 768, two rounds of
+// 192 or 256 wide Q/K/V tiles: 10.8 and 12.2 us; M = 40960, width 1024: 34, 51
+// and 26 rounds of 192, 128 and 256 in 194, 237 and 176 us.)
+enum { T_BF16, T_RESID, T_RESID_HALF, T_OTHER };  // bf16 out, residual below and from K = 2048, gated / SiLU / E4M3
+static int tile_time(int bn, int kind) {
+  static const int t[4][4] = {{256, 225, 180, 153}, {256, 224, 167, 153}, {256, 199, 153, 110}, {256, 243, 187, 153}};
+  return t[kind][bn == 256 ? 0 : bn == 192 ? 1 : bn == 128 ? 2 : 3];
 }
 
 // Tile width with the fewest rounds of tiles over the SMs x the time of one
-// tile, and that cost; kPair + width for tiles of 256 rows on CTA pairs.
+// tile; kPair + width for tiles of 256 rows on CTA pairs.
 //
 // A pair's round is shorter than a single CTA's of the same width, because an
 // SM fills and reads 256 instead of 384 operand rows per K step (measured, us
 // per round: Q/K/V at K = 768 4.7 against 5.5, fc2 at K = 3072 17.5 against
-// 20.3, 14.8 against 16.3 at width 192, out-projection at K = 1024 9.4 against
-// 10.0), but a launch of pairs costs about 1.5 us more, which is 54000 / K of
-// the unit (1 / 256 of a single CTA's 256-wide round). The out-projection at
-// K = 768, bound by its residual rows, is slower on pairs (9.2 against 8.2 us
-// a round). Whole GEMMs, one CTA -> pairs (us): M = 20480, width 768: Q/K/V
-// 55.3 -> 46.8, fc1 68.9 -> 67.5, fc2 81.5 -> 70.2; M = 40960, width 1024: Q/K/V
-// 169.8 -> 148.1, out 91.5 -> 87.3, fc1 226.9 -> 201.0, fc2 228.8 -> 211.0. Where
-// the 256-row tiles need more rounds or there is only one short one, single
-// CTAs win (M = 3200, width 768: Q/K/V 11.9 against 13.5, fc2 15.1 against 19.1).
-static int choose_bn(const Ctx& c, int dtype, int M, int N, const GemmEpi& epi, int K, long* cost) {
+// 20.3, 14.8 against 16.3 at width 192), but a launch of pairs costs about 1.5 us
+// more, which is 54000 / K of the unit (1 / 256 of a single CTA's 256-wide
+// round). Whole GEMMs, one CTA -> pairs (us): M = 20480, width 768: Q/K/V 55.3 ->
+// 46.8, fc1 68.9 -> 67.5, fc2 81.5 -> 70.2; M = 40960, width 1024: Q/K/V 169.8 ->
+// 148.1, fc1 226.9 -> 201.0, fc2 228.8 -> 211.0. The out-projection, bound by its
+// residual rows, stays on single CTAs (width 1024, with split last rounds: M =
+// 17408 42.6 against 44.5, M = 40960 86.8 against 89.0; width 768 8.2 against 9.2 a
+// round). Where the 256-row tiles need more rounds or there is only one short
+// one, single CTAs win too (M = 3200, width 768: Q/K/V 11.9 against 13.5, fc2 15.1
+// against 19.1).
+static int choose_bn(const Ctx& c, int dtype, int M, int N, const GemmEpi& epi, int K) {
   const long mt = (M + tc::BM - 1) / tc::BM;
   const bool resid = epi.mode == LAZYMAR_EPI_RESIDUAL;
   const bool resid_half = resid && !epi.gate && K >= 2048;
+  // kinds of tile_time; the first two have a kernel that splits the last round
+  const bool plain = dtype == LAZYMAR_BF16 && epi.mode != LAZYMAR_EPI_SILU && !epi.gate;
+  const int kind = resid_half ? T_RESID_HALF : !plain ? T_OTHER : resid ? T_RESID : T_BF16;
   const int widths[4] = {256, 192, 128, 64};
   int bn = 128;
   long best = -1;
   for (int i = 0; i < 4; ++i) {
     if (N % widths[i] != 0) continue;
-    const long rounds = (mt * (N / widths[i]) + c.num_sms - 1) / c.num_sms;
-    const long t = rounds * tile_time(widths[i], resid_half);
+    const long tiles = mt * (N / widths[i]), time = tile_time(widths[i], kind);
+    int whole, split;
+    const long t = widths[i] == 256 && (kind == T_BF16 || kind == T_RESID)
+                       ? rounds_cost(tiles, c.num_sms, 256, time, false, resid, K, &whole, &split)
+                       : (tiles + c.num_sms - 1) / c.num_sms * time;
     if (best < 0 || t < best) {
       best = t;
       bn = widths[i];
     }
   }
-  if (dtype == LAZYMAR_BF16 && epi.mode != LAZYMAR_EPI_SILU && !epi.gate && !(resid && K < 1024)) {
+  if (plain && kind != T_RESID) {
     const long pt = (mt + 1) / 2, pairs = c.num_sms / 2;
     auto consider = [&](int width, int time) {
       if (pairs < 1 || N % width != 0) return;
       int whole, split;
-      const long t = pair_rounds(pt * (N / width), pairs, width, time, &whole, &split) + 54000 / K;
+      const long t = rounds_cost(pt * (N / width), pairs, width, time, true, resid, K, &whole, &split) + 54000 / K;
       if (t < best) {
         best = t;
         bn = kPair + width;
       }
     };
-    consider(256, resid_half ? 219 : resid ? 228 : 236);
+    consider(256, resid_half ? 219 : 236);
     if (resid_half) consider(192, 186);
   }
   // Few rows: 64 x 64 tiles while they fit in one round. Measured, 128 x 64 tiles ->
@@ -1064,45 +1089,11 @@ static int choose_bn(const Ctx& c, int dtype, int M, int N, const GemmEpi& epi, 
   else if (bn == 128 && dtype == LAZYMAR_BF16 && resid && !epi.gate && K % 128 == 0 &&
            (long)((M + 63) / 64) * (N / 128) <= c.num_sms)
     bn = kRows64 + 128;
-  *cost = best;
   return bn;
 }
 
-// The epilogue of rows [m0, M) of a GEMM as a GEMM of its own.
-static GemmEpi epi_from_row(const GemmEpi& e, int m0) {
-  GemmEpi t = e;
-  if (e.mode == LAZYMAR_EPI_QKV) {
-    t.out = static_cast<bf16*>(e.out) + (size_t)m0 * e.D;
-    if (e.row_map) {
-      t.row_map = e.row_map + m0;
-    } else {
-      t.k_out = static_cast<bf16*>(e.k_out) + (size_t)m0 * e.D;
-      t.v_out = static_cast<bf16*>(e.v_out) + (size_t)m0 * e.D;
-    }
-  } else if (e.mode == LAZYMAR_EPI_RESIDUAL) {
-    t.out = static_cast<float*>(e.out) + (size_t)m0 * e.ldo;
-    if (e.gate) t.gate = static_cast<const bf16*>(e.gate) + (size_t)m0 * e.ldg;
-  } else {
-    t.out = static_cast<bf16*>(e.out) + (size_t)m0 * e.ldo;
-  }
-  return t;
-}
-
-// Kernels issued by launch_gemm on this thread (a last-wave split issues two).
-static thread_local long long t_gemm_kernels = 0;
-long long gemm_kernels_issued() { return t_gemm_kernels; }
-
-static cudaError_t launch_bn_impl(const Ctx& c, int dtype, const void* A, const void* W, int M, int N, int K,
-                                  const GemmEpi& epi, int bn);
 static cudaError_t launch_bn(const Ctx& c, int dtype, const void* A, const void* W, int M, int N, int K,
                              const GemmEpi& epi, int bn) {
-  const cudaError_t e = launch_bn_impl(c, dtype, A, W, M, N, K, epi, bn);
-  if (e == cudaSuccess) ++t_gemm_kernels;
-  return e;
-}
-
-static cudaError_t launch_bn_impl(const Ctx& c, int dtype, const void* A, const void* W, int M, int N, int K,
-                                  const GemmEpi& epi, int bn) {
   if (dtype == LAZYMAR_E4M3) {
     // E4M3 operands (bf16-output kinds): a 128-element stage is one atom; the
     // tile width follows the bf16 choice
@@ -1128,7 +1119,6 @@ static cudaError_t launch_bn_impl(const Ctx& c, int dtype, const void* A, const 
   }
   if (bn == kPair + 192) return launch_tc<192, tc::RESID_HALF, 64, 0, 1>(c, A, W, M, N, K, epi);
   if (bn == kPair + 256) {
-    if (ek == tc::RESID_WIDE) return launch_tc<256, tc::RESID_WIDE, 64, 0, 1>(c, A, W, M, N, K, epi);
     if (ek == tc::RESID_HALF) return launch_tc<256, tc::RESID_HALF, 64, 0, 1>(c, A, W, M, N, K, epi);
     return launch_tc<256, tc::BF16OUT, 64, 0, 1>(c, A, W, M, N, K, epi);
   }
@@ -1174,8 +1164,6 @@ static cudaError_t launch_bn_impl(const Ctx& c, int dtype, const void* A, const 
   return launch_tc<128, tc::BF16OUT, 64>(c, A, W, M, N, K, epi);
 }
 
-
-
 cudaError_t launch_gemm(const Ctx& c, int dtype, const void* A, const void* W, int M, int N, int K,
                         const GemmEpi& epi, int flags) {
   if (M == 0) return cudaSuccess;
@@ -1183,65 +1171,21 @@ cudaError_t launch_gemm(const Ctx& c, int dtype, const void* A, const void* W, i
     const float *a = static_cast<const float*>(A), *w = static_cast<const float*>(W);
     dim3 grid((N + 63) / 64, (M + 63) / 64);
     const long tiles32 = (long)((N + 31) / 32) * ((M + 31) / 32);
-    cudaError_t e;
     // 64 x 64 tiles once they fill the SMs several times (4 per SM: 2560 x 1024 x
     // 256 takes 48.5 against 49.4 us; 2560 x 768 x 256 still 48.0 against 38.0);
     // 16 x 16 tiles while 32 x 32 ones would leave half of the SMs idle (40 x 256 x
     // 1024: 5.3 against 11.7 us)
     if ((long)grid.x * grid.y > 4L * c.num_sms)
-      e = launch_pdl(gemm_f32_kernel, grid, dim3(256), 0, c.stream, a, w, M, N, K, epi);
-    else if (tiles32 * 2 <= c.num_sms)
-      e = K > 512 ? launch_f32_splitk<16, 16>(c, a, w, M, N, K, epi) : launch_f32_splitk<8, 16>(c, a, w, M, N, K, epi);
-    else
-      e = K > 512 ? launch_f32_splitk<16, 32>(c, a, w, M, N, K, epi) : launch_f32_splitk<8, 32>(c, a, w, M, N, K, epi);
-    if (e == cudaSuccess) ++t_gemm_kernels;
-    return e;
+      return launch_pdl(gemm_f32_kernel, grid, dim3(256), 0, c.stream, a, w, M, N, K, epi);
+    if (tiles32 * 2 <= c.num_sms)
+      return K > 512 ? launch_f32_splitk<16, 16>(c, a, w, M, N, K, epi) : launch_f32_splitk<8, 16>(c, a, w, M, N, K, epi);
+    return K > 512 ? launch_f32_splitk<16, 32>(c, a, w, M, N, K, epi) : launch_f32_splitk<8, 32>(c, a, w, M, N, K, epi);
   }
-  // Tile width: the one with the fewest rounds of tiles over the SMs x the
-  // time of one tile, on single CTAs or pairs (choose_bn). Relative tile times 187 : 243 : 256 for BN = 128 : 192 :
-  // 256 (measured, one round of 128 x BN x 3072 tiles): a narrower tile does
-  // proportionally less work per pipeline stage and runs well below the
-  // BN = 256 rate. BN = 64 (153, on the line through the 128 and 256 points)
-  // wins only when the 128-wide tiles fit in one round with SMs to spare: the
-  // few-row GEMMs of the diffusion head. The fp32-residual epilogue over long K
-  // (fc2) costs in proportion to the tile width: its measured round times at
-  // K = 3072 are 153 : 199 : 256 (110 for 64).
   if (flags == 2 && N % 256 == 0) return launch_bn(c, dtype, A, W, M, N, K, epi, 256);
   if (flags == 3 && N % 192 == 0) return launch_bn(c, dtype, A, W, M, N, K, epi, 192);
   if (flags == 4) return launch_bn(c, dtype, A, W, M, N, K, epi, 64);
   if (flags != 0) return launch_bn(c, dtype, A, W, M, N, K, epi, 128);
-  long cost = 0;
-  const int bn = choose_bn(c, dtype, M, N, epi, K, &cost);
-  // Last-wave split of the fp32-residual GEMM over short K (the
-  // out-projection): when its tiles fill several rounds but the last one only
-  // partly, the row tiles of the whole waves run as one launch and the
-  // remaining rows as a second launch, with the tile width that suits their
-  // count (narrower tiles spread them over all SMs), if the model puts the
-  // pair at least 2 % below the one launch. Measured on the MAR-B full layer:
-  // the partial fourth round of 256-wide tiles costs a whole round (8.2 us),
-  // while the last 8 row tiles as 64-wide tiles take 4.9 us (34.1 -> 30.9
-  // us). The other kinds lose: the residual over long K (fc2) runs its partial
-  // last round faster than a full one (32 tiles of 192 in 10.8 us against
-  // 17.1 us), and the full-layer Q/K/V went 55.9 -> 57.6 us split.
-  if (dtype == LAZYMAR_BF16 && epi.mode == LAZYMAR_EPI_RESIDUAL && !epi.gate && K < 2048 && bn < kPair) {
-    const long mt = (M + tc::BM - 1) / tc::BM, nn = N / bn;
-    const long rounds = (mt * nn + c.num_sms - 1) / c.num_sms;
-    const long body_rt = rounds >= 3 ? (rounds - 1) * c.num_sms / nn : 0;  // whole row tiles of the full waves
-    if (body_rt > 0 && body_rt < mt) {
-      const int Mb = (int)(body_rt * tc::BM);
-      long tail_cost = 0;
-      const int tail_bn = choose_bn(c, dtype, M - Mb, N, epi, K, &tail_cost);
-      const long body_rounds = (body_rt * nn + c.num_sms - 1) / c.num_sms;
-      const long split_cost = body_rounds * tile_time(bn, false) + tail_cost;
-      if (split_cost * 50 <= cost * 49) {
-        const cudaError_t e = launch_bn(c, dtype, A, W, Mb, N, K, epi, bn);
-        if (e != cudaSuccess) return e;
-        return launch_bn(c, dtype, static_cast<const bf16*>(A) + (size_t)Mb * K, W, M - Mb, N, K,
-                         epi_from_row(epi, Mb), tail_bn);
-      }
-    }
-  }
-  return launch_bn(c, dtype, A, W, M, N, K, epi, bn);
+  return launch_bn(c, dtype, A, W, M, N, K, epi, choose_bn(c, dtype, M, N, epi, K));
 }
 
 }  // namespace lm

@@ -348,6 +348,42 @@ def test_linear_pairs_equal_single_ctas(M, N, K, epi):
         assert (res[1][0][M:] == 7.0).all()
 
 
+@pytest.mark.parametrize("M,N,K,epi", [
+    # on 152 SMs: one round of 256-wide tiles and 4 or 8 tiles in quarters, 64 in halves
+    (1571, 3072, 128, lm.LAZYMAR_EPI_GELU),
+    (1600, 3072, 832, lm.LAZYMAR_EPI_BIAS),
+    (2500, 2048, 1024, lm.LAZYMAR_EPI_RESIDUAL),
+    (3377, 2048, 64, lm.LAZYMAR_EPI_RESIDUAL),
+    (2241, 3072, 256, lm.LAZYMAR_EPI_QKV),
+    (20480, 768, 768, lm.LAZYMAR_EPI_RESIDUAL),     # four rounds, the last in quarters
+])
+def test_linear_split_round_equals_equal_tiles(M, N, K, epi):
+    """256-wide tiles whose last round is split into narrower ones (forced width,
+    and the automatic choice) give the 128-wide tiles' results bit for bit."""
+    torch = torch_cuda()
+    g = torch.Generator(device="cuda")
+    g.manual_seed(M + N + K)
+    r = lambda *s: torch.randn(s, generator=g, device="cuda")
+    a, w, b = r(M, K).bfloat16(), (0.05 * r(N, K)).bfloat16(), r(N).bfloat16()
+    D = N // 3
+    maps = [None, torch.randperm(M + 40, generator=g, device="cuda")[:M].int()] if epi == lm.LAZYMAR_EPI_QKV else [None]
+    for row_map in maps:
+        res = []
+        for flags in (1, 2, 0):
+            if epi == lm.LAZYMAR_EPI_QKV:
+                outs = [torch.full((M + 40, D), 7.0, device="cuda", dtype=torch.bfloat16) for _ in range(3)]
+                lm.lazymar_linear(DT["bf16"], epi, a, w, b, M, N, K, outs[0], D, outs[1], outs[2], row_map, flags)
+            else:
+                dt = torch.float32 if epi == lm.LAZYMAR_EPI_RESIDUAL else torch.bfloat16
+                outs = [torch.full((M + 40, N), 7.0, device="cuda", dtype=dt)]
+                lm.lazymar_linear(DT["bf16"], epi, a, w, b, M, N, K, outs[0], N, flags=flags)
+            sync()
+            res.append(outs)
+        for other in res[1:]:
+            assert all(torch.equal(x, y) for x, y in zip(res[0], other))
+        assert (res[1][0][M:] == 7.0).all()
+
+
 @pytest.mark.parametrize("M,N,K", [(1, 384, 128), (63, 768, 256), (65, 768, 3072), (200, 2304, 768), (449, 1024, 1024),
                                    (320, 1536, 640), (1537, 768, 768), (1600, 768, 3072)])
 @pytest.mark.parametrize("epi", [lm.LAZYMAR_EPI_BIAS, lm.LAZYMAR_EPI_GELU, lm.LAZYMAR_EPI_RESIDUAL,
