@@ -142,9 +142,9 @@ __global__ void __launch_bounds__(128) attention_f32_kernel(const float* __restr
 // ---------------------------------------------------------------------------
 // bf16: tcgen05 tensor cores, accumulators in tensor memory
 // ---------------------------------------------------------------------------
-// One CTA per (128-query tile, head, row). Warps 0-3 run the softmax (thread t
-// owns query row t = tensor-memory lane t) and issue the TMA loads; lane 0 of
-// warp 4 issues the MMAs. Keys stream in 64-key chunks c:
+// One CTA per (128-query tile, head, row), or (head, row) of at most 64 queries.
+// Warps 0-3 (0-1) run the softmax (thread t owns query row t = tensor-memory
+// lane t) and issue the TMA loads; lane 0 of the last warp issues the MMAs. Keys stream in 64-key chunks c:
 //   S(c)  = Q K(c)^T      (tcgen05.mma 128 x 64 x DH, K-major operands) into
 //                         tensor-memory columns [0, 64);
 //   P(c)  = exp2(S(c) * log2(e)/sqrt(d) - m), written as bf16 to shared memory;
@@ -165,25 +165,26 @@ __global__ void __launch_bounds__(128) attention_f32_kernel(const float* __restr
 // N = 64 MMA on the first part of V into O columns [64, 128) and an N = 16 MMA
 // on the remainder into [128, 144).
 namespace at2 {
-constexpr int QT = 128;   // queries per CTA (MMA M)
+constexpr int QT = 128;   // rows of an MMA
 constexpr int KC = 64;    // keys per chunk
-constexpr int THREADS = 160;
-constexpr int Q_BYTES = QT * 128;    // 128 rows x 64 bf16, 128B swizzle
 constexpr int KV_BYTES = KC * 128;   // 64 rows x 64 bf16
-constexpr int P_BYTES = QT * 128;    // 128 rows x 64 keys
 constexpr int Q2_BYTES = QT * 32;    // 128 rows x 16 bf16, 32B swizzle (80-wide heads)
 constexpr int KV2_BYTES = KC * 32;   // 64 rows x 16 bf16
 constexpr float RESCALE_THRESHOLD = 8.0f;
-template <int DH>
+template <int DH, int QR>
 struct Cfg {
-  static_assert(DH == 64 || DH == 80, "head width 64 or 80");
+  static_assert((DH == 64 && (QR == 64 || QR == QT)) || (DH == 80 && QR == QT), "head width 64 or 80");
   static constexpr bool TAIL = DH == 80;
+  static constexpr int THREADS = QR + 32;
+  static constexpr int Q_BYTES = QR * 128;  // QR rows x 64 bf16, 128B swizzle
+  static constexpr int P_BYTES = QR * 128;  // QR rows x 64 keys
   static constexpr int TAIL_BYTES = TAIL ? Q2_BYTES + 4 * KV2_BYTES : 0;
   static constexpr int SMEM = 1024 + Q_BYTES + 4 * KV_BYTES + P_BYTES + TAIL_BYTES + 256;
   static constexpr uint32_t TMEM_COLS = TAIL ? 256 : 128;  // S [0, 64), O [64, 64 + DH)
   static constexpr uint32_t Q_TX = Q_BYTES + (TAIL ? Q2_BYTES : 0);
   static constexpr uint32_t KV_TX = KV_BYTES + (TAIL ? KV2_BYTES : 0);
-  static constexpr int MIN_BLOCKS = TAIL ? 2 : 3;  // shared memory allows three (64) or two (80) per SM
+  // shared memory allows three (64) or two (80) per SM, of 64 queries four
+  static constexpr int MIN_BLOCKS = TAIL ? 2 : QR == QT ? 3 : 4;
 };
 // kind::f16, D fp32, A/B bf16, M = 128, N = 64 (or 16); bit 16 marks B as MN-major.
 constexpr uint32_t IDESC_S = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(64 >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
@@ -217,35 +218,38 @@ __device__ __forceinline__ uint32_t sw(int r, int c) { return (uint32_t)(r * 128
 enum { B_Q = 0, B_K = 1, B_V = 3, B_S_FULL = 5, B_S_FREE = 6, B_P_FULL = 7, B_O_DONE = 8, N_BARS = 9 };
 }  // namespace at2
 
-template <int DH>
-__global__ void __launch_bounds__(at2::THREADS, at2::Cfg<DH>::MIN_BLOCKS)
+template <int DH, int QR>
+__global__ void __launch_bounds__(at2::Cfg<DH, QR>::THREADS, at2::Cfg<DH, QR>::MIN_BLOCKS)
     attention_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                         const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmQ2,
                         const __grid_constant__ CUtensorMap tmK2, const __grid_constant__ CUtensorMap tmV2, bf16* o,
                         int n_q, int T, int D, float scale_log2, unsigned* err) {
   using namespace at2;
-  using C = Cfg<DH>;
+  using C = Cfg<DH, QR>;
   constexpr bool TAIL = C::TAIL;
+  constexpr int MMA_WARP = QR / 32;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  uint8_t* sQ = smem;                    // 16 KB
-  uint8_t* sK = sQ + Q_BYTES;            // 2 x 8 KB
+  // With 64 queries the MMAs read what follows Q and P as their other 64 rows,
+  // whose results nobody reads.
+  uint8_t* sQ = smem;                    // 16 KB (8 KB)
+  uint8_t* sP = sQ + C::Q_BYTES;         // 16 KB (8 KB), also the output staging tile
+  uint8_t* sK = sP + C::P_BYTES;         // 2 x 8 KB
   uint8_t* sV = sK + 2 * KV_BYTES;       // 2 x 8 KB
-  uint8_t* sP = sV + 2 * KV_BYTES;       // 16 KB (also the output staging tile)
-  uint8_t* sQ2 = sP + P_BYTES;           // 80-wide heads: 4 KB, then 2 x 2 KB of K and of V remainders
+  uint8_t* sQ2 = sV + 2 * KV_BYTES;      // 80-wide heads: 4 KB, then 2 x 2 KB of K and of V remainders
   uint8_t* sK2 = sQ2 + Q2_BYTES;
   uint8_t* sV2 = sK2 + 2 * KV2_BYTES;
-  uint64_t* bars = reinterpret_cast<uint64_t*>(sP + P_BYTES + C::TAIL_BYTES);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(sQ2 + C::TAIL_BYTES);
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + N_BARS);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int qt = blockIdx.x, h = blockIdx.y, r = blockIdx.z;
-  const int q0 = r * n_q + qt * QT, kv0 = r * T, col = h * DH;
+  const int q0 = r * n_q + qt * QR, kv0 = r * T, col = h * DH;
   const int nck = (T + KC - 1) / KC;
   // Softmax warps whose 32 query rows all lie beyond n_q sit out: their rows of
   // S, P and O are never read back (matrix rows are independent).
-  const int n_valid = min(QT, n_q - qt * QT);
+  const int n_valid = min(QR, n_q - qt * QR);
   const int n_act = (n_valid + 31) / 32;
 
   if (tid == 0) {
@@ -262,7 +266,7 @@ __global__ void __launch_bounds__(at2::THREADS, at2::Cfg<DH>::MIN_BLOCKS)
       prefetch_tmap(&tmV2);
     }
   }
-  if (warp == 4) {
+  if (warp == MMA_WARP) {
     tmem_alloc(tmem_slot, C::TMEM_COLS);
     tmem_relinquish();
   }
@@ -286,7 +290,7 @@ __global__ void __launch_bounds__(at2::THREADS, at2::Cfg<DH>::MIN_BLOCKS)
     if (TAIL) tma_load_2d(&tmV2, bar, sV2 + (c & 1) * KV2_BYTES, col + 64, kv0 + c * KC);
   };
 
-  if (warp == 4) {
+  if (warp == MMA_WARP) {
     // ---------------- MMA issuer ----------------
     if (lane == 0) {
       const uint64_t qd = sw128_desc(smem_u32(sQ)), pd = sw128_desc(smem_u32(sP));
@@ -474,7 +478,7 @@ __global__ void __launch_bounds__(at2::THREADS, at2::Cfg<DH>::MIN_BLOCKS)
         uint32_t rt[16];
         tmem_ld16(tmem + t_lane + 128, rt);
         tmem_wait_ld();
-        const int qi = qt * QT + tid;
+        const int qi = qt * QR + tid;
         if (qi < n_q) {
           uint4 t0, t1;
           t0.x = pack_bf16(__uint_as_float(rt[0]) * inv, __uint_as_float(rt[1]) * inv);
@@ -495,7 +499,7 @@ __global__ void __launch_bounds__(at2::THREADS, at2::Cfg<DH>::MIN_BLOCKS)
 #pragma unroll
       for (int i = 0; i < 8; ++i) {
         const int row = warp * 32 + i * 4 + (lane >> 3), ch = lane & 7;
-        const int qi = qt * QT + row;
+        const int qi = qt * QR + row;
         if (qi < n_q) {
           const uint4 val = *reinterpret_cast<const uint4*>(sP + sw(row, ch));
           *reinterpret_cast<uint4*>(o + (size_t)(r * n_q + qi) * D + col + 8 * ch) = val;
@@ -505,7 +509,7 @@ __global__ void __launch_bounds__(at2::THREADS, at2::Cfg<DH>::MIN_BLOCKS)
     tc_fence_before();
   }
   __syncthreads();
-  if (warp == 4) {
+  if (warp == MMA_WARP) {
     tc_fence_after();
     tmem_dealloc(tmem, C::TMEM_COLS);
   }
@@ -892,22 +896,39 @@ bool attention_supported(int dtype, int heads, int dh, const char** why) {
   return true;
 }
 
-template <int DH>
+// Dynamic shared memory with which no more CTAs of a grid fit an SM than an even
+// spread over the waves of a kernel that allows `most` needs: the CTAs that start
+// when the predecessor's leave would else fill the first SMs and leave others
+// idle, and waves be uneven. Measured, the attention between its Q/K/V and output
+// projections, as many CTAs as fit -> spread (us): 96 CTAs of 50 queries and 320
+// keys 18.0 -> 16.0, 240 19.5 -> 18.2, 384 23.5 -> 22.8; 96 CTAs of 128 queries and 320
+// keys 28.7 -> 27.5; width 80, 384 CTAs of 50 and 320 36.2 -> 34.7. By itself, two waves
+// of 768 CTAs of 50 queries, their keys and values not in L2, 17.5 -> 17.0.
+constexpr int SM_SMEM = 228 * 1024, CTA_RESERVED = 1024;  // of an SM; taken by the system for each CTA
+constexpr int SPREAD_MAX = SM_SMEM / 2;                   // one CTA per SM
+static int spread_smem(int smem, int most, long long ctas, int sms) {
+  const long long slots = (long long)most * sms, waves = (ctas + slots - 1) / slots;
+  const int per = (int)((ctas + waves * sms - 1) / (waves * sms));
+  const int least = SM_SMEM / (per + 1) - CTA_RESERVED + 256;  // per + 1 CTAs do not fit
+  return per < most && smem < least ? least : smem;
+}
+
+template <int DH, int QR>
 static cudaError_t launch_attn_tc(const Ctx& c, const void* q, const void* k, const void* v, void* o, int rows,
                                   int n_q, int T, int heads) {
-  using C = at2::Cfg<DH>;
+  using C = at2::Cfg<DH, QR>;
   if (T < 1) return cudaErrorInvalidValue;  // the kernel's final wait needs at least one key chunk
   const int D = heads * DH;
   const uint64_t pitch = (uint64_t)D * 2;
   CUtensorMap mq, mk, mv, mq2, mk2, mv2;
-  if (!make_tmap_bf16(&mq, q, D, (uint64_t)rows * n_q, pitch, 64, at2::QT, CU_TENSOR_MAP_SWIZZLE_128B) ||
+  if (!make_tmap_bf16(&mq, q, D, (uint64_t)rows * n_q, pitch, 64, QR, CU_TENSOR_MAP_SWIZZLE_128B) ||
       !make_tmap_bf16(&mk, k, D, (uint64_t)rows * T, pitch, 64, at2::KC, CU_TENSOR_MAP_SWIZZLE_128B) ||
       !make_tmap_bf16(&mv, v, D, (uint64_t)rows * T, pitch, 64, at2::KC, CU_TENSOR_MAP_SWIZZLE_128B))
     return cudaErrorInvalidValue;
   if (C::TAIL) {
     // 16-column remainders: x = h * 80 + 64 elements = 160 h + 128 bytes, a
     // multiple of 16 bytes as TMA requires
-    if (!make_tmap_bf16(&mq2, q, D, (uint64_t)rows * n_q, pitch, 16, at2::QT, CU_TENSOR_MAP_SWIZZLE_32B) ||
+    if (!make_tmap_bf16(&mq2, q, D, (uint64_t)rows * n_q, pitch, 16, QR, CU_TENSOR_MAP_SWIZZLE_32B) ||
         !make_tmap_bf16(&mk2, k, D, (uint64_t)rows * T, pitch, 16, at2::KC, CU_TENSOR_MAP_SWIZZLE_32B) ||
         !make_tmap_bf16(&mv2, v, D, (uint64_t)rows * T, pitch, 16, at2::KC, CU_TENSOR_MAP_SWIZZLE_32B))
       return cudaErrorInvalidValue;
@@ -921,13 +942,14 @@ static cudaError_t launch_attn_tc(const Ctx& c, const void* q, const void* k, co
   cudaGetDevice(&dev);
   if (dev >= 0 && dev < 64 && !attr_set[dev]) {
     cudaError_t e =
-        cudaFuncSetAttribute(attention_tc_kernel<DH>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
+        cudaFuncSetAttribute(attention_tc_kernel<DH, QR>, cudaFuncAttributeMaxDynamicSharedMemorySize, SPREAD_MAX);
     if (e != cudaSuccess) return e;
     attr_set[dev] = 1;
   }
   const float scale_log2 = 1.4426950408889634f / sqrtf((float)DH);  // log2(e) / sqrt(d)
-  dim3 grid((n_q + at2::QT - 1) / at2::QT, heads, rows);
-  return launch_pdl(attention_tc_kernel<DH>, grid, dim3(at2::THREADS), (size_t)C::SMEM, c.stream, mq, mk, mv, mq2,
+  dim3 grid((n_q + QR - 1) / QR, heads, rows);
+  const size_t smem = spread_smem(C::SMEM, C::MIN_BLOCKS, (long long)grid.x * heads * rows, c.num_sms);
+  return launch_pdl(attention_tc_kernel<DH, QR>, grid, dim3(C::THREADS), smem, c.stream, mq, mk, mv, mq2,
                     mk2, mv2, static_cast<bf16*>(o), n_q, T, D, scale_log2, c.err);
 }
 
@@ -960,13 +982,18 @@ static cudaError_t launch_attn_tm(const Ctx& c, const void* q, const void* k, co
   cudaGetDevice(&dev);
   if (dev >= 0 && dev < 64 && !attr_set[dev]) {
     cudaError_t e =
-        cudaFuncSetAttribute(attention_tm_kernel<DH>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
+        cudaFuncSetAttribute(attention_tm_kernel<DH>, cudaFuncAttributeMaxDynamicSharedMemorySize, SPREAD_MAX);
     if (e != cudaSuccess) return e;
     attr_set[dev] = 1;
   }
   const float scale_log2 = 1.4426950408889634f / sqrtf((float)DH);  // log2(e) / sqrt(d)
   dim3 grid((n_q + at4::QT - 1) / at4::QT, heads, rows);
-  return launch_pdl(attention_tm_kernel<DH>, grid, dim3(at4::THREADS), (size_t)C::SMEM, c.stream, mq, mk, mv, mq2,
+  // (more than one wave is not evened out: 26 rows x 16 heads x 320 x 320, two waves of
+  // four or three of three CTAs per SM, 23.8 against 25.2 us)
+  const long long ctas = (long long)grid.x * heads * rows;
+  const size_t smem =
+      ctas <= (long long)C::MIN_BLOCKS * c.num_sms ? spread_smem(C::SMEM, C::MIN_BLOCKS, ctas, c.num_sms) : C::SMEM;
+  return launch_pdl(attention_tm_kernel<DH>, grid, dim3(at4::THREADS), smem, c.stream, mq, mk, mv, mq2,
                     mk2, static_cast<bf16*>(o), n_q, T, D, scale_log2, c.err);
 }
 
@@ -987,19 +1014,30 @@ cudaError_t launch_attention(const Ctx& c, int dtype, const void* q, const void*
                       static_cast<const float*>(k), static_cast<const float*>(v), static_cast<float*>(o), n_q, T,
                       heads * dh, dh, 1.0f / sqrtf((float)dh));
   }
-  // attention_tm_kernel overlaps four CTAs of an SM, attention_tc_kernel the
-  // chunks of one (it may issue S(c + 1) while P(c) is on its way): the former
-  // needs more CTAs than one wave of the latter. Below that, and for 64-wide heads with at
-  // most 64 queries (bound by the stream of keys and values, of which fewer are
-  // in flight), the latter is faster: 32 rows x 12 heads x 50 x 320 7.7 against
-  // 9.3 us, 64 rows 14.5 against 15.7, 2 x 16 x 320 x 320 6.2 against 7.1; width
-  // 80, 3 x 12 x 129 x 200 6.4 against 7.3.
+  // attention_tm_kernel overlaps four CTAs of an SM, attention_tc_kernel, of which
+  // three or (width 80) two fit, the chunks of one (it may issue S(c + 1) while P(c)
+  // is on its way). The former is faster where it saves a wave, the latter where
+  // the waves are as many. Measured, latter against former (us): width 64, 16 heads,
+  // 300 queries, 1088 keys: 432 CTAs 23.4 : 25.0, 576 37.4 : 28.1, 912 44.8 : 50.8,
+  // 1008 58.5 : 51.6, 1344 64.0 : 69.5, 1392 72.3 : 70.6, 2496 118.1 : 112.8; 320 keys:
+  // 480 15.7 : 11.7, 768 18.2 : 19.1, 1008 23.9 : 21.1. Width 80, 320 keys: 384 17.0 :
+  // 13.6, 624 23.3 : 22.5, 912 27.2 : 26.8, 1200 34.5 : 29.0; two waves against three
+  // lose with many keys, in whose short last wave an SM has one or two CTAs: 704 CTAs
+  // of 500 keys 34.1 : 33.4, 850 51.4 : 49.1, 1088 59.7 : 62.3.
+  // With at most 64 queries (of width 64) attention_tc_kernel's CTAs hold 64 rows and
+  // four of them fit too (two softmax warps each): 64 rows x 12 heads x 50 x 320
+  // 13.9 against 14.4 us with 128 rows and 15.7 in attention_tm_kernel, 64 x 8
+  // 8.6 against 12.6 with 128, 64 rows x 16 heads x 64 x 320 17.3 against 21.3.
+  if (dh == 64 && n_q <= 64) return launch_attn_tc<64, 64>(c, q, k, v, o, rows, n_q, T, heads);
   const long long ctas = (long long)((n_q + 127) / 128) * heads * rows;
+  const long long tm_slots = 4LL * c.num_sms, tc_slots = (dh == 64 ? 3LL : 2LL) * c.num_sms;
+  const long long tm_waves = (ctas + tm_slots - 1) / tm_slots, tc_waves = (ctas + tc_slots - 1) / tc_slots;
+  const bool tm = tm_waves < tc_waves && !(dh == 80 && tm_waves == 2 && tc_waves == 3 && T >= 1024);
   if (dh == 64)
-    return n_q > 64 && ctas > 3LL * c.num_sms ? launch_attn_tm<64>(c, q, k, v, o, rows, n_q, T, heads)
-                                              : launch_attn_tc<64>(c, q, k, v, o, rows, n_q, T, heads);
-  return ctas > 2LL * c.num_sms ? launch_attn_tm<80>(c, q, k, v, o, rows, n_q, T, heads)
-                                : launch_attn_tc<80>(c, q, k, v, o, rows, n_q, T, heads);
+    return tm ? launch_attn_tm<64>(c, q, k, v, o, rows, n_q, T, heads)
+              : launch_attn_tc<64, 128>(c, q, k, v, o, rows, n_q, T, heads);
+  return tm ? launch_attn_tm<80>(c, q, k, v, o, rows, n_q, T, heads)
+            : launch_attn_tc<80, 128>(c, q, k, v, o, rows, n_q, T, heads);
 }
 
 }  // namespace lm

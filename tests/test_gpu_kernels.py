@@ -618,6 +618,15 @@ def test_attention_large_grids(rows, n_q, T, heads, dh, q_std):
     assert max_rel(got, host(ref)) < 1e-2
 
 
+@pytest.mark.parametrize("rows,n_q,T,q_std", [
+    (1, 1, 65, 1.0), (2, 31, 64, 1.0), (10, 33, 320, 1.0), (24, 63, 129, 1.0), (32, 64, 1, 1.0),
+    (40, 64, 320, 1.0), (64, 32, 63, 1.0), (40, 50, 1088, 4.0),     # four CTAs per SM
+])
+def test_attention_up_to_64_queries(rows, n_q, T, q_std):
+    """CTAs of 64 query rows, one to four per SM: the large grids' checks."""
+    test_attention_large_grids(rows, n_q, T, 12, 64, q_std)
+
+
 @pytest.mark.parametrize("M,D,gather,dtype", [(100, 768, False, "bf16"), (50, 1280, True, "bf16"),
                                               (80, 256, True, "fp32"), (3, 1024, False, "fp32")])
 def test_layernorm(M, D, gather, dtype):
