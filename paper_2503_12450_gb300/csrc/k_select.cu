@@ -26,12 +26,11 @@
 // selections. The kernel computes the three sums exactly on the integer pipe
 // (GB300's fp64 rate is a small fraction of its integer rate) and rounds each
 // once. fp32 x fp32 products are exact in fp64 too, but a sum of them is
-// rounded at every addition, so the kernel's lane-strided order and the
-// oracle's pairwise order can differ in the last bits of S (a relative 1e-15
-// or so). Two tokens whose similarities lie that close may then be ordered
-// differently; every other fp32 selection is identical.
+// rounded at every addition: the kernel's sums (correctly rounded but for the
+// last bit) and the oracle's pairwise ones can differ in the last bits of S (a
+// relative 1e-15 or so). Two tokens whose similarities lie that close may then be
+// ordered differently; every other fp32 selection is identical.
 #include <cfloat>
-#include <climits>
 
 #include "lazymar_internal.cuh"
 
@@ -48,18 +47,24 @@ __device__ __forceinline__ unsigned long long sim_key(double s) {
   return (u >> 63) ? ~u : (u | 0x8000000000000000ull);
 }
 
-// The sums of one token: dot, |a|^2, |c|^2 as v[i] * 2^e[i] with integer v,
-// or, with e[0] == INT_MIN, as the bits of three doubles.
+// The sums of one token: dot, |a|^2, |c|^2, as v[i] * 2^e[i] with integer v, as
+// the bits of a double in v[i], or as the sum of three floats: the bits of two in
+// v[i] and of one in e[i].
+enum { SUMS_INT, SUMS_F64, SUMS_F32X3 };
 struct SimSums {
   long long v[3];
-  int e[3];
+  int e[3], kind;
 };
 
 __device__ __forceinline__ double sim_value(const SimSums& s) {
   double d[3];
 #pragma unroll
-  for (int i = 0; i < 3; ++i)
-    d[i] = s.e[0] == INT_MIN ? __longlong_as_double(s.v[i]) : ldexp((double)s.v[i], s.e[i]);
+  for (int i = 0; i < 3; ++i) {
+    const float hi = __int_as_float((int)s.v[i]), mid = __int_as_float((int)(s.v[i] >> 32)), lo = __int_as_float(s.e[i]);
+    d[i] = s.kind == SUMS_F64     ? __longlong_as_double(s.v[i])
+           : s.kind == SUMS_F32X3 ? ((double)hi + (double)mid) + (double)lo
+                                  : ldexp((double)s.v[i], s.e[i]);
+  }
   const double eps = 1e-8;
   return d[0] / sqrt(fmax(d[1] * d[2], eps * eps));
 }
@@ -107,8 +112,101 @@ __device__ __forceinline__ void sums_fp64(const T* a, const T* c, int D, int lan
   s.v[0] = __double_as_longlong(dot);
   s.v[1] = __double_as_longlong(na);
   s.v[2] = __double_as_longlong(nc);
-  s.e[0] = INT_MIN;
-  s.e[1] = s.e[2] = 0;
+  s.kind = SUMS_F64;
+}
+
+// Two running sums, one per half of the packed registers, each the unevaluated
+// sum of three floats, of which each is about 2^-24 of the one before.
+struct F32x3 {
+  unsigned long long s, c, d;
+};
+__device__ __forceinline__ unsigned long long f32x2_sub(unsigned long long a, unsigned long long b) {
+  return f32x2_fma(b, 0xBF800000BF800000ull, a);  // a - 1 b
+}
+// a + b = s + e exactly (Knuth's two-sum)
+__device__ __forceinline__ void two_sum(unsigned long long a, unsigned long long b, unsigned long long& s,
+                                        unsigned long long& e) {
+  const unsigned long long t = f32x2_add(a, b), bb = f32x2_sub(t, a);
+  e = f32x2_add(f32x2_sub(a, f32x2_sub(t, bb)), f32x2_sub(b, bb));
+  s = t;
+}
+// x y = p + e exactly; both join the sum.
+__device__ __forceinline__ void add_product(F32x3& t, unsigned long long x, unsigned long long y) {
+  const unsigned long long p = f32x2_fma(x, y, 0ull);
+  const unsigned long long e = f32x2_fma(x, y, p ^ 0x8000000080000000ull);
+  unsigned long long q, r, u;
+  two_sum(t.s, p, t.s, q);
+  two_sum(t.c, q, t.c, r);
+  two_sum(t.c, e, t.c, u);
+  t.d = f32x2_add(t.d, f32x2_add(r, u));
+}
+__device__ __forceinline__ void add_sum(F32x3& t, const F32x3& o) {
+  unsigned long long q, r, u;
+  two_sum(t.s, o.s, t.s, q);
+  two_sum(t.c, o.c, t.c, r);
+  two_sum(t.c, q, t.c, u);
+  t.d = f32x2_add(f32x2_add(t.d, o.d), f32x2_add(r, u));
+}
+
+// Sums of one fp32 token in triples of floats (Ogita, Rump and Oishi's compensated
+// dot product with one more level): products and the errors of the first two
+// levels are exact, and the third's roundings lie 2^-72 below the sum of the
+// terms' magnitudes, so the sums are rounded to double once, where an fp64 sum
+// rounds at every addition. GB300 has about two fp64 lanes per SM, and an element
+// pair costs five fp64 instructions, 320 issue cycles of a scheduler, against about
+// 45 here with two elements per instruction. Measured, fp64 sums -> this (us a
+// call): 64 rows x 320 tokens x 768 200 -> 74, 26 x 320 x 1024 132 -> 51, 1 x 1088 x
+// 1280 146 -> 63 (84 with fp64 sums spread over all SMs), 8 x 320 x 1280 83 -> 32.
+// Largest error of the sums of 60 vectors of 256 to 1280 normal elements: 1.1e-16 of
+// the sum, of fp64 sums 1.2e-14.
+// Vectors with an element of magnitude from 2^52 or (nonzero) below 2^-51, whose
+// products could overflow or lose bits, and ones with Inf or NaN take fp64 sums.
+__device__ __forceinline__ void sums_f32(const float* a, const float* c, int D, int lane, SimSums& s) {
+  F32x3 dot{}, na{}, nc{};
+  uint32_t most = 0, least = 0xFFFFFFFFu;  // of the magnitudes' bits; of those - 1, in which zeros are the largest
+#pragma unroll 2
+  for (int i = lane * 4; i < D; i += 128) {
+    const ulonglong2 x = *reinterpret_cast<const ulonglong2*>(a + i), y = *reinterpret_cast<const ulonglong2*>(c + i);
+    const unsigned long long w[4] = {x.x, x.y, y.x, y.y};
+#pragma unroll
+    for (int h = 0; h < 4; ++h) {
+      const uint32_t m0 = (uint32_t)w[h] & 0x7FFFFFFFu, m1 = (uint32_t)(w[h] >> 32) & 0x7FFFFFFFu;
+      most = max(most, max(m0, m1));
+      least = min(least, min(m0 - 1u, m1 - 1u));
+    }
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      add_product(dot, w[h], w[2 + h]);
+      add_product(na, w[h], w[h]);
+      add_product(nc, w[2 + h], w[2 + h]);
+    }
+  }
+  most = __reduce_max_sync(0xffffffffu, most);
+  least = __reduce_min_sync(0xffffffffu, least);
+  if (most >= (179u << 23) || least < (76u << 23) - 1u) {
+    sums_fp64(a, c, D, lane, s);
+    return;
+  }
+  // (dot, |a|^2) and (|c|^2, 0): the halves of each, then the lanes
+  auto low = [](unsigned long long x, unsigned long long y) { return (x & 0xFFFFFFFFull) | (y << 32); };
+  auto high = [](unsigned long long x, unsigned long long y) { return (x >> 32) | (y & 0xFFFFFFFF00000000ull); };
+  F32x3 u{low(dot.s, na.s), low(dot.c, na.c), low(dot.d, na.d)}, w{low(nc.s, 0), low(nc.c, 0), low(nc.d, 0)};
+  add_sum(u, F32x3{high(dot.s, na.s), high(dot.c, na.c), high(dot.d, na.d)});
+  add_sum(w, F32x3{high(nc.s, 0), high(nc.c, 0), high(nc.d, 0)});
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    auto other = [&](unsigned long long x) { return __shfl_xor_sync(0xffffffffu, x, o); };
+    auto first = [&](unsigned long long x) { return (unsigned long long)__shfl_xor_sync(0xffffffffu, (uint32_t)x, o); };
+    add_sum(u, F32x3{other(u.s), other(u.c), other(u.d)});
+    add_sum(w, F32x3{first(w.s), first(w.c), first(w.d)});
+  }
+  s.v[0] = (long long)low(u.s, u.c);
+  s.v[1] = (long long)high(u.s, u.c);
+  s.v[2] = (long long)low(w.s, w.c);
+  s.e[0] = (int)(uint32_t)u.d;
+  s.e[1] = (int)(u.d >> 32);
+  s.e[2] = (int)(uint32_t)w.d;
+  s.kind = SUMS_F32X3;
 }
 
 // Exact sums of a bf16 token of which each lane has NCH 16-byte chunks of
@@ -184,6 +282,7 @@ __device__ __forceinline__ void sums_bf16(const uint4* sa, const uint4* sc, cons
     warp_sum64(v0, -(ka + kc), s.v[0], s.e[0]);
     warp_sum64(v1, -2 * ka, s.v[1], s.e[1]);
     warp_sum64(v2, -2 * kc, s.v[2], s.e[2]);
+    s.kind = SUMS_INT;
     return;
   }
   bool inexact = ema == 255 || emc == 255;  // Inf or NaN present
@@ -218,6 +317,7 @@ __device__ __forceinline__ void sums_bf16(const uint4* sa, const uint4* sc, cons
   warp_sum64(v0, bd - 268, s.v[0], s.e[0]);
   warp_sum64(v1, ba - 268, s.v[1], s.e[1]);
   warp_sum64(v2, bc - 268, s.v[2], s.e[2]);
+  s.kind = SUMS_INT;
 }
 
 constexpr int kSelThreads = 256;
@@ -234,8 +334,8 @@ __device__ __forceinline__ void cp_async_wait() {
 }
 
 // One cluster per row r (blockIdx.x / cluster size). T: element type; NCH > 0:
-// bf16 vectors of at most 256 NCH elements; NCH == 0: fp64 sums streamed from
-// memory (fp32, and wider bf16 vectors). N == 0 only moves the current vectors
+// bf16 vectors of at most 256 NCH elements; NCH == 0: vectors streamed from
+// memory (fp32 in triples of floats, wider bf16 vectors in fp64). N == 0 only moves the current vectors
 // into the cache.
 //
 // With NCH > 0 every lane copies its chunks of the warp's next token to shared
@@ -312,7 +412,11 @@ __global__ void __launch_bounds__(kSelThreads, NCH <= 3 ? 4 : 2)
           if (i < D) *reinterpret_cast<uint4*>(c + i) = sa[32 * j];
         }
       } else {
-        if (need_s) sums_fp64(a, c, D, lane, s);
+        if constexpr (sizeof(T) == 4) {
+          if (need_s) sums_f32(a, c, D, lane, s);
+        } else {
+          if (need_s) sums_fp64(a, c, D, lane, s);
+        }
         for (int i = lane * V; i < D; i += 32 * V)
           *reinterpret_cast<uint4*>(c + i) = *reinterpret_cast<const uint4*>(a + i);
       }

@@ -163,6 +163,36 @@ def test_select_tokens_fixed_point_span(D, octaves, rows, T):
     assert torch.equal(g_ref, g_cur)
 
 
+@pytest.mark.parametrize("rows,T,D", [(1, 9, 8), (2, 333, 256), (21, 65, 768), (3, 130, 1288), (1, 700, 1280)])
+def test_select_tokens_fp32_ranges(rows, T, D):
+    """fp32 sums in triples of floats, and the fp64 sums of vectors whose products
+    leave the floats' range: magnitudes on both sides of 2^52 and 2^-51, zeros, Inf
+    and NaN. The similarities are random, so that their gaps exceed the roundings."""
+    torch = torch_cuda()
+    rng = np.random.default_rng(rows + T + D)
+    cur, ref = rng.standard_normal((2, rows, T, D))
+    ref += 0.5 * cur
+    for t, x, y in [(0, 2.0**51, 1.0), (1, 2.0**54, 2.0**-54), (2, 2.0**-49, 2.0**-48), (3, 2.0**-60, 1.0)]:
+        cur[:, t] *= x
+        ref[:, t] *= y
+    cur[:, 4, ::2] = 0.0
+    cur[:, 5] = 0.0
+    cur[:, 6, :] *= np.exp2(rng.integers(-40, 41, D))
+    cur[:, 7, D // 2] = np.inf
+    ref[:, 8, D - 1] = np.nan
+    cur, ref = cur.astype(np.float32), ref.astype(np.float32)
+    g_cur, g_ref = dev(cur), dev(ref)
+    N = max(1, T // 3)
+    idx = torch.full((rows, N), -1, dtype=torch.int32, device="cuda")
+    lm.lazymar_select_tokens(DT["fp32"], g_cur, g_ref, rows, T, D, N, idx)
+    sync()
+    got = idx.cpu().numpy()
+    with np.errstate(invalid="ignore", over="ignore"):
+        for r in range(rows):
+            assert got[r].tolist() == O.select_compute(O.cosine_similarity(cur[r], ref[r]), N).tolist(), "row %d" % r
+    assert torch.equal(g_ref.view(torch.int32), g_cur.view(torch.int32))
+
+
 def test_select_tokens_fp32_near_ties():
     """fp32 similarities are fp64 sums rounded at every addition, in the
     kernel's order on the GPU and in numpy's on the CPU, so mathematically
