@@ -6,7 +6,7 @@
 // bf16: attention_tc_kernel and attention_tm_kernel, tcgen05 tensor cores with
 // the accumulators in tensor memory and Q/K/V tiles staged by TMA, for heads of
 // width 64 (MAR-B, MAR-L) and 80 (MAR-H); the latter keeps the probabilities in
-// tensor memory too and serves the larger grids.
+// tensor memory too and serves the grids where that saves a wave of CTAs.
 //
 // f32: one warp per query on CUDA cores (fp32 configuration).
 #include <cuda.h>

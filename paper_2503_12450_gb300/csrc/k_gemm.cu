@@ -6,12 +6,14 @@
 // tiles with TMA (128B swizzle) into a ring of shared-memory stages, warp 1
 // issues tcgen05.mma (128 x BN x 16, fp32 accumulators in tensor memory,
 // double-buffered so the epilogue of one tile overlaps the main loop of the
-// next) and eight epilogue warps drain the accumulators with tcgen05.ld and
+// next) and 8 to 16 epilogue warps drain the accumulators with tcgen05.ld and
 // apply the fused epilogue: bias, GELU, fp32 residual add, or the Q/K/V split
-// with the K/V rows scattered into the token cache (row_map).
+// with the K/V rows scattered into the token cache (row_map). Few rows take
+// tiles of 64 rows.
 //
-// f32: a 64x64 register-tiled CUDA-core kernel with the same epilogues (the
-// tensor cores have no fp32 kind; this serves the fp32 configuration).
+// f32: CUDA-core kernels with the same epilogues (the tensor cores have no fp32
+// kind; these serve the fp32 configuration): small tiles with K split over the
+// warps, and for many rows a 64 x 64 register-tiled kernel.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
