@@ -1077,7 +1077,10 @@ static int choose_bn(const Ctx& c, int dtype, int M, int N, const GemmEpi& epi, 
         bn = kPair + width;
       }
     };
-    consider(256, resid_half ? 219 : 236);
+    // short K with GELU: the epilogue takes a larger part of a round (fc1 at width
+    // 768, pairs against single CTAs (us): M = 5632 22.9 : 21.7, 6144 24.5 : 23.4,
+    // 7680 29.0 : 28.2, but 12800 43.6 : 45.0)
+    consider(256, resid_half ? 219 : epi.mode == LAZYMAR_EPI_GELU && K < 1024 ? 243 : 236);
     if (resid_half) consider(192, 186);
   }
   // Few rows: 64 x 64 tiles while they fit in one round. Measured, 128 x 64 tiles ->
