@@ -71,9 +71,9 @@ __device__ __forceinline__ double sim_value(const SimSums& s) {
 
 // Sum of v * 2^e over the warp's lanes as an integer times a power of two
 // that rounds to the same double as the exact sum. Three 22-, 22- and 20-bit
-// pieces go through the warp's integer reduction; a total beyond 62 bits is
-// shifted right by 4 with its lost bits kept as a sticky lowest bit, far below
-// the 53 that a double holds.
+// pieces go through the warp's integer reduction. A total, below 2^68 in
+// magnitude, that has reached 2^62 is shifted right by 6 with its lost bits kept as a
+// sticky lowest bit: at least 56 bits are left, of which a double holds 53.
 __device__ __forceinline__ void warp_sum64(long long v, int e, long long& out_v, int& out_e) {
   const unsigned p0 = __reduce_add_sync(0xffffffffu, (unsigned)(v & 0x3FFFFF));
   const unsigned p1 = __reduce_add_sync(0xffffffffu, (unsigned)((v >> 22) & 0x3FFFFF));
@@ -81,8 +81,8 @@ __device__ __forceinline__ void warp_sum64(long long v, int e, long long& out_v,
   const long long hi = (long long)p2 * (1ll << 22) + (long long)p1 + (long long)(p0 >> 22);  // total = hi 2^22 + lo
   const long long lo = (long long)(p0 & 0x3FFFFFu);
   const bool wide = hi >= (1ll << 40) || hi < -(1ll << 40);
-  out_v = wide ? (hi * (1ll << 18)) | (lo >> 4) | ((lo & 15) != 0) : hi * (1ll << 22) + lo;
-  out_e = wide ? e + 4 : e;
+  out_v = wide ? (hi * (1ll << 16)) | (lo >> 6) | ((lo & 63) != 0) : hi * (1ll << 22) + lo;
+  out_e = wide ? e + 6 : e;
 }
 
 // fp64 sums of one token in lane-strided order; no copy.

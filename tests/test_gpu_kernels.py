@@ -163,6 +163,31 @@ def test_select_tokens_fixed_point_span(D, octaves, rows, T):
     assert torch.equal(g_ref, g_cur)
 
 
+@pytest.mark.parametrize("magnitude", [1.5, 1.75, 1.9921875, None])
+@pytest.mark.parametrize("rows,T,D", [(2, 120, 256), (1, 97, 512), (2, 120, 768), (1, 97, 1024), (1, 97, 1280),
+                                      (1, 97, 1272)])
+def test_select_tokens_nearly_constant_magnitudes(rows, T, D, magnitude):
+    """Vectors whose elements are all of (nearly) the largest magnitude: the
+    fixed-point sums of 32 lanes come close to 2^68, in the norms, and in dot
+    products of both signs (cur = ref, cur = -ref, and some signs flipped).
+    None: magnitudes of [1.5, 2), 1.9921875 is the largest bf16 below 2."""
+    torch = torch_cuda()
+    rng = np.random.default_rng(D + T)
+    mag = magnitude or rng.uniform(1.5, 1.99, (rows, T, D))
+    ref = mag * rng.choice([-1.0, 1.0], (rows, T, D)) * np.exp2(rng.choice([-3, 0, 5], (rows, T, 1)))
+    flips = rng.choice([0.0, 0.02, 0.5, 0.98, 1.0], (rows, T, 1))
+    cur = np.where(rng.random((rows, T, D)) < flips, -ref, ref)
+    cur, ref = synth.round_bf16(cur.astype(np.float32)), synth.round_bf16(ref.astype(np.float32))
+    g_cur, g_ref = dev(cur, "bf16"), dev(ref, "bf16")
+    N = T // 2
+    idx = torch.full((rows, N), -1, dtype=torch.int32, device="cuda")
+    lm.lazymar_select_tokens(DT["bf16"], g_cur, g_ref, rows, T, D, N, idx)
+    sync()
+    got = idx.cpu().numpy()
+    for r in range(rows):
+        assert got[r].tolist() == O.select_compute(O.cosine_similarity(cur[r], ref[r]), N).tolist(), "row %d" % r
+
+
 @pytest.mark.parametrize("rows,T,D", [(1, 9, 8), (2, 333, 256), (21, 65, 768), (3, 130, 1288), (1, 700, 1280)])
 def test_select_tokens_fp32_ranges(rows, T, D):
     """fp32 sums in triples of floats, and the fp64 sums of vectors whose products
