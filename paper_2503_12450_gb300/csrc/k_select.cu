@@ -493,21 +493,29 @@ __global__ void __launch_bounds__(kSelThreads, NCH <= 3 ? 4 : 2)
   }
 }
 
+// Dynamic shared memory of a CTA that ranks (N > 0).
+template <int NCH>
+static size_t select_smem(int n_tok, int ncta) {
+  const size_t per = (size_t)((n_tok + ncta - 1) / ncta);
+  return kSelRing<NCH> + (size_t)n_tok * sizeof(unsigned long long) +
+         (per < kSelThreads ? per : (size_t)kSelThreads) * sizeof(SimSums) + per;
+}
+
 // CTAs per row. 8 (the portable limit) keeps a row's tokens on 64 warps; with
 // few rows, clusters of 16 spread them over twice as many SMs.
+constexpr int kSelMaxTokens = 16384;  // of a row, in every entry point
 template <typename T, int NCH>
 static cudaError_t launch_select_t(const Ctx& c, const void* cur, void* cache, int rows, int n_tok, int D, int span,
                                    int N, int* idx, int* row_map, int rule, const uint8_t* prio,
                                    const uint32_t* keys) {
   auto kernel = select_kernel<T, NCH>;
   const int ncta = rows * 16 <= c.num_sms ? 16 : 8;
-  const size_t per = (size_t)((n_tok + ncta - 1) / ncta);
-  const size_t smem =
-      kSelRing<NCH> + (N > 0 ? (size_t)n_tok * sizeof(unsigned long long) +
-                                   (per < kSelThreads ? per : (size_t)kSelThreads) * sizeof(SimSums) + per
-                             : 0);
+  const size_t smem = N > 0 ? select_smem<NCH>(n_tok, ncta) : kSelRing<NCH>;
   if (smem > 40 * 1024) {
-    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    // always the largest size: the attribute is the process's, and another host
+    // thread may be about to launch the kernel for more tokens
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               (int)select_smem<NCH>(kSelMaxTokens, 8));
     if (e != cudaSuccess) return e;
   }
   static int attr_set[64] = {};

@@ -1,5 +1,7 @@
 """Kernel-level parity: each CUDA kernel, called through the C ABI, against
 the CPU oracle on the same seeded inputs."""
+import threading
+
 import numpy as np
 import pytest
 
@@ -216,6 +218,56 @@ def test_select_tokens_fp32_ranges(rows, T, D):
         for r in range(rows):
             assert got[r].tolist() == O.select_compute(O.cosine_similarity(cur[r], ref[r]), N).tolist(), "row %d" % r
     assert torch.equal(g_ref.view(torch.int32), g_cur.view(torch.int32))
+
+
+def _in_threads(jobs):
+    """Runs the jobs on host threads of their own, each on a CUDA stream of its
+    own, at the same time; the first error any of them raised, or None."""
+    torch = torch_cuda()
+    errors, start = [], threading.Barrier(len(jobs))
+
+    def go(job):
+        try:
+            stream = torch.cuda.Stream()
+            start.wait()
+            with torch.cuda.stream(stream):
+                job()
+            stream.synchronize()
+        except Exception as e:  # raised again by the caller
+            errors.append(e)
+
+    threads = [threading.Thread(target=go, args=(j,)) for j in jobs]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    return errors[0] if errors else None
+
+
+def test_select_tokens_from_two_threads():
+    """Selections of 320 and of 1088 tokens, which take different amounts of
+    shared memory in one kernel, called from two host threads at once."""
+    torch = torch_cuda()
+    jobs, results = [], []
+    for T, N in ((320, 50), (1088, 272)):
+        cur, ref = (dev(x, "bf16") for x in synth.similarity_inputs(4, T, 768, seed=T, dtype="bf16"))
+        first, idx = (torch.empty((4, N), dtype=torch.int32, device="cuda") for _ in range(2))
+        cache = ref.clone()
+        lm.lazymar_select_tokens(DT["bf16"], cur, cache, 4, T, 768, N, first)
+        sync()
+
+        def job(cur=cur, ref=ref, cache=cache, T=T, N=N, idx=idx):
+            for _ in range(3000):
+                lm.lazymar_select_tokens(DT["bf16"], cur, cache, 4, T, 768, N, idx)
+            cache.copy_(ref)
+            lm.lazymar_select_tokens(DT["bf16"], cur, cache, 4, T, 768, N, idx)
+
+        jobs.append(job)
+        results.append((idx, first))
+    error = _in_threads(jobs)
+    assert error is None, error
+    sync()
+    assert all(torch.equal(idx, first) for idx, first in results)
 
 
 def test_select_tokens_fp32_near_ties():
