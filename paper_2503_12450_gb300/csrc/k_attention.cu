@@ -531,13 +531,23 @@ __global__ void __launch_bounds__(at2::Cfg<DH, QR>::THREADS, at2::Cfg<DH, QR>::M
 // the tensor pipe as much as S (and P's way there a proxy fence per chunk).
 // Measured, against attention_tc_kernel (us): 64 rows x 12 heads x 320 x 320 of
 // width 64 45.2 -> 39.6, 128 x 16 109 -> 93.4, 16 x 16 x 1088 x 1088 118 -> 101; of
-// width 80, 64 x 16 x 320 x 320 85.9 -> 67.4, 50 queries 32.2 -> 26.7.
+// width 80, 64 x 16 x 320 x 320 85.9 -> 68.8, 50 queries 28.8 -> 24.6.
 //
 // The running max m is raised only when a row's chunk max exceeds it by more
 // than 8 (log2 units): the final O / l is the same for any m that is at least
 // every key's score - 8 and P stays below 2^8, while O in tensor memory is
 // rescaled only on those (rare) raises. K and V have two-stage rings: K(c + 2)
 // refills once S(c) has been read, V(c + 2) once P(c) V(c) is complete.
+//
+// The probability of the key that sets m is 1, which bf16 holds exactly, so the
+// error of P falls with the number of keys m is first taken over. Chunks of 48
+// keys would give up some of that against attention_tc_kernel's 64 (error of the
+// results, 64 rows x 16 heads x 320 x 320 2.304e-3 against 2.296e-3; 65 x 65 2.155e-3
+// against 2.114e-3), so S(0) is 64 keys wide, 16 of them from K(1), which follows
+// K(0) in shared memory and is loaded in two parts so that S(0) waits for no more;
+// their scores, in columns of O that P(0) V(0) writes later, join the first maximum
+// only. The probabilities are then those of attention_tc_kernel, for 2 % of the time
+// (64 x 16 x 320 x 320 67.1 us without, 68.8 with; 70 with K(1) loaded whole).
 //
 // A head of width 80: Q and K are a 64-column part (128-byte swizzle, as for
 // width 64) and a 16-column remainder (32-byte swizzle: rows of 32 bytes, 8-row
@@ -599,8 +609,9 @@ template <int DH>
 __global__ void __launch_bounds__(at4::THREADS, at4::Cfg<DH>::MIN_BLOCKS)
     attention_tm_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                         const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmQ2,
-                        const __grid_constant__ CUtensorMap tmK2, bf16* o, int n_q, int T, int D,
-                        float scale_log2, unsigned* err) {
+                        const __grid_constant__ CUtensorMap tmK2, const __grid_constant__ CUtensorMap tmKx,
+                        const __grid_constant__ CUtensorMap tmKx2, bf16* o, int n_q, int T, int D, float scale_log2,
+                        unsigned* err) {
   using namespace at4;
   using C = Cfg<DH>;
   constexpr bool TAIL = C::TAIL;
@@ -624,6 +635,7 @@ __global__ void __launch_bounds__(at4::THREADS, at4::Cfg<DH>::MIN_BLOCKS)
   // S, P and O are never read back (matrix rows are independent).
   const int n_valid = min(QT, n_q - qt * QT);
   const int n_act = (n_valid + 31) / 32;
+  const bool wide0 = KC < 64 && nck > 1;  // S(0) takes 64 keys
 
   if (tid == 0) {
     for (int i = 0; i < N_BARS; ++i) mbar_init(&bars[i], i == B_P_FULL ? (uint32_t)n_act : 1u);
@@ -636,6 +648,8 @@ __global__ void __launch_bounds__(at4::THREADS, at4::Cfg<DH>::MIN_BLOCKS)
     if (TAIL) {
       prefetch_tmap(&tmQ2);
       prefetch_tmap(&tmK2);
+      prefetch_tmap(&tmKx);
+      prefetch_tmap(&tmKx2);
     }
   }
   if (warp == 4) {
@@ -658,6 +672,11 @@ __global__ void __launch_bounds__(at4::THREADS, at4::Cfg<DH>::MIN_BLOCKS)
         tma_load_2d(&tmK, &bars[B_K + st], sK + st * C::K_BYTES, col, kv0 + c * KC);
         if (TAIL) tma_load_2d(&tmK2, &bars[B_K + st], sK2 + st * C::K2_BYTES, col + 64, kv0 + c * KC);
       };
+      // 16 keys from key k (of the first two chunks) on
+      auto load_k16 = [&](uint64_t* bar, int k) {
+        tma_load_2d(&tmKx, bar, sK + k * 128, col, kv0 + k);
+        tma_load_2d(&tmKx2, bar, sK2 + k * 32, col + 64, kv0 + k);
+      };
       auto load_v = [&](int c) {
         const int st = c & 1;
         mbar_arrive_expect_tx(&bars[B_V + st], C::V_TX);
@@ -672,20 +691,32 @@ __global__ void __launch_bounds__(at4::THREADS, at4::Cfg<DH>::MIN_BLOCKS)
       mbar_arrive_expect_tx(&bars[B_Q], C::Q_TX);
       tma_load_2d(&tmQ, &bars[B_Q], sQ, col, q0);
       if (TAIL) tma_load_2d(&tmQ2, &bars[B_Q], sQ2, col + 64, q0);
-      load_k(0);
-      load_v(0);
-      if (nck > 1) {
-        load_k(1);
+      if (wide0) {  // K(0) and the first 16 keys of K(1), then the other 32
+        mbar_arrive_expect_tx(&bars[B_K], C::K_TX + 16 * 160);
+        tma_load_2d(&tmK, &bars[B_K], sK, col, kv0);
+        tma_load_2d(&tmK2, &bars[B_K], sK2, col + 64, kv0);
+        load_k16(&bars[B_K], KC);
+        load_v(0);
+        mbar_arrive_expect_tx(&bars[B_K + 1], C::K_TX - 16 * 160);
+        load_k16(&bars[B_K + 1], KC + 16);
+        load_k16(&bars[B_K + 1], KC + 32);
         load_v(1);
+      } else {
+        load_k(0);
+        load_v(0);
+        if (nck > 1) {
+          load_k(1);
+          load_v(1);
+        }
       }
       const uint64_t qd = sw128_desc(smem_u32(sQ));
       auto issue_s = [&](int c) {
         const uint64_t kd = sw128_desc(smem_u32(sK + (c & 1) * C::K_BYTES));
+        const uint32_t id = wide0 && c == 0 ? idesc(64) : idesc(KC);
 #pragma unroll
-        for (int k = 0; k < 4; ++k) umma_bf16(tmem, qd + 2 * k, kd + 2 * k, idesc(KC), k != 0 ? 1u : 0u);
+        for (int k = 0; k < 4; ++k) umma_bf16(tmem, qd + 2 * k, kd + 2 * k, id, k != 0 ? 1u : 0u);
         if (TAIL)
-          umma_bf16(tmem, sw32_desc(smem_u32(sQ2), 256), sw32_desc(smem_u32(sK2 + (c & 1) * C::K2_BYTES), 256),
-                    idesc(KC), 1u);
+          umma_bf16(tmem, sw32_desc(smem_u32(sQ2), 256), sw32_desc(smem_u32(sK2 + (c & 1) * C::K2_BYTES), 256), id, 1u);
         umma_commit(&bars[B_S_FULL]);
       };
       bool ok = mbar_wait<false>(&bars[B_Q], 0, abort_flag, err) && mbar_wait<false>(&bars[B_K], 0, abort_flag, err);
@@ -726,6 +757,17 @@ __global__ void __launch_bounds__(at4::THREADS, at4::Cfg<DH>::MIN_BLOCKS)
     const uint32_t t_lane = (uint32_t)(warp * 32) << 16;
     float m_run = -FLT_MAX, l_run = 0.f;
     bool ok = true;
+    if (wide0 && __all_sync(0xffffffffu, mbar_wait<false>(&bars[B_S_FULL], 0, abort_flag, err))) {
+      tc_fence_after();
+      uint32_t rx[16];
+      tmem_ld16(tmem + t_lane + KC, rx);
+      tmem_wait_ld_regs(rx);
+      float mx[2] = {-FLT_MAX, -FLT_MAX};
+#pragma unroll
+      for (int i = 0; i < 16; ++i)
+        if (KC + i < T) mx[i & 1] = fmaxf(mx[i & 1], __uint_as_float(rx[i]));
+      m_run = fmaxf(mx[0], mx[1]) * scale_log2;
+    }
     for (int c = 0; c < nck; ++c) {
       ok = __all_sync(0xffffffffu, mbar_wait<false>(&bars[B_S_FULL], (uint32_t)c & 1u, abort_flag, err));
       if (!ok) break;
@@ -773,7 +815,7 @@ __global__ void __launch_bounds__(at4::THREADS, at4::Cfg<DH>::MIN_BLOCKS)
       float alpha = 1.f;
       bool raise = false;
       if (c == 0) {
-        m_run = mloc;
+        m_run = fmaxf(m_run, mloc);
       } else if (mloc > m_run + RESCALE_THRESHOLD) {
         raise = true;
         alpha = exp2_approx(m_run - mloc);
@@ -960,7 +1002,7 @@ static cudaError_t launch_attn_tm(const Ctx& c, const void* q, const void* k, co
   if (T < 1) return cudaErrorInvalidValue;  // the kernel's final wait needs at least one key chunk
   const int D = heads * DH;
   const uint64_t pitch = (uint64_t)D * 2;
-  CUtensorMap mq, mk, mv, mq2, mk2;
+  CUtensorMap mq, mk, mv, mq2, mk2, mkx, mkx2;
   if (!make_tmap_bf16(&mq, q, D, (uint64_t)rows * n_q, pitch, 64, at4::QT, CU_TENSOR_MAP_SWIZZLE_128B) ||
       !make_tmap_bf16(&mk, k, D, (uint64_t)rows * T, pitch, 64, C::KC, CU_TENSOR_MAP_SWIZZLE_128B))
     return cudaErrorInvalidValue;
@@ -969,13 +1011,15 @@ static cudaError_t launch_attn_tm(const Ctx& c, const void* q, const void* k, co
     // multiple of 16 bytes as TMA requires
     if (!make_tmap_bf16(&mv, v, D, (uint64_t)rows * T, pitch, 16, C::KC, CU_TENSOR_MAP_SWIZZLE_32B) ||
         !make_tmap_bf16(&mq2, q, D, (uint64_t)rows * n_q, pitch, 16, at4::QT, CU_TENSOR_MAP_SWIZZLE_32B) ||
-        !make_tmap_bf16(&mk2, k, D, (uint64_t)rows * T, pitch, 16, C::KC, CU_TENSOR_MAP_SWIZZLE_32B))
+        !make_tmap_bf16(&mk2, k, D, (uint64_t)rows * T, pitch, 16, C::KC, CU_TENSOR_MAP_SWIZZLE_32B) ||
+        !make_tmap_bf16(&mkx, k, D, (uint64_t)rows * T, pitch, 64, 16, CU_TENSOR_MAP_SWIZZLE_128B) ||
+        !make_tmap_bf16(&mkx2, k, D, (uint64_t)rows * T, pitch, 16, 16, CU_TENSOR_MAP_SWIZZLE_32B))
       return cudaErrorInvalidValue;
   } else {
     if (!make_tmap_bf16(&mv, v, D, (uint64_t)rows * T, pitch, 64, C::KC, CU_TENSOR_MAP_SWIZZLE_128B))
       return cudaErrorInvalidValue;
     mq2 = mq;
-    mk2 = mk;
+    mk2 = mkx = mkx2 = mk;
   }
   static int attr_set[64] = {};
   int dev = 0;
@@ -994,7 +1038,7 @@ static cudaError_t launch_attn_tm(const Ctx& c, const void* q, const void* k, co
   const size_t smem =
       ctas <= (long long)C::MIN_BLOCKS * c.num_sms ? spread_smem(C::SMEM, C::MIN_BLOCKS, ctas, c.num_sms) : C::SMEM;
   return launch_pdl(attention_tm_kernel<DH>, grid, dim3(at4::THREADS), smem, c.stream, mq, mk, mv, mq2,
-                    mk2, static_cast<bf16*>(o), n_q, T, D, scale_log2, c.err);
+                    mk2, mkx, mkx2, static_cast<bf16*>(o), n_q, T, D, scale_log2, c.err);
 }
 
 cudaError_t launch_attention(const Ctx& c, int dtype, const void* q, const void* k, const void* v, void* o,
@@ -1020,10 +1064,12 @@ cudaError_t launch_attention(const Ctx& c, int dtype, const void* q, const void*
   // the waves are as many. Measured, latter against former (us): width 64, 16 heads,
   // 300 queries, 1088 keys: 432 CTAs 23.4 : 25.0, 576 37.4 : 28.1, 912 44.8 : 50.8,
   // 1008 58.5 : 51.6, 1344 64.0 : 69.5, 1392 72.3 : 70.6, 2496 118.1 : 112.8; 320 keys:
-  // 480 15.7 : 11.7, 768 18.2 : 19.1, 1008 23.9 : 21.1. Width 80, 320 keys: 384 17.0 :
-  // 13.6, 624 23.3 : 22.5, 912 27.2 : 26.8, 1200 34.5 : 29.0; two waves against three
-  // lose with many keys, in whose short last wave an SM has one or two CTAs: 704 CTAs
-  // of 500 keys 34.1 : 33.4, 850 51.4 : 49.1, 1088 59.7 : 62.3.
+  // 480 15.7 : 11.7, 768 18.2 : 19.1, 1008 23.9 : 21.1. Width 80, 320 keys: 320 15.7 :
+  // 13.6, 608 17.7 : 15.3, 928 31.9 : 27.1, 1216 38.2 : 31.7. Two waves against three, where
+  // an SM has one or two CTAs in the short last one, pay off at width 80 only with a tenth
+  // fewer chunks in all, of 48 keys against 64: 912 CTAs of 65 keys 16.7 : 14.2, 200 23.5 : 21.5,
+  // 850 57.2 : 55.5, but 128 keys 16.2 : 16.6, 320 26.7 : 26.8 (with 50 queries 23.2 : 23.8), 700
+  // 47.9 : 48.0; and not with many keys (1088 65.8 : 67.6).
   // With at most 64 queries (of width 64) attention_tc_kernel's CTAs hold 64 rows and
   // four of them fit too (two softmax warps each): 64 rows x 12 heads x 50 x 320
   // 13.9 against 14.4 us with 128 rows and 15.7 in attention_tm_kernel, 64 x 8
@@ -1032,7 +1078,9 @@ cudaError_t launch_attention(const Ctx& c, int dtype, const void* q, const void*
   const long long ctas = (long long)((n_q + 127) / 128) * heads * rows;
   const long long tm_slots = 4LL * c.num_sms, tc_slots = (dh == 64 ? 3LL : 2LL) * c.num_sms;
   const long long tm_waves = (ctas + tm_slots - 1) / tm_slots, tc_waves = (ctas + tc_slots - 1) / tc_slots;
-  const bool tm = tm_waves < tc_waves && !(dh == 80 && tm_waves == 2 && tc_waves == 3 && T >= 1024);
+  bool tm = tm_waves < tc_waves;
+  if (dh == 80 && tm_waves == 2 && tc_waves == 3)
+    tm = T < 1024 && 10 * tm_waves * ((T + 47) / 48) <= 9 * tc_waves * ((T + 63) / 64);
   if (dh == 64)
     return tm ? launch_attn_tm<64>(c, q, k, v, o, rows, n_q, T, heads)
               : launch_attn_tc<64, 128>(c, q, k, v, o, rows, n_q, T, heads);

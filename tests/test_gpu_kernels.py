@@ -725,6 +725,29 @@ def test_attention_large_grids(rows, n_q, T, heads, dh, q_std):
     assert max_rel(got, host(ref)) < 1e-2
 
 
+@pytest.mark.parametrize("T", [48, 49, 63, 64, 65, 97, 200, 320])
+@pytest.mark.parametrize("heads,dh", [(16, 80), (16, 64)])
+def test_attention_large_grid_equals_small(T, heads, dh):
+    """A row computed in a large grid (attention_tm_kernel) and by itself
+    (attention_tc_kernel): the probabilities are the same bf16 values, because
+    both kernels take the first running maximum over 64 keys; only the fp32 row
+    sums are in another order, 2^-24 against the 2^-9 of the results, so that
+    about 1 result in 2^14 may fall on the other side of a rounding."""
+    torch = torch_cuda()
+    rows, n_q, D = 64, 65, heads * dh
+    q = dev(synth.tensor((rows, n_q, D), 51, dtype="bf16"), "bf16")
+    k = dev(synth.tensor((rows, T, D), 52, dtype="bf16"), "bf16")
+    v = dev(synth.tensor((rows, T, D), 53, dtype="bf16"), "bf16")
+    o = empty((rows, n_q, D), "bf16")
+    lm.lazymar_attention(DT["bf16"], q, k, v, o, rows, n_q, T, heads, dh)
+    sync()
+    for r in (0, rows // 2, rows - 1):
+        one = empty((1, n_q, D), "bf16")
+        lm.lazymar_attention(DT["bf16"], q[r:r + 1], k[r:r + 1], v[r:r + 1], one, 1, n_q, T, heads, dh)
+        sync()
+        assert (one[0] != o[r]).sum().item() <= n_q * D * 2.0 ** -9, "row %d" % r
+
+
 @pytest.mark.parametrize("rows,n_q,T,q_std", [
     (1, 1, 65, 1.0), (2, 31, 64, 1.0), (10, 33, 320, 1.0), (24, 63, 129, 1.0), (32, 64, 1, 1.0),
     (40, 64, 320, 1.0), (64, 32, 63, 1.0), (40, 50, 1088, 4.0),     # four CTAs per SM
