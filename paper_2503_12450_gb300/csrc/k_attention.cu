@@ -28,6 +28,7 @@ bool make_tmap_bf16(CUtensorMap* m, const void* base, uint64_t inner, uint64_t o
 // fp32 configuration's sizes (80 keys, 20 or 80 queries): 2 rows x 20 queries
 // 18.6 -> 5.6 us, 2 x 80 27.8 -> 6.5, 16 x 80 173 -> 19.9, against lanes that each
 // read a key row of their own from global memory four bytes at a time.
+constexpr int F32_SMEM_MAX = 227 * 1024;  // of a CTA
 __host__ __device__ inline int att32_chunk(int T) { return T >= 128 ? 128 : (T + 31) & ~31; }
 template <int DH>  // head width, 0: the argument's
 __global__ void __launch_bounds__(128) attention_f32_kernel(const float* __restrict__ q, const float* __restrict__ k,
@@ -1050,7 +1051,10 @@ cudaError_t launch_attention(const Ctx& c, int dtype, const void* q, const void*
         ((T <= (int)kc ? 2 : 1) * kc * (dq + 4) + 4 * dq + (size_t)4 * ((T + 3) & ~3)) * sizeof(float);
     auto kernel = dh == 64 ? attention_f32_kernel<64> : attention_f32_kernel<0>;
     if (smem > 48 * 1024) {
-      cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      // always the largest size there is: the attribute is the process's, and another
+      // host thread may be about to launch the kernel for more keys
+      const cudaError_t e =
+          cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, F32_SMEM_MAX);
       if (e != cudaSuccess) return e;
     }
     dim3 grid((n_q + 3) / 4, heads, rows);

@@ -555,6 +555,30 @@ def test_attention_fp32_chunks(rows, n_q, T, heads, dh):
     assert max_rel(host(o), ref) < 1e-5
 
 
+def test_attention_fp32_from_threads():
+    """fp32 attention over 80 and over 128 keys, which takes different amounts of
+    shared memory in one kernel, called from four host threads at once, for long
+    enough to fill their streams."""
+    torch = torch_cuda()
+    jobs, results = [], []
+    for T in (80, 128, 80, 128):
+        q, k, v = (dev(synth.tensor((32, n, 256), T + i)) for i, n in enumerate((80, T, T)))
+        first, o = empty((32, 80, 256)), empty((32, 80, 256))
+        lm.lazymar_attention(DT["fp32"], q, k, v, first, 32, 80, T, 4, 64)
+        sync()
+
+        def job(q=q, k=k, v=v, o=o, T=T):
+            for _ in range(4000):
+                lm.lazymar_attention(DT["fp32"], q, k, v, o, 32, 80, T, 4, 64)
+
+        jobs.append(job)
+        results.append((o, first))
+    error = _in_threads(jobs)
+    assert error is None, error
+    sync()
+    assert all(torch.equal(o, first) for o, first in results)
+
+
 # --------------------------------------------------------------------------
 # E4M3 Q/K/V projection (qkv_e4m3): weight quantization, LayerNorm to E4M3,
 # the kind::f8f6f4 GEMM
