@@ -20,8 +20,9 @@ namespace lm {
 bool make_tmap_bf16(CUtensorMap* m, const void* base, uint64_t inner, uint64_t outer, uint64_t pitch_bytes,
                     uint32_t box_inner, uint32_t box_outer, CUtensorMapSwizzle swz);
 
-// fp32: one warp per query, four queries of one head per CTA, the scores of
-// all T keys in shared memory. Keys and values pass through shared memory in
+// fp32: one warp per query, NQ queries of one head per CTA, the scores of
+// all T keys in shared memory (four queries; two where the scores of four leave
+// no room for the keys, from 10177 keys at width 128 and 12289 at 64). Keys and values pass through shared memory in
 // chunks of up to 128 that the CTA loads as whole rows (float4, rows padded by
 // one float4 so that a lane reading its own key's row meets no bank conflict);
 // a sequence of one chunk has both in flight at once. Bound by latency at the
@@ -30,8 +31,8 @@ bool make_tmap_bf16(CUtensorMap* m, const void* base, uint64_t inner, uint64_t o
 // read a key row of their own from global memory four bytes at a time.
 constexpr int F32_SMEM_MAX = 227 * 1024;  // of a CTA
 __host__ __device__ inline int att32_chunk(int T) { return T >= 128 ? 128 : (T + 31) & ~31; }
-template <int DH>  // head width, 0: the argument's
-__global__ void __launch_bounds__(128) attention_f32_kernel(const float* __restrict__ q, const float* __restrict__ k,
+template <int DH, int NQ>  // DH: head width, 0: the argument's
+__global__ void __launch_bounds__(NQ * 32) attention_f32_kernel(const float* __restrict__ q, const float* __restrict__ k,
                                                             const float* __restrict__ v, float* __restrict__ o,
                                                             int n_q, int T, int D, int dh_arg, float scale) {
   extern __shared__ __align__(16) float sm[];
@@ -45,8 +46,8 @@ __global__ void __launch_bounds__(128) attention_f32_kernel(const float* __restr
   float* sk = sm;                                          // [KC][pitch] keys
   float* sv = one ? sk + KC * pitch : sk;                  // values: a buffer of their own for a single chunk
   float* qv = sm + (one ? 2 : 1) * KC * pitch + warp * dq; // this warp's query
-  float* sc = sm + (one ? 2 : 1) * KC * pitch + 4 * dq + (size_t)warp * Tp;
-  const int qi = blockIdx.x * 4 + warp, h = blockIdx.y, r = blockIdx.z;
+  float* sc = sm + (one ? 2 : 1) * KC * pitch + NQ * dq + (size_t)warp * Tp;
+  const int qi = blockIdx.x * NQ + warp, h = blockIdx.y, r = blockIdx.z;
   const bool act = qi < n_q;
   const bool vec = dh % 4 == 0;  // then rows and heads start on 16-byte boundaries
   auto stage = [&](float* dst, const float* src, int t0) {  // rows t0 .. t0 + KC - 1 of the head's keys or values
@@ -54,13 +55,13 @@ __global__ void __launch_bounds__(128) attention_f32_kernel(const float* __restr
     if (vec) {
       const int n4 = dq / 4;
 #pragma unroll 8
-      for (int i = tid; i < KC * n4; i += 128) {
+      for (int i = tid; i < KC * n4; i += NQ * 32) {
         const int t = i / n4, c = (i - t * n4) * 4;
         *reinterpret_cast<float4*>(dst + t * pitch + c) =
             t0 + t < T ? *reinterpret_cast<const float4*>(base + (size_t)(t0 + t) * D + c) : make_float4(0.f, 0.f, 0.f, 0.f);
       }
     } else {
-      for (int i = tid; i < KC * dq; i += 128) {
+      for (int i = tid; i < KC * dq; i += NQ * 32) {
         const int t = i / dq, c = i - t * dq;
         dst[t * pitch + c] = t0 + t < T && c < dh ? base[(size_t)(t0 + t) * D + c] : 0.f;
       }
@@ -1042,25 +1043,32 @@ static cudaError_t launch_attn_tm(const Ctx& c, const void* q, const void* k, co
                     mk2, mkx, mkx2, static_cast<bf16*>(o), n_q, T, D, scale_log2, c.err);
 }
 
+template <int NQ>
+static cudaError_t launch_attn_f32(const Ctx& c, const float* q, const float* k, const float* v, float* o, int rows,
+                                   int n_q, int T, int heads, int dh, size_t smem) {
+  auto kernel = dh == 64 ? attention_f32_kernel<64, NQ> : attention_f32_kernel<0, NQ>;
+  if (smem > 48 * 1024) {
+    // always the largest size there is: the attribute is the process's, and another
+    // host thread may be about to launch the kernel for more keys
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, F32_SMEM_MAX);
+    if (e != cudaSuccess) return e;
+  }
+  return launch_pdl(kernel, dim3((n_q + NQ - 1) / NQ, heads, rows), dim3(NQ * 32), smem, c.stream, q, k, v, o, n_q, T,
+                    heads * dh, dh, 1.0f / sqrtf((float)dh));
+}
+
 cudaError_t launch_attention(const Ctx& c, int dtype, const void* q, const void* k, const void* v, void* o,
                              int rows, int n_q, int T, int heads, int dh) {
   if (rows == 0 || n_q == 0) return cudaSuccess;
   if (dtype == LAZYMAR_F32) {
-    const size_t dq = (size_t)((dh + 3) & ~3), kc = (size_t)att32_chunk(T);
-    const size_t smem =
-        ((T <= (int)kc ? 2 : 1) * kc * (dq + 4) + 4 * dq + (size_t)4 * ((T + 3) & ~3)) * sizeof(float);
-    auto kernel = dh == 64 ? attention_f32_kernel<64> : attention_f32_kernel<0>;
-    if (smem > 48 * 1024) {
-      // always the largest size there is: the attribute is the process's, and another
-      // host thread may be about to launch the kernel for more keys
-      const cudaError_t e =
-          cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, F32_SMEM_MAX);
-      if (e != cudaSuccess) return e;
-    }
-    dim3 grid((n_q + 3) / 4, heads, rows);
-    return launch_pdl(kernel, grid, dim3(128), smem, c.stream, static_cast<const float*>(q),
-                      static_cast<const float*>(k), static_cast<const float*>(v), static_cast<float*>(o), n_q, T,
-                      heads * dh, dh, 1.0f / sqrtf((float)dh));
+    const size_t dq = (size_t)((dh + 3) & ~3), kc = (size_t)att32_chunk(T), tp = (size_t)((T + 3) & ~3);
+    const size_t kv = (T <= (int)kc ? 2 : 1) * kc * (dq + 4);
+    const size_t smem = (kv + 4 * (dq + tp)) * sizeof(float);
+    const float *fq = static_cast<const float*>(q), *fk = static_cast<const float*>(k), *fv = static_cast<const float*>(v);
+    if (smem > F32_SMEM_MAX)
+      return launch_attn_f32<2>(c, fq, fk, fv, static_cast<float*>(o), rows, n_q, T, heads, dh,
+                                (kv + 2 * (dq + tp)) * sizeof(float));
+    return launch_attn_f32<4>(c, fq, fk, fv, static_cast<float*>(o), rows, n_q, T, heads, dh, smem);
   }
   // attention_tm_kernel overlaps four CTAs of an SM, attention_tc_kernel, of which
   // three or (width 80) two fit, the chunks of one (it may issue S(c + 1) while P(c)

@@ -138,6 +138,18 @@ def test_embedding_of_many_pairs(batch, dtype, over):
     assert max_rel(z1g, z1) < TOL[dtype]
 
 
+@pytest.mark.parametrize("T,heads", [(12292, 2), (14400, 1)])
+def test_fp32_step_of_long_sequences(T, heads):
+    """fp32 attention of so many keys that the scores of four queries and a chunk
+    of keys do not fit in shared memory together: heads of 64 just above that
+    line, and of 128 well above it."""
+    r = Run("tiny", batch=1, depth=1, width=128, heads=heads, n_img=T - 16)
+    c = O.Cache(r.cfg, 1)
+    st = r.state(4000)
+    z, _ = O.full_step(r.cfg, r.W, c, st[0], st[1], r.labels, GAMMA)
+    assert max_rel(r.full(st)[0], z) < TOL["fp32"]
+
+
 def _valid_rule_selection(I, S, n, rule, prio, keys, margin=1e-6):
     """I is a valid choice of the n first tokens under the rule's order, with
     similarities allowed to differ from the oracle's S by `margin` (fp32)."""
