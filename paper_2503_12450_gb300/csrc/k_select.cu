@@ -347,8 +347,12 @@ __device__ __forceinline__ void cp_async_wait() {
 // the order-preserving key of S; MOST_SIMILAR (strategy IV) its complement,
 // i.e. S descending (NaN, as -inf, last); RANDOM (strategy III) the caller's
 // 32-bit random keys.
+
+// A CTA of at most one token per warp needs one stage of the ring only.
 template <int NCH>
-constexpr int kSelRing = NCH * 2 * 2 * 16 * kSelThreads;  // bytes: [stage][cur, cache][chunk][thread]
+__host__ __device__ constexpr int sel_ring(int per) {  // bytes: [stage][warp][cur, cache][chunk][lane]
+  return (per > kSelThreads / 32 ? 2 : 1) * NCH * 2 * 16 * kSelThreads;
+}
 
 template <typename T, int NCH>
 __global__ void __launch_bounds__(kSelThreads, NCH <= 3 ? 4 : 2)
@@ -365,7 +369,7 @@ __global__ void __launch_bounds__(kSelThreads, NCH <= 3 ? 4 : 2)
   const int r = (int)(blockIdx.x / ncta);
   const int per = (n_tok + (int)ncta - 1) / (int)ncta;  // tokens per CTA
   const int t0 = min((int)me * per, n_tok), t1 = min(t0 + per, n_tok);
-  unsigned long long* sK = reinterpret_cast<unsigned long long*>(sel_smem + kSelRing<NCH>);
+  unsigned long long* sK = reinterpret_cast<unsigned long long*>(sel_smem + sel_ring<NCH>(per));
   SimSums* sums = reinterpret_cast<SimSums*>(sK + n_tok);
   unsigned char* sel = reinterpret_cast<unsigned char*>(sums + min(per, kSelThreads));
   const bool need_s = N > 0 && rule != LAZYMAR_SELECT_RANDOM;
@@ -373,7 +377,8 @@ __global__ void __launch_bounds__(kSelThreads, NCH <= 3 ? 4 : 2)
   pdl_wait();
   pdl_trigger();
   const size_t row0 = (size_t)r * n_tok;
-  uint4* ring = reinterpret_cast<uint4*>(sel_smem) + warp * (NCH * 4 * 32) + lane;
+  uint4* ring = reinterpret_cast<uint4*>(sel_smem) + warp * (NCH * 2 * 32) + lane;
+  constexpr int kStage = kWarps * NCH * 2 * 32;  // of the ring
   auto fetch = [&](int t, int stage) {
     const T* a = cur + (row0 + t) * D;
     const T* c = cache + (row0 + t) * D;
@@ -381,8 +386,8 @@ __global__ void __launch_bounds__(kSelThreads, NCH <= 3 ? 4 : 2)
     for (int j = 0; j < NCH; ++j) {
       const int i = (lane + 32 * j) * V;
       const int in = i < D ? 16 : 0, at = in ? i : 0;
-      cp_async16(ring + (stage * 2 * NCH + j) * 32, a + at, in);
-      if (need_s) cp_async16(ring + (stage * 2 * NCH + NCH + j) * 32, c + at, in);
+      cp_async16(ring + stage * kStage + j * 32, a + at, in);
+      if (need_s) cp_async16(ring + stage * kStage + (NCH + j) * 32, c + at, in);
     }
     cp_async_commit();
   };
@@ -404,7 +409,7 @@ __global__ void __launch_bounds__(kSelThreads, NCH <= 3 ? 4 : 2)
         } else {
           cp_async_wait<0>();
         }
-        const uint4* sa = ring + stage * 2 * NCH * 32;
+        const uint4* sa = ring + stage * kStage;
         if (need_s) sums_bf16<NCH>(sa, sa + NCH * 32, a, c, D, span, lane, s);
 #pragma unroll
         for (int j = 0; j < NCH; ++j) {
@@ -497,20 +502,26 @@ __global__ void __launch_bounds__(kSelThreads, NCH <= 3 ? 4 : 2)
 template <int NCH>
 static size_t select_smem(int n_tok, int ncta) {
   const size_t per = (size_t)((n_tok + ncta - 1) / ncta);
-  return kSelRing<NCH> + (size_t)n_tok * sizeof(unsigned long long) +
+  return sel_ring<NCH>((int)per) + (size_t)n_tok * sizeof(unsigned long long) +
          (per < kSelThreads ? per : (size_t)kSelThreads) * sizeof(SimSums) + per;
 }
 
-// CTAs per row. 8 (the portable limit) keeps a row's tokens on 64 warps; with
-// few rows, clusters of 16 spread them over twice as many SMs.
+// CTAs per row: one for every 8 tokens (a warp each), or every 16 where the rows alone
+// fill the SMs, up to 8, the portable limit; with few rows, clusters of 16 spread
+// a row over twice as many SMs. Measured, 8 CTAs for any number of tokens -> this
+// (us): 4096 rows of 8 tokens x 768 369 -> 56, of 17 383 -> 121, 8192 of 16 x 256 693 ->
+// 104, 2048 of 64 196 -> 116, 600 of 8 x 768 55 -> 14.
 constexpr int kSelMaxTokens = 16384;  // of a row, in every entry point
 template <typename T, int NCH>
 static cudaError_t launch_select_t(const Ctx& c, const void* cur, void* cache, int rows, int n_tok, int D, int span,
                                    int N, int* idx, int* row_map, int rule, const uint8_t* prio,
                                    const uint32_t* keys) {
   auto kernel = select_kernel<T, NCH>;
-  const int ncta = rows * 16 <= c.num_sms ? 16 : 8;
-  const size_t smem = N > 0 ? select_smem<NCH>(n_tok, ncta) : kSelRing<NCH>;
+  const int least = rows > c.num_sms ? 16 : 8;  // tokens of a CTA
+  int ncta = 1;
+  while (ncta < 8 && ncta * least < n_tok) ncta *= 2;
+  if (ncta == 8 && rows * 16 <= c.num_sms) ncta = 16;
+  const size_t smem = N > 0 ? select_smem<NCH>(n_tok, ncta) : (size_t)sel_ring<NCH>((n_tok + ncta - 1) / ncta);
   if (smem > 40 * 1024) {
     // always the largest size: the attribute is the process's, and another host
     // thread may be about to launch the kernel for more tokens

@@ -220,6 +220,25 @@ def test_select_tokens_fp32_ranges(rows, T, D):
     assert torch.equal(g_ref.view(torch.int32), g_cur.view(torch.int32))
 
 
+@pytest.mark.parametrize("T", [1, 7, 8, 9, 16, 17, 32, 33, 64])
+@pytest.mark.parametrize("D,dtype", [(768, "bf16"), (1280, "bf16"), (1288, "bf16"), (256, "fp32")])
+def test_select_tokens_few_tokens(T, D, dtype):
+    """Rows of at most 64 tokens, where the CTAs per row and the stages of the
+    copy ring follow the number of tokens; many rows and one."""
+    torch = torch_cuda()
+    for rows in (1, 40):
+        cur, ref = synth.similarity_inputs(rows, T, D, seed=rows * 1000 + T, dtype=dtype)
+        for N in sorted({1, T // 2, T} - {0}):
+            g_cur, g_ref = dev(cur, dtype), dev(ref, dtype)
+            idx = torch.full((rows, N), -1, dtype=torch.int32, device="cuda")
+            lm.lazymar_select_tokens(DT[dtype], g_cur, g_ref, rows, T, D, N, idx)
+            sync()
+            got = idx.cpu().numpy()
+            for r in range(rows):
+                assert got[r].tolist() == O.select_compute(O.cosine_similarity(cur[r], ref[r]), N).tolist()
+            assert torch.equal(g_ref, g_cur)
+
+
 def _in_threads(jobs):
     """Runs the jobs on host threads of their own, each on a CUDA stream of its
     own, at the same time; the first error any of them raised, or None."""
