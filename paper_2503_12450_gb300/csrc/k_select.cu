@@ -31,6 +31,7 @@
 // relative 1e-15 or so). Two tokens whose similarities lie that close may then be
 // ordered differently; every other fp32 selection is identical.
 #include <cfloat>
+#include <climits>
 
 #include "lazymar_internal.cuh"
 
@@ -520,7 +521,7 @@ static cudaError_t launch_select_t(const Ctx& c, const void* cur, void* cache, i
   const int least = rows > c.num_sms ? 16 : 8;  // tokens of a CTA
   int ncta = 1;
   while (ncta < 8 && ncta * least < n_tok) ncta *= 2;
-  if (ncta == 8 && rows * 16 <= c.num_sms) ncta = 16;
+  if (ncta == 8 && rows <= c.num_sms / 16) ncta = 16;
   const size_t smem = N > 0 ? select_smem<NCH>(n_tok, ncta) : (size_t)sel_ring<NCH>((n_tok + ncta - 1) / ncta);
   if (smem > 40 * 1024) {
     // always the largest size: the attribute is the process's, and another host
@@ -537,6 +538,7 @@ static cudaError_t launch_select_t(const Ctx& c, const void* cur, void* cache, i
     if (e != cudaSuccess) return e;
     attr_set[dev] = 1;
   }
+  if ((long long)rows * ncta > INT_MAX) return cudaErrorInvalidValue;  // (more than 500 GB of vectors)
   return launch_pdl_cluster(kernel, dim3((unsigned)(rows * ncta)), dim3(kSelThreads), smem, ncta, c.stream,
                             static_cast<const T*>(cur), static_cast<T*>(cache), n_tok, D, span, N, idx, row_map,
                             rule, prio, keys);

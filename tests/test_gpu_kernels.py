@@ -239,6 +239,19 @@ def test_select_tokens_few_tokens(T, D, dtype):
             assert torch.equal(g_ref, g_cur)
 
 
+def test_select_tokens_more_than_2_to_the_28_rows():
+    """The CTAs of all rows are counted without overflow: every row is copied and
+    selected (2^28 + 1 rows of one token of 8 elements)."""
+    torch = torch_cuda()
+    rows = 2 ** 28 + 1
+    cur = torch.full((rows, 1, 8), 2.0, dtype=torch.bfloat16, device="cuda")
+    cache = torch.ones_like(cur)
+    idx = torch.full((rows, 1), -1, dtype=torch.int32, device="cuda")
+    lm.lazymar_select_tokens(DT["bf16"], cur, cache, rows, 1, 8, 1, idx)
+    sync()
+    assert (cache == 2.0).all() and (idx == 0).all()
+
+
 def _in_threads(jobs):
     """Runs the jobs on host threads of their own, each on a CUDA stream of its
     own, at the same time; the first error any of them raised, or None."""
