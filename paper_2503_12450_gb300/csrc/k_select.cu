@@ -30,6 +30,7 @@
 // last bit) and the oracle's pairwise ones can differ in the last bits of S (a
 // relative 1e-15 or so). Two tokens whose similarities lie that close may then be
 // ordered differently; every other fp32 selection is identical.
+#include <atomic>
 #include <cfloat>
 #include <climits>
 
@@ -507,21 +508,56 @@ static size_t select_smem(int n_tok, int ncta) {
          (per < kSelThreads ? per : (size_t)kSelThreads) * sizeof(SimSums) + per;
 }
 
-// CTAs per row: one for every 8 tokens (a warp each), or every 16 where the rows alone
-// fill the SMs, up to 8, the portable limit; with few rows, clusters of 16 spread
-// a row over twice as many SMs. Measured, 8 CTAs for any number of tokens -> this
+// CTAs per row, up to 8, the portable limit: one for every 8 tokens (a warp each), for
+// every 16 where the rows alone fill the SMs, for every token where 8 CTAs a row would
+// not; with half as many rows, clusters of 16 spread a row over twice as many SMs. Measured, 8 CTAs for any number of tokens -> this
 // (us): 4096 rows of 8 tokens x 768 369 -> 56, of 17 383 -> 121, 8192 of 16 x 256 693 ->
 // 104, 2048 of 64 196 -> 116, 600 of 8 x 768 55 -> 14.
 constexpr int kSelMaxTokens = 16384;  // of a row, in every entry point
+
+// Whether clusters of 16 CTAs of the kernel fit the device (a partition of it may
+// have no 16 SMs together), with the shared memory of the most tokens; allows them.
+template <typename T, int NCH>
+static bool clusters_of_16() {
+  static std::atomic<signed char> known[64];  // per device: 1 yes, -1 no
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return false;
+  if (known[dev] != 0) return known[dev] > 0;
+  const int smem = (int)select_smem<NCH>(kSelMaxTokens, 8);
+  auto kernel = select_kernel<T, NCH>;
+  if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
+      cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(16);
+  cfg.blockDim = dim3(kSelThreads);
+  cfg.dynamicSmemBytes = (size_t)smem;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = 16;
+  attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  int n = 0;
+  if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  known[dev] = n >= 1 ? 1 : -1;
+  return n >= 1;
+}
+
 template <typename T, int NCH>
 static cudaError_t launch_select_t(const Ctx& c, const void* cur, void* cache, int rows, int n_tok, int D, int span,
                                    int N, int* idx, int* row_map, int rule, const uint8_t* prio,
                                    const uint32_t* keys) {
   auto kernel = select_kernel<T, NCH>;
-  const int least = rows > c.num_sms ? 16 : 8;  // tokens of a CTA
+  const int least = rows <= c.num_sms / 8 ? 1 : rows <= c.num_sms ? 8 : 16;  // tokens of a CTA
   int ncta = 1;
   while (ncta < 8 && ncta * least < n_tok) ncta *= 2;
-  if (ncta == 8 && rows <= c.num_sms / 16) ncta = 16;
+  if (ncta == 8 && rows <= c.num_sms / 16 && clusters_of_16<T, NCH>()) ncta = 16;
   const size_t smem = N > 0 ? select_smem<NCH>(n_tok, ncta) : (size_t)sel_ring<NCH>((n_tok + ncta - 1) / ncta);
   if (smem > 40 * 1024) {
     // always the largest size: the attribute is the process's, and another host
@@ -529,14 +565,6 @@ static cudaError_t launch_select_t(const Ctx& c, const void* cur, void* cache, i
     const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                (int)select_smem<NCH>(kSelMaxTokens, 8));
     if (e != cudaSuccess) return e;
-  }
-  static int attr_set[64] = {};
-  int dev = 0;
-  cudaGetDevice(&dev);
-  if (ncta > 8 && dev >= 0 && dev < 64 && !attr_set[dev]) {
-    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    if (e != cudaSuccess) return e;
-    attr_set[dev] = 1;
   }
   if ((long long)rows * ncta > INT_MAX) return cudaErrorInvalidValue;  // (more than 500 GB of vectors)
   return launch_pdl_cluster(kernel, dim3((unsigned)(rows * ncta)), dim3(kSelThreads), smem, ncta, c.stream,

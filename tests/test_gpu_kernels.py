@@ -239,6 +239,23 @@ def test_select_tokens_few_tokens(T, D, dtype):
             assert torch.equal(g_ref, g_cur)
 
 
+@pytest.mark.parametrize("rows,T,D,dtype", [(1, 16384, 1280, "bf16"), (9, 16384, 64, "bf16"), (2, 16384, 64, "fp32"),
+                                            (3, 5000, 768, "bf16")])
+def test_select_tokens_many_tokens_of_few_rows(rows, T, D, dtype):
+    """Clusters of 16 CTAs with up to the largest shared memory a selection takes."""
+    torch = torch_cuda()
+    cur, ref = synth.similarity_inputs(rows, T, D, seed=rows + T, dtype=dtype)
+    g_cur, g_ref = dev(cur, dtype), dev(ref, dtype)
+    N = T // 5
+    idx = torch.full((rows, N), -1, dtype=torch.int32, device="cuda")
+    lm.lazymar_select_tokens(DT[dtype], g_cur, g_ref, rows, T, D, N, idx)
+    sync()
+    got = idx.cpu().numpy()
+    for r in range(rows):
+        assert got[r].tolist() == O.select_compute(O.cosine_similarity(cur[r], ref[r]), N).tolist(), "row %d" % r
+    assert torch.equal(g_ref, g_cur)
+
+
 def test_select_tokens_more_than_2_to_the_28_rows():
     """The CTAs of all rows are counted without overflow: every row is copied and
     selected (2^28 + 1 rows of one token of 8 elements)."""
