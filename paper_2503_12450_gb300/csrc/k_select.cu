@@ -24,8 +24,8 @@
 // for any realistic dynamic range, which makes S independent of the summation
 // order: the oracle's fp64 sum gives bit-identical S, hence bit-identical
 // selections. The kernel computes the three sums exactly on the integer pipe
-// (GB300's fp64 rate is a small fraction of its integer rate) and rounds each
-// once. fp32 x fp32 products are exact in fp64 too, but a sum of them is
+// (GB300's fp64 rate is a small fraction of its integer rate) or, wider than 1280,
+// in triples of floats, and rounds each once. fp32 x fp32 products are exact in fp64 too, but a sum of them is
 // rounded at every addition: the kernel's sums (correctly rounded but for the
 // last bit) and the oracle's pairwise ones can differ in the last bits of S (a
 // relative 1e-15 or so). Two tokens whose similarities lie that close may then be
@@ -150,7 +150,20 @@ __device__ __forceinline__ void add_sum(F32x3& t, const F32x3& o) {
   t.d = f32x2_add(f32x2_add(t.d, o.d), f32x2_add(r, u));
 }
 
-// Sums of one fp32 token in triples of floats (Ogita, Rump and Oishi's compensated
+// 16 bytes of elements as pairs of floats.
+__device__ __forceinline__ void load_pairs(const float* p, unsigned long long (&w)[2]) {
+  const ulonglong2 q = *reinterpret_cast<const ulonglong2*>(p);
+  w[0] = q.x;
+  w[1] = q.y;
+}
+__device__ __forceinline__ void load_pairs(const bf16* p, unsigned long long (&w)[4]) {
+  const uint4 q = *reinterpret_cast<const uint4*>(p);
+  const uint32_t v[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+  for (int i = 0; i < 4; ++i) w[i] = (unsigned long long)(v[i] << 16) | ((unsigned long long)(v[i] & 0xFFFF0000u) << 32);
+}
+
+// Sums of one token in triples of floats (Ogita, Rump and Oishi's compensated
 // dot product with one more level): products and the errors of the first two
 // levels are exact, and the third's roundings lie 2^-72 below the sum of the
 // terms' magnitudes, so the sums are rounded to double once, where an fp64 sum
@@ -160,27 +173,32 @@ __device__ __forceinline__ void add_sum(F32x3& t, const F32x3& o) {
 // call): 64 rows x 320 tokens x 768 200 -> 74, 26 x 320 x 1024 132 -> 51, 1 x 1088 x
 // 1280 146 -> 63 (84 with fp64 sums spread over all SMs), 8 x 320 x 1280 83 -> 32.
 // Largest error of the sums of 60 vectors of 256 to 1280 normal elements: 1.1e-16 of
-// the sum, of fp64 sums 1.2e-14.
+// the sum, of fp64 sums 1.2e-14. bf16 vectors wider than 1280 (whose products are exact
+// in a float): 1 row x 320 x 2048 66 -> 26, 1024 x 65 x 2048 1509 -> 467.
 // Vectors with an element of magnitude from 2^52 or (nonzero) below 2^-51, whose
 // products could overflow or lose bits, and ones with Inf or NaN take fp64 sums.
-__device__ __forceinline__ void sums_f32(const float* a, const float* c, int D, int lane, SimSums& s) {
+template <typename T>
+__device__ __forceinline__ void sums_f32x3(const T* a, const T* c, int D, int lane, SimSums& s) {
+  constexpr int V = 16 / sizeof(T);
   F32x3 dot{}, na{}, nc{};
   uint32_t most = 0, least = 0xFFFFFFFFu;  // of the magnitudes' bits; of those - 1, in which zeros are the largest
 #pragma unroll 2
-  for (int i = lane * 4; i < D; i += 128) {
-    const ulonglong2 x = *reinterpret_cast<const ulonglong2*>(a + i), y = *reinterpret_cast<const ulonglong2*>(c + i);
-    const unsigned long long w[4] = {x.x, x.y, y.x, y.y};
+  for (int i = lane * V; i < D; i += 32 * V) {
+    unsigned long long x[V / 2], y[V / 2];  // two elements each
+    load_pairs(a + i, x);
+    load_pairs(c + i, y);
 #pragma unroll
-    for (int h = 0; h < 4; ++h) {
-      const uint32_t m0 = (uint32_t)w[h] & 0x7FFFFFFFu, m1 = (uint32_t)(w[h] >> 32) & 0x7FFFFFFFu;
-      most = max(most, max(m0, m1));
-      least = min(least, min(m0 - 1u, m1 - 1u));
-    }
+    for (int h = 0; h < V / 2; ++h) {
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      add_product(dot, w[h], w[2 + h]);
-      add_product(na, w[h], w[h]);
-      add_product(nc, w[2 + h], w[2 + h]);
+      for (int j = 0; j < 2; ++j) {
+        const unsigned long long w = j ? y[h] : x[h];
+        const uint32_t m0 = (uint32_t)w & 0x7FFFFFFFu, m1 = (uint32_t)(w >> 32) & 0x7FFFFFFFu;
+        most = max(most, max(m0, m1));
+        least = min(least, min(m0 - 1u, m1 - 1u));
+      }
+      add_product(dot, x[h], y[h]);
+      add_product(na, x[h], x[h]);
+      add_product(nc, y[h], y[h]);
     }
   }
   most = __reduce_max_sync(0xffffffffu, most);
@@ -337,8 +355,8 @@ __device__ __forceinline__ void cp_async_wait() {
 
 // One cluster per row r (blockIdx.x / cluster size). T: element type; NCH > 0:
 // bf16 vectors of at most 256 NCH elements; NCH == 0: vectors streamed from
-// memory (fp32 in triples of floats, wider bf16 vectors in fp64). N == 0 only moves the current vectors
-// into the cache.
+// memory (fp32 and wider bf16 vectors) and summed in triples of floats. N == 0 only moves
+// the current vectors into the cache.
 //
 // With NCH > 0 every lane copies its chunks of the warp's next token to shared
 // memory while the warp works on the current one. A lane reads back only what
@@ -419,11 +437,7 @@ __global__ void __launch_bounds__(kSelThreads, NCH <= 3 ? 4 : 2)
           if (i < D) *reinterpret_cast<uint4*>(c + i) = sa[32 * j];
         }
       } else {
-        if constexpr (sizeof(T) == 4) {
-          if (need_s) sums_f32(a, c, D, lane, s);
-        } else {
-          if (need_s) sums_fp64(a, c, D, lane, s);
-        }
+        if (need_s) sums_f32x3(a, c, D, lane, s);
         for (int i = lane * V; i < D; i += 32 * V)
           *reinterpret_cast<uint4*>(c + i) = *reinterpret_cast<const uint4*>(a + i);
       }

@@ -136,6 +136,13 @@ def test_select_tokens_exponent_range_and_specials(D):
     assert torch.equal(g_ref.view(torch.int16), g_cur.view(torch.int16))
 
 
+@pytest.mark.parametrize("D", [1288, 2048])
+def test_select_tokens_wide_bf16_vectors(D):
+    """bf16 wider than 1280: sums in triples of floats, and in fp64 where exponents
+    or Inf/NaN ask for it."""
+    test_select_tokens_exponent_range_and_specials(D)
+
+
 @pytest.mark.parametrize("D,octaves", [(8, 22), (8, 23), (256, 19), (256, 20), (768, 18), (768, 19), (1280, 18),
                                        (1280, 19), (1288, 18)])
 @pytest.mark.parametrize("rows,T", [(1, 9), (1, 333), (20, 333)])
