@@ -748,7 +748,7 @@ __global__ void __launch_bounds__(256) gemm_f32_kernel(const float* __restrict__
 // loads in flight meanwhile), and the partial tiles are summed in warp order
 // through shared memory. Measured,
 // against the 64 x 64 tiles (us): 40 x 768 x 256 13.0 -> 2.5, 40 x 256 x 1024
-// 47.6 -> 5.3, 160 x 1024 x 256 13.2 -> 6.6, 640 x 256 x 1024 48.8 -> 23.0
+// 47.6 -> 5.3, 160 x 1024 x 256 13.2 -> 6.6, 640 x 256 x 1024 48.8 -> 21.2
 constexpr int kF32Chunk = 32;               // K per staged chunk
 constexpr int kF32Pitch = kF32Chunk + 4;    // floats: rows 16 bytes apart in banks
 template <int NW, int TS>
@@ -1169,22 +1169,47 @@ static cudaError_t launch_bn(const Ctx& c, int dtype, const void* A, const void*
   return launch_tc<128, tc::BF16OUT, 64>(c, A, W, M, N, K, epi);
 }
 
+// fp32: tile width, and the warps that split K of the narrower tiles.
+//
+// 16 x 16 tiles while 32 x 32 ones would leave half of the SMs idle (40 x 256 x 1024:
+// 5.3 against 11.7 us); 16 warps rather than 8 for K > 512 while the tiles leave SMs
+// idle too (160 x 768 x 1024 12.3 against 14.2 us, but 160 x 1024 x 1024 23.3 : 21.2 and
+// 640 x 768 x 768 44.6 : 31.2); 64 x 64 tiles from four per SM on, and before that where
+// they take less time by the estimates below, in ns, fitted to M = 1..10000, N = 64..20000
+// and K = 4..2048. A splitting warp works on chunks of 32, so a slice of K shorter
+// than that saves nothing: 1280 x 768 x 64 21.2 against 9.0 us in 64 x 64 tiles, 2400 x
+// 768 x 768 90 : 82, but 2560 x 768 x 256 38.3 : 48.3.
+enum { F32_64, F32_32_8, F32_32_16, F32_16_8, F32_16_16 };
+static int choose_f32(const Ctx& c, int M, int N, int K) {
+  const long sms = c.num_sms;
+  const long t64 = (long)((M + 63) / 64) * ((N + 63) / 64), t32 = (long)((M + 31) / 32) * ((N + 31) / 32);
+  if (t64 > 4 * sms) return F32_64;
+  if (t32 * 2 <= sms) return K > 512 ? F32_16_16 : F32_16_8;
+  const bool w16 = K > 512 && t32 <= sms;
+  const long k = K, slices = w16 ? 512 : 256;  // K of one chunk in every warp
+  const double split = 2500 + t32 * 152.0 / sms * (3.7 + 0.0625 * ((k + slices - 1) / slices * slices));
+  const double wide = t64 <= sms           ? 2000 + 45.0 * k
+                      : t64 * 3 <= sms * 4 ? 3000 + 77.0 * k
+                      : t64 <= 3 * sms     ? 3000 + 103.0 * k
+                                           : 4000 + 175.0 * k;
+  if (wide < 0.9375 * split) return F32_64;
+  return w16 ? F32_32_16 : F32_32_8;
+}
+
 cudaError_t launch_gemm(const Ctx& c, int dtype, const void* A, const void* W, int M, int N, int K,
                         const GemmEpi& epi, int flags) {
   if (M == 0) return cudaSuccess;
   if (dtype == LAZYMAR_F32) {
     const float *a = static_cast<const float*>(A), *w = static_cast<const float*>(W);
-    dim3 grid((N + 63) / 64, (M + 63) / 64);
-    const long tiles32 = (long)((N + 31) / 32) * ((M + 31) / 32);
-    // 64 x 64 tiles once they fill the SMs several times (4 per SM: 2560 x 1024 x
-    // 256 takes 48.5 against 49.4 us; 2560 x 768 x 256 still 48.0 against 38.0);
-    // 16 x 16 tiles while 32 x 32 ones would leave half of the SMs idle (40 x 256 x
-    // 1024: 5.3 against 11.7 us)
-    if ((long)grid.x * grid.y > 4L * c.num_sms)
-      return launch_pdl(gemm_f32_kernel, grid, dim3(256), 0, c.stream, a, w, M, N, K, epi);
-    if (tiles32 * 2 <= c.num_sms)
-      return K > 512 ? launch_f32_splitk<16, 16>(c, a, w, M, N, K, epi) : launch_f32_splitk<8, 16>(c, a, w, M, N, K, epi);
-    return K > 512 ? launch_f32_splitk<16, 32>(c, a, w, M, N, K, epi) : launch_f32_splitk<8, 32>(c, a, w, M, N, K, epi);
+    switch (choose_f32(c, M, N, K)) {
+      case F32_64:
+        return launch_pdl(gemm_f32_kernel, dim3((N + 63) / 64, (M + 63) / 64), dim3(256), 0, c.stream, a, w, M, N, K,
+                          epi);
+      case F32_32_8: return launch_f32_splitk<8, 32>(c, a, w, M, N, K, epi);
+      case F32_32_16: return launch_f32_splitk<16, 32>(c, a, w, M, N, K, epi);
+      case F32_16_8: return launch_f32_splitk<8, 16>(c, a, w, M, N, K, epi);
+      default: return launch_f32_splitk<16, 16>(c, a, w, M, N, K, epi);
+    }
   }
   if (flags == 2 && N % 256 == 0) return launch_bn(c, dtype, A, W, M, N, K, epi, 256);
   if (flags == 3 && N % 192 == 0) return launch_bn(c, dtype, A, W, M, N, K, epi, 192);

@@ -597,6 +597,13 @@ def test_linear_fp32_tiles(M, N, K, epi):
     _linear_case("fp32", epi, M, N, K, 0, seed=M + N + K + epi)
 
 
+@pytest.mark.parametrize("M,N,K", [(641, 1028, 68), (641, 1028, 260), (2399, 772, 772), (161, 1028, 1028), (159, 772, 1028),
+                                   (9, 20004, 64), (1279, 772, 128)])
+def test_linear_fp32_tile_choice(M, N, K):
+    """Sizes on either side of the lines between the fp32 tiles and splits of K."""
+    _linear_case("fp32", lm.LAZYMAR_EPI_BIAS, M, N, K, 0, seed=M + N + K)
+
+
 @pytest.mark.parametrize("rows,n_q,T,heads,dh", [(2, 5, 32, 2, 64), (1, 9, 33, 3, 30), (1, 4, 127, 1, 128), (2, 3, 128, 2, 64),
                                                  (1, 6, 129, 2, 64), (1, 2, 300, 2, 66), (3, 1, 1, 2, 1), (1, 5, 8192, 1, 8)])
 def test_attention_fp32_chunks(rows, n_q, T, heads, dh):
