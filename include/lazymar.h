@@ -272,6 +272,12 @@ lazymar_status lazymar_linear(int dtype, int epilogue, const void *a, const void
                               void *k_out, void *v_out, const int32_t *row_map, int flags,
                               void *stream);
 
+/* The tiles that lazymar_linear with flags 0 works on for a bf16 shape on a
+ * device of num_sms SMs, on the host alone: tiles[0] rows (256: a tile of two
+ * CTAs) and tiles[1] columns of a tile, tiles[2] tiles at that width, and the
+ * others, a last round, in tiles[3] equal parts each. */
+lazymar_status lazymar_linear_tiles(int epilogue, int M, int N, int K, int num_sms, int32_t *tiles);
+
 /* lazymar_linear with E4M3 operands (kind::f8f6f4 tensor cores, fp32
  * accumulation): a [M, K] and w [N, K] hold E4M3 bytes, wscale [N] fp32 the
  * per-output-column scale of w; y = (a w^T) * wscale + bias (bias bf16, may be

@@ -951,6 +951,13 @@ static long rounds_cost(long base, long slots, int bn, long time, bool pair, boo
   return rounds * time + best;
 }
 
+// Whether the kernel of these tiles has a form that splits its last round. Single
+// CTAs have a kernel of their own for it: a tile width known only at run time
+// costs short launches 2 to 5 % (out at M = 1600, width 768: 5.6 against 5.8 us).
+constexpr bool can_split(int bn, int ek, bool f8, bool pair) {
+  return pair || (bn == 256 && !f8 && (ek == tc::BF16OUT || ek == tc::RESID_WIDE));
+}
+
 template <int BN, int EK, int BK, int F8 = 0, int PAIR = 0, int ROWS = 128>
 static cudaError_t launch_tc(const Ctx& c, const void* A, const void* W, int M, int N, int K, const GemmEpi& epi) {
   using C = tc::Cfg<BN, EK, BK, F8, PAIR, ROWS>;
@@ -961,10 +968,7 @@ static cudaError_t launch_tc(const Ctx& c, const void* A, const void* W, int M, 
       !make_tmap_2d(dt, &tb, W, (uint64_t)K, (uint64_t)N, (uint64_t)K * C::EB, C::ATOM_E, C::B_ROWS,
                     CU_TENSOR_MAP_SWIZZLE_128B))
     return cudaErrorInvalidValue;
-  // Single CTAs have a kernel of their own for launches with a split round: a
-  // tile width known only at run time costs short launches 2 to 5 % (out at M =
-  // 1600, width 768: 5.6 against 5.8 us).
-  constexpr bool CAN_SPLIT = PAIR || (BN == 256 && !F8 && (EK == tc::BF16OUT || EK == tc::RESID_WIDE));
+  constexpr bool CAN_SPLIT = can_split(BN, EK, F8 != 0, PAIR != 0);
   const auto kernel = gemm_bf16_tc_kernel<BN, EK, BK, F8, PAIR, ROWS, PAIR != 0>;
   const auto split_kernel = gemm_bf16_tc_kernel<BN, EK, BK, F8, PAIR, ROWS, CAN_SPLIT>;
   static int attr_set[64] = {};
@@ -1097,6 +1101,29 @@ static int choose_bn(const Ctx& c, int dtype, int M, int N, const GemmEpi& epi, 
   return bn;
 }
 
+static int epi_kind(const GemmEpi& epi, int K) {
+  return epi.mode == LAZYMAR_EPI_SILU       ? tc::BF16OUT_SILU
+         : epi.mode != LAZYMAR_EPI_RESIDUAL ? tc::BF16OUT
+         : epi.gate                          ? tc::RESID_WIDE_GATED
+         : K < 2048                          ? tc::RESID_WIDE
+                                             : tc::RESID_HALF;
+}
+
+// The bf16 tiles of launch_gemm's automatic choice: rows (256: on CTA pairs) and
+// width of a tile, the tiles at full width, the parts of each of the others.
+void gemm_tiles(int num_sms, int M, int N, int K, const GemmEpi& epi, int* rows, int* width, int* whole, int* split) {
+  const Ctx c{nullptr, nullptr, num_sms};
+  const int bn = choose_bn(c, LAZYMAR_BF16, M, N, epi, K);
+  *rows = bn >= kRows64 ? 64 : bn >= kPair ? 256 : 128;
+  *width = bn % kPair;
+  const int base = (M + *rows - 1) / *rows * (N / *width);
+  const bool pair = *rows == 256;
+  *whole = base;
+  *split = 1;
+  if (*rows >= 128 && can_split(*width, epi_kind(epi, K), false, pair))
+    rounds_cost(base, pair ? num_sms / 2 : num_sms, *width, 100, pair, epi.mode == LAZYMAR_EPI_RESIDUAL, K, whole, split);
+}
+
 static cudaError_t launch_bn(const Ctx& c, int dtype, const void* A, const void* W, int M, int N, int K,
                              const GemmEpi& epi, int bn) {
   if (dtype == LAZYMAR_E4M3) {
@@ -1106,11 +1133,7 @@ static cudaError_t launch_bn(const Ctx& c, int dtype, const void* A, const void*
     if (bn == 192) return launch_tc<192, tc::BF16OUT, 128, 1>(c, A, W, M, N, K, epi);
     return launch_tc<128, tc::BF16OUT, 128, 1>(c, A, W, M, N, K, epi);
   }
-  const int ek = epi.mode == LAZYMAR_EPI_SILU       ? tc::BF16OUT_SILU
-                 : epi.mode != LAZYMAR_EPI_RESIDUAL ? tc::BF16OUT
-                 : epi.gate                          ? tc::RESID_WIDE_GATED
-                 : K < 2048                          ? tc::RESID_WIDE
-                                                     : tc::RESID_HALF;
+  const int ek = epi_kind(epi, K);
   if (bn == kRows64 + 128) {
     if (ek == tc::RESID_WIDE) return launch_tc<128, tc::RESID_WIDE, 128, 0, 0, 64>(c, A, W, M, N, K, epi);
     return launch_tc<128, tc::RESID_HALF, 128, 0, 0, 64>(c, A, W, M, N, K, epi);

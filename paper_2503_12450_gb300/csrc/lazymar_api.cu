@@ -945,6 +945,16 @@ extern "C" lazymar_status lazymar_linear(int dtype, int epilogue, const void* a,
   return err == cudaSuccess ? LAZYMAR_OK : cuda_fail(err, "gemm kernel");
 }
 
+extern "C" lazymar_status lazymar_linear_tiles(int epilogue, int M, int N, int K, int num_sms, int32_t* tiles) {
+  if (epilogue < LAZYMAR_EPI_BIAS || epilogue > LAZYMAR_EPI_SILU) return fail(LAZYMAR_ERR_INVALID_ARG, "epilogue");
+  if (M < 1 || num_sms < 1 || !tiles) return fail(LAZYMAR_ERR_INVALID_ARG, "M >= 1, num_sms >= 1 and tiles required");
+  GemmEpi e{epilogue, nullptr, nullptr, N, nullptr, nullptr, nullptr, epilogue == LAZYMAR_EPI_QKV ? N / 3 : 0};
+  const char* why = "";
+  if (!gemm_supported(LAZYMAR_BF16, M, N, K, e, &why)) return fail(LAZYMAR_ERR_UNSUPPORTED, why);
+  gemm_tiles(num_sms, M, N, K, e, tiles, tiles + 1, tiles + 2, tiles + 3);
+  return LAZYMAR_OK;
+}
+
 extern "C" lazymar_status lazymar_linear_e4m3(int epilogue, const void* a, const void* w, const float* wscale,
                                               const void* bias, int M, int N, int K, void* out, int ldo, void* k_out,
                                               void* v_out, const int32_t* row_map, int flags, void* stream) {

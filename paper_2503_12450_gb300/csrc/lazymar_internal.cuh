@@ -626,6 +626,8 @@ struct GemmEpi {
 };
 cudaError_t launch_gemm(const Ctx& c, int dtype, const void* A, const void* W, int M, int N, int K,
                         const GemmEpi& epi, int flags);
+// The tiles launch_gemm chooses for a bf16 GEMM on num_sms SMs (lazymar_linear_tiles).
+void gemm_tiles(int num_sms, int M, int N, int K, const GemmEpi& epi, int* rows, int* width, int* whole, int* split);
 // Checks the preconditions of launch_gemm; returns false with a message.
 bool gemm_supported(int dtype, int M, int N, int K, const GemmEpi& epi, const char** why);
 

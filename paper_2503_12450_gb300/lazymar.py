@@ -106,6 +106,7 @@ def lib():
         "lazymar_cfg_combine": (st, [i, i, vp, vp, vp, f, sz, vp, vp, vp]),
         "lazymar_linear": (st, [i, i, vp, vp, vp, i, i, i, vp, i, vp, vp, vp, i, vp]),
         "lazymar_attention": (st, [i, vp, vp, vp, vp, i, i, i, i, i, vp]),
+        "lazymar_linear_tiles": (st, [i, i, i, i, i, vp]),
         "lazymar_linear_e4m3": (st, [i, vp, vp, vp, vp, i, i, i, vp, i, vp, vp, vp, i, vp]),
         "lazymar_quantize_e4m3": (st, [vp, i, i, vp, vp, vp]),
         "lazymar_layernorm": (st, [i, vp, vp, vp, vp, vp, i, i, f, vp]),
@@ -277,6 +278,13 @@ def lazymar_linear(dtype, epilogue, a, w, bias, M, N, K, out, ldo, k_out=None, v
     _check(lib().lazymar_linear(int(dtype), int(epilogue), _ptr(a), _ptr(w), _ptr(bias), int(M), int(N), int(K),
                                 _ptr(out), int(ldo), _ptr(k_out), _ptr(v_out), _ptr(row_map), int(flags),
                                 _stream(stream)))
+
+
+def lazymar_linear_tiles(epilogue, M, N, K, num_sms=152):
+    """(rows, width, whole tiles, parts of the others) that a bf16 lazymar_linear chooses."""
+    tiles = (ctypes.c_int32 * 4)()
+    _check(lib().lazymar_linear_tiles(int(epilogue), int(M), int(N), int(K), int(num_sms), ctypes.addressof(tiles)))
+    return tuple(tiles)
 
 
 def lazymar_linear_e4m3(epilogue, a, w, wscale, bias, M, N, K, out, ldo, k_out=None, v_out=None, row_map=None,

@@ -113,6 +113,23 @@ def test_linear_rejects_unsupported_shapes(lib, args, status):
     assert lib.lazymar_linear(dtype, epi, a, w, b, M, N, K, None, ldo, None, None, None, 0, None) == status
 
 
+def test_linear_tiles_of_the_model_shapes(lib):
+    """The host-side choice of tiles on 152 SMs: (rows, width, whole tiles, parts of
+    the others), and its argument checks."""
+    res, gelu = lm.LAZYMAR_EPI_RESIDUAL, lm.LAZYMAR_EPI_GELU
+    assert lm.lazymar_linear_tiles(gelu, 50, 3072, 768) == (64, 64, 48, 1)
+    assert lm.lazymar_linear_tiles(gelu, 20480, 3072, 768)[:2] == (256, 256)
+    assert lm.lazymar_linear_tiles(gelu, 1600, 3072, 768) == (128, 256, 152, 4)
+    assert lm.lazymar_linear_tiles(res, 20480, 768, 3072) == (256, 256, 228, 4)
+    assert lm.lazymar_linear_tiles(res, 7040, 768, 3072) == (256, 192, 76, 2)
+    tiles = (ctypes.c_int32 * 4)()
+    assert lib.lazymar_linear_tiles(2, 0, 768, 768, 152, ctypes.addressof(tiles)) == 1     # M
+    assert lib.lazymar_linear_tiles(2, 64, 768, 768, 0, ctypes.addressof(tiles)) == 1      # num_sms
+    assert lib.lazymar_linear_tiles(9, 64, 768, 768, 152, ctypes.addressof(tiles)) == 1    # epilogue
+    assert lib.lazymar_linear_tiles(2, 64, 768, 768, 152, None) == 1
+    assert lib.lazymar_linear_tiles(2, 64, 100, 768, 152, ctypes.addressof(tiles)) == 6    # N % 128
+
+
 def test_component_argument_checks(lib):
     assert lib.lazymar_select_tokens(1, None, None, 2, 10, 12, 3, None, None) == 1      # D % 8
     assert lib.lazymar_select_tokens(1, None, None, 2, 10, 16, 11, None, None) == 1     # N > T

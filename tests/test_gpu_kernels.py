@@ -454,40 +454,49 @@ def test_linear_bf16_tcgen05(M, N, K, epi):
         _linear_case("bf16", epi, M, N, K, flags, seed=M + N + K + epi)
 
 
-@pytest.mark.parametrize("M,N,K,epi", [
-    (20480, 768, 768, lm.LAZYMAR_EPI_RESIDUAL),    # out-projection: three waves of 256-wide tiles, then 8 row tiles 64 wide
-    (20480, 768, 3072, lm.LAZYMAR_EPI_RESIDUAL),   # residual over long K (fc2): one launch
-    (20480, 2304, 768, lm.LAZYMAR_EPI_QKV),        # other epilogues: one launch
+def _tiles(epi, M, N, K):
+    """(rows, width, parts of a tile of the last round) of the automatic choice."""
+    sms = torch_cuda().cuda.get_device_properties(0).multi_processor_count
+    rows, width, _, parts = lm.lazymar_linear_tiles(epi, M, N, K, sms)
+    return rows, width, parts
+
+
+@pytest.mark.parametrize("M,N,K,epi,tiles", [
+    (20480, 768, 768, lm.LAZYMAR_EPI_RESIDUAL, (128, 256, 4)),    # out-projection: three rounds, then 96 tiles 64 wide
+    (20480, 768, 3072, lm.LAZYMAR_EPI_RESIDUAL, (256, 256, 4)),   # fc2: three rounds of CTA pairs, then 48 tiles 64 wide
+    (20480, 2304, 768, lm.LAZYMAR_EPI_QKV, (256, 256, 2)),        # Q/K/V: nine rounds of pairs, then 72 tiles 128 wide
 ])
-def test_linear_last_wave_split(M, N, K, epi):
-    """With the automatic tile width (flags 0) the fp32-residual GEMM over
-    short K whose last round of tiles would run mostly empty is launched as
-    two: the row tiles of the whole waves, then the remaining rows (their A
-    rows and residual rows offset) with narrower tiles."""
+def test_linear_last_wave_split(M, N, K, epi, tiles):
+    """Full layers, whose last round of tiles would leave most SMs idle: it runs
+    as narrower tiles of the same launch."""
+    assert _tiles(epi, M, N, K) == tiles
     _linear_case("bf16", epi, M, N, K, 0, seed=M + N + K + epi)
     if epi == lm.LAZYMAR_EPI_QKV:
         _linear_case("bf16", epi, M, N, K, 0, seed=M + N + K, scatter=False)
 
 
-@pytest.mark.parametrize("M,N,K,epi", [
-    (20353, 2304, 768, lm.LAZYMAR_EPI_QKV),        # one row in the even CTA's half of the last tile
-    (20480, 2304, 768, lm.LAZYMAR_EPI_QKV),
-    (6529, 4096, 1024, lm.LAZYMAR_EPI_GELU),       # one row in the odd CTA's half
-    (8577, 1024, 1024, lm.LAZYMAR_EPI_RESIDUAL),
-    (9700, 768, 3072, lm.LAZYMAR_EPI_RESIDUAL),    # 192-wide pairs
-    (2561, 1280, 5120, lm.LAZYMAR_EPI_RESIDUAL),
-    (12345, 768, 3072, lm.LAZYMAR_EPI_RESIDUAL),
-    (20480, 3072, 832, lm.LAZYMAR_EPI_BIAS),       # 13 K steps: the ring wraps within a tile
-    # a last round of 64-wide tiles (the first three also have one of 128-wide ones)
-    (20480, 768, 3072, lm.LAZYMAR_EPI_RESIDUAL),
-    (10001, 1024, 1024, lm.LAZYMAR_EPI_RESIDUAL),
-    (5000, 1024, 1024, lm.LAZYMAR_EPI_BIAS),
+@pytest.mark.parametrize("M,N,K,epi,tiles", [
+    (20353, 2304, 768, lm.LAZYMAR_EPI_QKV, (256, 256, 2)),        # one row in the even CTA's half of the last tile
+    (20480, 2304, 768, lm.LAZYMAR_EPI_QKV, (256, 256, 2)),
+    (6529, 4096, 1024, lm.LAZYMAR_EPI_GELU, (256, 256, 2)),       # one row in the odd CTA's half
+    (20480, 3072, 832, lm.LAZYMAR_EPI_BIAS, (256, 256, 1)),       # 13 K steps: the ring wraps within a tile
+    (9700, 768, 3072, lm.LAZYMAR_EPI_RESIDUAL, (256, 256, 2)),
+    (12345, 768, 3072, lm.LAZYMAR_EPI_RESIDUAL, (256, 256, 1)),
+    (20480, 768, 3072, lm.LAZYMAR_EPI_RESIDUAL, (256, 256, 4)),
+    (7169, 768, 3072, lm.LAZYMAR_EPI_RESIDUAL, (256, 256, 4)),
+    # 192-wide pairs: whole, and a last round of halves (96 wide, 48 rows of W in each CTA) or thirds
+    (2049, 1152, 4608, lm.LAZYMAR_EPI_RESIDUAL, (256, 192, 1)),
+    (6464, 768, 3072, lm.LAZYMAR_EPI_RESIDUAL, (256, 192, 2)),
+    (7040, 768, 3072, lm.LAZYMAR_EPI_RESIDUAL, (256, 192, 2)),
+    (7041, 768, 3072, lm.LAZYMAR_EPI_RESIDUAL, (256, 192, 2)),
+    (3201, 1152, 4608, lm.LAZYMAR_EPI_RESIDUAL, (256, 192, 3)),
 ])
-def test_linear_pairs_equal_single_ctas(M, N, K, epi):
+def test_linear_pairs_equal_single_ctas(M, N, K, epi, tiles):
     """At these sizes the automatic choice is 256-row tiles on CTA pairs. An
     accumulator sums the same products in the same order as a single CTA's, so
     the results equal the 128-wide tiles' bit for bit; rows past M and cache
     rows outside the row map stay as they were."""
+    assert _tiles(epi, M, N, K) == tiles
     torch = torch_cuda()
     g = torch.Generator(device="cuda")
     g.manual_seed(M + N + K)
@@ -521,8 +530,10 @@ def test_linear_pairs_equal_single_ctas(M, N, K, epi):
     (20480, 768, 768, lm.LAZYMAR_EPI_RESIDUAL),     # four rounds, the last in quarters
 ])
 def test_linear_split_round_equals_equal_tiles(M, N, K, epi):
-    """256-wide tiles whose last round is split into narrower ones (forced width,
-    and the automatic choice) give the 128-wide tiles' results bit for bit."""
+    """256-wide tiles of single CTAs whose last round is split into narrower ones (by
+    forced width, and in the automatic choice but for the Q/K/V case) give the
+    128-wide tiles' results bit for bit."""
+    assert epi == lm.LAZYMAR_EPI_QKV or _tiles(epi, M, N, K) in ((128, 256, 2), (128, 256, 4))
     torch = torch_cuda()
     g = torch.Generator(device="cuda")
     g.manual_seed(M + N + K)
@@ -562,6 +573,10 @@ def test_linear_few_rows_equal_128_row_tiles(M, N, K, epi):
     D = N // 3
     if epi == lm.LAZYMAR_EPI_QKV and (N % 3 or D % 32):
         pytest.skip("not a QKV shape")
+    if M < 1000:
+        assert _tiles(epi, M, N, K)[:2] == (64, 64)
+    elif epi == lm.LAZYMAR_EPI_RESIDUAL:
+        assert _tiles(epi, M, N, K)[:2] == (64, 128)
     maps = [None, torch.randperm(M + 40, generator=g, device="cuda")[:M].int()] if epi == lm.LAZYMAR_EPI_QKV else [None]
     for row_map in maps:
         res = []
