@@ -1045,9 +1045,13 @@ static int tile_time(int bn, int kind) {
 // 148.1, fc1 226.9 -> 201.0, fc2 228.8 -> 211.0. The out-projection, bound by its
 // residual rows, stays on single CTAs (width 1024, with split last rounds: M =
 // 17408 42.6 against 44.5, M = 40960 86.8 against 89.0; width 768 8.2 against 9.2 a
-// round). Where the 256-row tiles need more rounds or there is only one short
-// one, single CTAs win too (M = 3200, width 768: Q/K/V 11.9 against 13.5, fc2 15.1
-// against 19.1).
+// round). Where the 256-row tiles need more rounds single CTAs win too (M = 3200,
+// width 768: Q/K/V 11.9 against 13.5, fc2 15.1 against 19.1), and where 256-wide tiles
+// of single CTAs fit in one round, which is the shorter the fewer SMs work in it
+// (single against pairs, fc2: width 768, M = 5120 21.8 : 23.2, 6400 23.5 : 24.1; width
+// 1024, M = 2560 25.6 : 26.6, 4500 27.9 : 28.1; width 1280, M = 2240 30.1 : 31.5, 3200 31.0 :
+// 32.1; and 3 to 10 % with bf16 outputs), except for a nearly full round of long K (width
+// 1024, M = 4864 30.0 : 28.8; width 1280, M = 3500 34.8 : 33.1, 3840 36.1 : 33.8).
 static int choose_bn(const Ctx& c, int dtype, int M, int N, const GemmEpi& epi, int K) {
   const long mt = (M + tc::BM - 1) / tc::BM;
   const bool resid = epi.mode == LAZYMAR_EPI_RESIDUAL;
@@ -1070,7 +1074,8 @@ static int choose_bn(const Ctx& c, int dtype, int M, int N, const GemmEpi& epi, 
       bn = widths[i];
     }
   }
-  if (plain && kind != T_RESID) {
+  const long single = N % 256 == 0 ? mt * (N / 256) : c.num_sms + 1L;  // 256-wide tiles of single CTAs
+  if (plain && kind != T_RESID && (single > c.num_sms || (K >= 4096 && single * 12 >= 11L * c.num_sms))) {
     const long pt = (mt + 1) / 2, pairs = c.num_sms / 2;
     auto consider = [&](int width, int time) {
       if (pairs < 1 || N % width != 0) return;

@@ -122,6 +122,13 @@ def test_linear_tiles_of_the_model_shapes(lib):
     assert lm.lazymar_linear_tiles(gelu, 1600, 3072, 768) == (128, 256, 152, 4)
     assert lm.lazymar_linear_tiles(res, 20480, 768, 3072) == (256, 256, 228, 4)
     assert lm.lazymar_linear_tiles(res, 7040, 768, 3072) == (256, 192, 76, 2)
+    # fc2 whose 256-wide tiles fit one round of single CTAs: no pairs, but in a nearly full round of long K
+    assert lm.lazymar_linear_tiles(res, 5120, 768, 3072) == (128, 256, 120, 1)
+    assert lm.lazymar_linear_tiles(res, 6400, 768, 3072) == (128, 256, 150, 1)
+    assert lm.lazymar_linear_tiles(res, 4200, 1024, 4096) == (128, 256, 132, 1)
+    assert lm.lazymar_linear_tiles(res, 4864, 1024, 4096)[:2] == (256, 256)
+    assert lm.lazymar_linear_tiles(res, 2240, 1280, 5120) == (128, 256, 90, 1)
+    assert lm.lazymar_linear_tiles(res, 3500, 1280, 5120)[:2] == (256, 256)
     tiles = (ctypes.c_int32 * 4)()
     assert lib.lazymar_linear_tiles(2, 0, 768, 768, 152, ctypes.addressof(tiles)) == 1     # M
     assert lib.lazymar_linear_tiles(2, 64, 768, 768, 0, ctypes.addressof(tiles)) == 1      # num_sms
