@@ -22,9 +22,9 @@ def z_rows(z, B, n_img, pos):
     return zc.reshape(B * n_new, -1), zu.reshape(B * n_new, -1)
 
 
-def setup(name, cond_dim, B, n_img, n_new, seed, z_dtype="bf16", steps=None):
+def setup(name, cond_dim, B, n_img, n_new, seed, z_dtype="bf16", steps=None, **over):
     torch_cuda()
-    hc = S.head_config(name, **({} if steps is None else {"n_steps": steps}))
+    hc = S.head_config(name, **over, **({} if steps is None else {"n_steps": steps}))
     W = S.make_head_weights(hc, cond_dim, TD, seed=seed)
     rng = np.random.default_rng(seed)
     z = rng.standard_normal((2 * B, n_img, cond_dim)).astype(np.float32)
@@ -40,9 +40,21 @@ def setup(name, cond_dim, B, n_img, n_new, seed, z_dtype="bf16", steps=None):
     ("mar_b", 768, 1, 256, 1, "bf16"),      # a single token
     ("tiny", 256, 2, 64, 5, "fp32"),        # fp32 features, width 128
     ("mar_h", 1280, 2, 256, 7, "bf16"),     # width 1536, 12 blocks
+    ("mar_b", 768, 2, 256, 128, "bf16"),    # 512 rows, the most that fc2 and LayerNorm share a kernel for
+    ("mar_b", 768, 1, 300, 257, "bf16"),    # 514 rows: separate kernels
 ])
 def test_network_output_matches_oracle(name, cond_dim, B, n_img, n_new, z_dtype):
-    hc, W, z, pos, h = setup(name, cond_dim, B, n_img, n_new, seed=11, z_dtype=z_dtype)
+    check_network(name, cond_dim, B, n_img, n_new, z_dtype)
+
+
+@pytest.mark.parametrize("width", [256, 384, 640, 896])
+def test_network_output_at_other_widths(width):
+    """Clusters of 4, 6, 10 and 14 CTAs in the kernel that joins fc2 and LayerNorm."""
+    check_network("tiny", 256, 3, 64, 23, "bf16", width=width, depth=3)
+
+
+def check_network(name, cond_dim, B, n_img, n_new, z_dtype, **over):
+    hc, W, z, pos, h = setup(name, cond_dim, B, n_img, n_new, seed=11, z_dtype=z_dtype, **over)
     M = B * n_new
     x = np.random.default_rng(12).standard_normal((M, TD)).astype(np.float32)
     zc, zu = z_rows(z, B, n_img, pos)

@@ -2,9 +2,8 @@
 
 lazymar_select_tokens_noalloc exists for callers that may not allocate device
 memory once they are running: a serving loop that fixes its memory budget at
-start-up, or a plug-in whose host framework owns the device allocator. Its
-similarity scratch is a fixed array inside the library instead of
-stream-ordered allocations.
+start-up, or a plug-in whose host framework owns the device allocator. Neither
+entry point allocates or keeps scratch; this one refuses rows x T above a limit.
 
 This file is collected last so that a run stopping at the first failure has
 already run every other test. It calls the new entry point twice in a row
@@ -21,8 +20,7 @@ from _gpu import DT, dev, sync, torch_cuda
 
 pytestmark = pytest.mark.gpu
 
-# Two calls in a row with different shapes: the second finds the first call's
-# similarities still in the shared scratch.
+# Two calls in a row with different shapes: nothing of the first is left for the second.
 CASES = [(64, 320, 768, 50, "bf16", 901), (32, 1088, 1024, 272, "bf16", 902)]
 
 
@@ -41,8 +39,8 @@ def test_noalloc_selection_matches_allocating_entry_point_on_two_calls():
         assert torch.equal(a_ref, b_ref) and torch.equal(b_ref, b_cur)
 
 
-# fp32 inputs; no token recomputed; T = 8192, where the top-N's key array
-# (64 KiB) needs the opt-in shared-memory size; rows x T at the limit.
+# fp32 inputs; no token recomputed; T = 8192, whose keys (64 KiB) need the
+# opt-in shared-memory size; rows x T at the limit.
 MORE_CASES = [(2, 80, 256, 20, "fp32", 903), (3, 320, 768, 0, "bf16", 904), (16, 8192, 64, 1000, "bf16", 905),
               (256, 1024, 8, 100, "bf16", 906)]
 
@@ -62,7 +60,7 @@ def test_noalloc_selection_more_shapes(rows, T, D, N, dtype, seed):
     assert torch.equal(a_ref, b_ref) and torch.equal(b_ref, b_cur)
 
 
-def test_noalloc_rejects_sizes_beyond_its_scratch():
+def test_noalloc_rejects_sizes_beyond_its_limit():
     torch_cuda()
     # 257 rows x 1024 tokens = 263,168 > LAZYMAR_SELECT_NOALLOC_MAX_TOKENS (262,144);
     # refused before any device work.
