@@ -652,7 +652,7 @@ bool width_ok(int w) {
 struct lazymar_head {
   lazymar_head_config cfg{};
   int dev = 0, num_sms = 0, w = 0, td = 0, nmod = 0;
-  bool fused = false;  // fc2_ln_kernel serves this width
+  int fuse_rows = 0;  // rows up to which fc2_ln_kernel serves this width
   int chunk = 1;  // kept steps whose modulations are computed by one GEMM
   uint8_t* arena = nullptr;
   // weights (bf16 unless noted)
@@ -760,7 +760,8 @@ cudaError_t launch_final(const Ctx& c, lazymar_head* h, size_t smem, const bf16*
   }
 }
 
-// Rows up to which fc2_ln_kernel is used: one wave of 16-CTA clusters.
+// Rows up to which fc2_ln_kernel is used at any width (and what one wave of its
+// clusters holds, if less).
 constexpr int kFuseRows = 512;
 
 // fc2_ln_kernel for block b's W2 and the modulations of block b + 1.
@@ -777,17 +778,20 @@ cudaError_t launch_fc2_ln(const Ctx& c, lazymar_head* h, int b, const bf16* mod,
                             3 * w * (b + 1), 3 * w * (b + 1) + w, h->xh, h->hb, R, w, h->cfg.ln_eps, h->err);
 }
 
-// Whether fc2_ln_kernel serves width w on the current device (a cluster of w /
-// 64 CTAs fits); sets its launch attributes.
-bool fc2_ln_fits(int w) {
+// Rows up to which fc2_ln_kernel serves width w on the current device: those of the
+// clusters of w / 64 CTAs that fit at once. (Of the 14- and 16-CTA clusters of widths 896
+// and 1024 seven do, 448 rows; the eighth row tile as a second wave took 1.72 ms a call
+// of 20 steps and 4 blocks at width 1024, separate launches 1.41.) Sets its launch
+// attributes.
+int fc2_ln_rows(int w) {
   using C = hd::FusedCfg;
   constexpr int BN = C::BN;
   auto kernel = hd::fc2_ln_kernel;
-  if (w % BN != 0 || w / BN > C::MAXC) return false;
+  if (w % BN != 0 || w / BN > C::MAXC) return 0;
   if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM) != cudaSuccess ||
       cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
     cudaGetLastError();
-    return false;
+    return 0;
   }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(w / BN));
@@ -802,9 +806,9 @@ bool fc2_ln_fits(int w) {
   int n = 0;
   if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) {
     cudaGetLastError();
-    return false;
+    return 0;
   }
-  return n >= 1;
+  return n * C::ROWS < kFuseRows ? n * C::ROWS : kFuseRows;
 }
 
 // Gathers the z rows and embeds them (W_c z + b_c), once per call.
@@ -848,7 +852,7 @@ lazymar_status modulations(lazymar_head* h, const Ctx& c, int M, int j0, int cnt
 lazymar_status network(lazymar_head* h, const Ctx& c, int M, int j, const bf16* mod, bool done, float* eval_out,
                        bool first_done = false, const bf16* next_mod = nullptr) {
   const int R = 2 * M, w = h->w, depth = h->cfg.depth, td = h->td;
-  const bool fuse = h->fused && R <= kFuseRows;
+  const bool fuse = R <= h->fuse_rows;
   for (int b = 0; b < depth; ++b) {
     const bool normed = b > 0 ? fuse : first_done;  // hb already holds this block's input
     if (!normed)
@@ -1022,7 +1026,7 @@ extern "C" lazymar_status lazymar_head_create(const lazymar_head_config* cfg, co
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&h->num_sms, cudaDevAttrMultiProcessorCount, h->dev);
   if (e != cudaSuccess) return destroy(head_cuda(e, "device query"));
 
-  h->fused = fc2_ln_fits(c.width);
+  h->fuse_rows = fc2_ln_rows(c.width);
   const size_t W = c.width, F = c.freq_dim, CD = c.cond_dim, TD = c.token_dim, NM = h->nmod, NS = c.n_steps;
   const size_t R = 2 * (size_t)c.max_tokens, MT = c.max_tokens;
   // modulations of up to `chunk` kept steps at once, within 1 GB and with
