@@ -928,7 +928,10 @@ bool gemm_supported(int dtype, int M, int N, int K, const GemmEpi& epi, const ch
 // = 20480, width 768: fc2 69.1 -> 65.3; width 1024: fc2 111.3 -> 104.7; M = 5440,
 // width 1024: fc2 44.4 -> 38.4. Single CTAs: out at M = 20480,
 // width 768 32.6 -> 29.6, M = 5440, width 1024 18.0 -> 14.6, M = 6400 19.1 -> 16.2;
-// fc1 at M = 1600, width 768 12.5 -> 10.7, width 1024 15.2 -> 14.0.
+// fc1 at M = 1600, width 768 12.5 -> 10.7, width 1024 15.2 -> 14.0. Not with bf16 outputs
+// of single CTAs at K < 512 from four rounds on, where the kernel that can split
+// costs more than the round it shortens (M = 40960, N = 1024, GELU: K = 64 27.0 -> 28.3, 192
+// 28.7 -> 30.4, 320 30.7 -> 32.1; but 20480 x 1024 x 512 21.0 -> 20.1).
 static long rounds_cost(long base, long slots, int bn, long time, bool pair, bool resid, int K, int* whole,
                         int* split) {
   const long rounds = base / slots, rem = base - rounds * slots;
@@ -936,7 +939,7 @@ static long rounds_cost(long base, long slots, int bn, long time, bool pair, boo
   *split = 1;
   if (rem == 0) return rounds * time;
   long best = time;
-  if (rounds > 0)
+  if (rounds > 0 && !(!pair && !resid && K < 512 && rounds >= 4))
     for (int s = 2; s <= 4; ++s) {
       if (bn % (32 * s) != 0 || bn / s < 64) continue;
       const long pct = resid ? (s == 2 ? 68 : s == 3 ? 56 : K < 2048 ? 60 : 50)

@@ -122,6 +122,9 @@ def test_linear_tiles_of_the_model_shapes(lib):
     assert lm.lazymar_linear_tiles(gelu, 1600, 3072, 768) == (128, 256, 152, 4)
     assert lm.lazymar_linear_tiles(res, 20480, 768, 3072) == (256, 256, 228, 4)
     assert lm.lazymar_linear_tiles(res, 7040, 768, 3072) == (256, 192, 76, 2)
+    # bf16 outputs at short K: no split after four rounds
+    assert lm.lazymar_linear_tiles(gelu, 40960, 1024, 192) == (128, 256, 1280, 1)
+    assert lm.lazymar_linear_tiles(gelu, 20480, 1024, 512) == (128, 256, 608, 4)
     # fc2 whose 256-wide tiles fit one round of single CTAs: no pairs, but in a nearly full round of long K
     assert lm.lazymar_linear_tiles(res, 5120, 768, 3072) == (128, 256, 120, 1)
     assert lm.lazymar_linear_tiles(res, 6400, 768, 3072) == (128, 256, 150, 1)
