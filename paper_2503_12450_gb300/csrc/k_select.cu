@@ -11,7 +11,7 @@
 // similarity reaches global memory, so a selection needs no scratch.
 //
 // Floor: streaming 3 x rows x T x D elements, 13.9 us at 64 rows x 320 tokens
-// x 768 bf16 (94 MB). Measured there, back to back: 31.9 us a call, against
+// x 768 bf16 (94 MB). Measured there: 31.6 us a call, against
 // 75.5 us for a similarity kernel (every token through the second tier below
 // and its own fp64 division), a top-N kernel with one CTA per row and scratch
 // allocated for the similarities in between. What is left above the floor is
